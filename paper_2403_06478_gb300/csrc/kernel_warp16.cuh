@@ -44,6 +44,18 @@
 // the table's edges run the same packed update with per-slot masks (the head
 // of the table, where the virtual row and column enter, runs the bulk or the
 // tail step wherever their values follow from the recurrence itself).
+//
+// The score path with one warp per pair (LAZY) goes further: nearly all its
+// anti-diagonals, the head's and the tail's too, run in blocks whose step
+// leaves out the maximum, the test and every mask (lazy_step, lazy_pair),
+// because the integer ALU pipe bounds this kernel (80% busy) and that step
+// has 75 of its instructions per 16-slot anti-diagonal where the bulk step
+// has 114 and the masked step about 250.  Measured on one GB300, whole calls:
+// 20,000 ONT-like pairs 59.5 -> 40.0 ms, 5,000 HiFi-like 35.9 -> 24.2, 100,000
+// pairs of Pareto lengths at w = 750 195.5 -> 82.1, 200,000 reads of 150 bp
+// 15.2 -> 5.2.  One copy of the loop in the instruction cache matters as much:
+// a second copy for the table's last rows took the Pareto batch from 75 to 100
+// ms, bands of many widths in one batch (each its own copy) 5x.
 #pragma once
 
 #include <climits>
@@ -88,6 +100,10 @@ struct Cold16 {
     int32_t mqe, mqe_t, mte, mte_q, gscore;
     int32_t gt, gq;               // cell of the global maximum
     int32_t Dp, LOWCHK, kint;     // step bound, lowest allowed score, rebase interval
+    // LAZY: the two checkpoints (their registers lie in dynamic shared memory):
+    // anti-diagonal, start of its drift, base, and the steps then left to the
+    // next rebase
+    int32_t ck_r[2], ck_rs[2], ck_base[2], ck_u0[2];
 };
 
 // What the K warps sharing one pair's band (K > 1) hand each other through
@@ -132,14 +148,16 @@ struct Xchg16 {
 // the edge steps defer their arg-max search like the bulk.  (The larger
 // register budget only: the extra state does not fit the smaller one
 // without spills.)
+// LAZY: blocks of anti-diagonals without a maximum (see lazy_run).
 template <int C, bool DMREG, bool DEFER = false, bool DIR = false, bool SCORE = !DIR, int K = 1,
-          bool FHEAD = false, bool EDEFER = false, int G = 32>
+          bool FHEAD = false, bool EDEFER = false, int G = 32, bool LAZY = false>
 struct WarpPair16 {
     static_assert(C == 4 || C == 6 || C == 8 || C == 12 || C == 16 || C == 20 || C == 24,
                   "16-bit lanes use 4, 6, 8, 12, 16, 20 or 24 slots per lane");
     static_assert(K == 1 || K == 2 || K == 4, "1, 2 or 4 warps per pair");
     static_assert(K == 1 || !DIR, "the traceback variants run one warp per pair");
     static_assert(G == 32 || (G == 16 && K == 1 && !DIR), "half-warp pairs: one group, score only");
+    static_assert(!LAZY || (G == 32 && K == 1 && !DIR && !DEFER), "lazy blocks: one warp per pair, score only");
     static constexpr int P = C / 2;
     static constexpr int32_t NS = G * C * K;      // slots of the frame
     // G lanes per pair: the whole warp, or a half warp (two pairs per warp,
@@ -185,12 +203,16 @@ struct WarpPair16 {
     int32_t pend_r, pend_m, pend_lm;   // its anti-diagonal (-3: none), maximum, lane maximum
     uint32_t pend_rb;              // lane bits of its band slots (~0: every slot of the bulk)
     bool in_head;                  // FHEAD: the pair loop is running head anti-diagonals
+    bool cover;                    // LAZY: the band covers the table with a slot to spare
+    bool blind;                    // LAZY: masked steps leave out the maximum and the test
     // base windows (2 bits per slot): Tw field jl = T[B + j0 + jl],
     // Qw field jl = Q[r - B - j0 - jl]
     Win Tw, Qw;
     uint32_t Tpf, Qpf;
     int32_t wcnt;          // pairs of shifts left in Tpf and Qpf (one count for both)
     int32_t tpos, qpos;    // next prefetch position (bases, word-relative)
+    int32_t tph, qph;      // phase of each sequence's first base in its first word
+    uint4 *ck;             // LAZY: the warp's two checkpoints and edge ring
     // relative scores
     int32_t base, OFF, last_m;
     int32_t until_rebase;  // anti-diagonals left before the next rebase
@@ -297,8 +319,7 @@ struct WarpPair16 {
                                                           int32_t a) {
         return (uint64_t)load_rel(p, span, a) | ((uint64_t)load_rel(p, span, a + 16) << 32);
     }
-    // tph/qph: the phase of the pair's first base in its first word
-    __device__ __forceinline__ void init_windows(int32_t r, int32_t tph, int32_t qph) {
+    __device__ __forceinline__ void init_windows(int32_t r) {
         const int32_t B = frame(r);
         const int32_t tb = B + j0 + tph;
         const int32_t qb = r - B - j0 + qph;
@@ -515,7 +536,8 @@ struct WarpPair16 {
                 group_sync();
                 tstar = xch->t[r & 1];
             }
-            if (max_and_zdrop(mt, tstar, r)) { zdropped = 1; return true; }
+            const bool drop = max_and_zdrop(mt, tstar, r);
+            if (LAZY ? __any_sync(FULL, drop) : drop) { zdropped = 1; return true; }
         }
         return false;
     }
@@ -592,8 +614,12 @@ struct WarpPair16 {
             rb = range_bits(st - B - j0, en - B - j0);
         }
         if constexpr (MODE == HEAD) {
-            if (r + 1 < qlen) vb |= slot_bit(-1 - B - j0);                 // (-1, r+1)
-            if (r >= -1 && r + 1 < tlen) vb |= slot_bit(r + 1 - B - j0);  // (r+1, -1)
+            // (LAZY runs it past the head as well, where no virtual cell is in
+            // the band)
+            if (!LAZY || r <= w + 1) {
+                if (r + 1 < qlen) vb |= slot_bit(-1 - B - j0);                 // (-1, r+1)
+                if (r >= -1 && r + 1 < tlen) vb |= slot_bit(r + 1 - B - j0);  // (r+1, -1)
+            }
             const int32_t vv = to_u(r == -2 ? 0 : -gap_cost(prm, r + 2));
             if (__any_sync(gmask(), vb != 0u) && (vv < cold.LOWCHK || vv > 0xffff - cold.Dp)) ovf = true;
             VVp = (uint32_t)vv * 0x10001u;
@@ -616,7 +642,7 @@ struct WarpPair16 {
             uint32_t f2R = __shfl_down_sync(gmask(), F2o[0], 1, G);
             if (K > 1 && wk < K - 1 && lane == 31) { fR = xe0; f2R = xe1; }
             uint32_t inj = NEGp, inj2 = NEGp;
-            if (MODE == HEAD && lane == G - 1 && (K == 1 || wk == K - 1)) {
+            if (MODE == HEAD && lane == G - 1 && (K == 1 || wk == K - 1) && (!LAZY || r <= w + 1)) {
                 // beyond the last lane: slot NS of r-1, the virtual column
                 // cell (t, -1) when q == -1 there
                 const int32_t ts = frame(r - 1) + NS, qs = r - 1 - ts;
@@ -744,9 +770,16 @@ struct WarpPair16 {
                 }
             }
             __syncwarp(gmask());
+            if constexpr (LAZY) {
+                if (blind) { --until_rebase; return false; }
+            }
             if (anti_diagonal_max<ODD>(r, B, lm, m_grp, Hd, [&](int p) { return ~half_mask_rt(rb, p); }, rb))
                 return true;
             if (set_gs && lane == 0) cold.gscore = gs;
+            if constexpr (LAZY) {
+                --until_rebase;
+                return false;
+            }
             if (--until_rebase <= 2) {
                 // slots off the table (past its end, or holding NEG) are
                 // reset; the virtual cells' values are kept
@@ -875,7 +908,7 @@ struct WarpPair16 {
     // reset like the slots beyond the band and not checked.
     __device__ __forceinline__ void rebase(int32_t m_u, int32_t r, uint32_t in_r = ~0u,
                                            uint32_t in_r1 = ~0u) {
-        until_rebase = cold.kint;
+        until_rebase = LAZY ? __reduce_max_sync(FULL, cold.kint) : cold.kint;
         const int32_t delta = m_u - OFF;
         const int32_t low = min(max(cold.LOWCHK - cold.Dp + delta, 0), 0xffff);
         const uint32_t low2 = (uint32_t)low * 0x10001u;
@@ -965,90 +998,472 @@ struct WarpPair16 {
         return lo > 2 * (int64_t)(prm.a + prm.b + oe2) && hi + 4 * (int64_t)cold.Dp < floor_virt;
     }
 
-    // ------------------------------------------------------------------ pair
-    // Returns false if the pair must be recomputed with int32 lanes.
-    // DIR (fused): dt is the pair's direction table, one row per anti-diagonal
-    // up to the last one the extension can reach.
-    __device__ __forceinline__ bool run(const DevBatch &Bt, int32_t pair, int32_t lane_, bool use_fast,
-                                        uint8_t *dt = nullptr) {
-        prm = Bt.params;
-        lane = lane_;
-        tlen = Bt.t_len[pair]; qlen = Bt.q_len[pair];
-        int32_t tph, qph;
-        {
-            const int64_t toff = Bt.t_off[pair], qoff = Bt.q_off[pair];
-            const int64_t tw0 = toff >> 4, qw0 = qoff >> 4;
-            tp = Bt.t_packed + tw0;
-            qp = Bt.q_packed + qw0;
-            tph = (int32_t)(toff & 15);
-            qph = (int32_t)(qoff & 15);
-            // the words the pair's bases occupy (inside the stream: checked by prep)
-            tspan = (int32_t)min(Bt.t_words - tw0, (int64_t)((tph + tlen + 15) >> 4));
-            qspan = (int32_t)min(Bt.q_words - qw0, (int64_t)((qph + qlen + 15) >> 4));
+    // ------------------------------------------------------- lazy blocks
+    // The termination rule needs an anti-diagonal's maximum only where it can
+    // change the global maximum for good or end the extension.  Blocks of up
+    // to 2 * LAZY_PAIRS anti-diagonals run without it where neither can happen
+    // unseen (lazy_run); this is their step.  Against the exact step it drops
+    // the running maximum, the warp reduction and the test, the masks of the
+    // slots off the band and the table, and half of the second gap piece's work:
+    //  - Scores drift upwards by d per anti-diagonal (d = e2, or e when the
+    //    gap cost has one piece): extending a gap of that piece then costs
+    //    nothing, E2' = max(E2, H - q2).
+    //  - H - q2 ("h") is kept in Hev/Hod instead of H, the constant q2 coming
+    //    back with the match score.
+    //  - E2 is brought up to date only on odd anti-diagonals (where it moves
+    //    up a slot), with the h of both: E2 = max3(E2, h of r-1, h of r), and
+    //    F2 only on even ones.  On the others the state lacks the gap of
+    //    length one out of r-1, which the first piece gives at no higher a
+    //    cost (q + e <= q2 + e2; run sees to it).
+    //  - Slots beyond the band run on: nothing above slot w reaches the band
+    //    except through F and F2 leaving slot w + 1 of an odd anti-diagonal,
+    //    nothing below it except through E and E2 leaving slot 0 of one (of
+    //    lane 0).  Those are set to minus infinity (register PR holds slot
+    //    w + 1; PR = P where the frame ends with slot w, whose F then comes
+    //    from past the last lane), so the shuffles' other end lanes need no
+    //    mask.  Cells past the table's end, or beyond the virtual row and
+    //    column, feed nothing of the table (see step and head_bounds_ok).
+    // Minus infinity stays at U_NEG under the drift; every score is then at
+    // least U_NEG, because the drifting gap state never falls.
+    static constexpr int LAZY_PAIRS = 16;                // one word of each sequence
+    static constexpr int CKV = 6 * P / 4;                // 16-byte words of a checkpoint per lane
+    static constexpr int RING = 2 * 2 * LAZY_PAIRS * P;  // words of the edge ring (row | column)
+    static constexpr int TW = C <= 16 ? 2 : 3;           // window words: C bases and 16 to come
+
+    struct LazyWin { uint32_t t[TW], q[TW]; };
+    // packed constants (H2: the offset of h; D: the drift), the slot w + 1 mask
+    struct LazyConst { uint32_t A, NE, OE, H2, D, top; };
+    // where the last row's and column's cells sit, as slots of this lane
+    // (on: the block may hold such cells; uniform) and the ring's shared address
+    struct LazyEdge { int32_t on, dt, dq; uint32_t ring; };
+
+    // Windows of anti-diagonal r and the 16 bases after them: t field i is
+    // T[B + j0 + i]; q holds the bases in falling order, field 16 + jl of the
+    // 16 * TW being Q[r - B - j0 - jl].
+    __device__ __forceinline__ void lazy_windows(LazyWin &W, int32_t r) const {
+        const int32_t B = frame(r);
+        const int32_t tb = B + j0 + tph, qb = r - B - j0 + qph + 1;
+#pragma unroll
+        for (int i = 0; i < TW; ++i) {
+            W.t[i] = load_rel(tp, tspan, tb + 16 * i);
+            W.q[i] = rev2_32(load_rel(qp, qspan, qb - 16 * i));
         }
-        agatha_result *out = Bt.out + pair;
-        if constexpr (DIR) { end_t = -1; end_q = -1; }
-        if (tlen <= 0 || qlen <= 0) {
-            if (leader()) write_empty_result(out);
-            return true;
+    }
+    template <bool ODD>
+    __device__ __forceinline__ Comb lazy_mismatch(LazyWin &W) const {
+        if constexpr (!ODD) {
+#pragma unroll
+            for (int i = 0; i + 1 < TW; ++i) W.t[i] = __funnelshift_r(W.t[i], W.t[i + 1], 2);
+            W.t[TW - 1] >>= 2;
+        } else {
+#pragma unroll
+            for (int i = TW - 1; i > 0; --i) W.q[i] = __funnelshift_l(W.q[i - 1], W.q[i], 2);
+            W.q[0] <<= 2;
         }
-        w = effective_w(prm.w, tlen, qlen);
-        oe = prm.q + prm.e; oe2 = prm.q2 + prm.e2;
-        j0 = (wk * G + lane) * C;
-        last_r = tlen + qlen - 2;
-        if constexpr (DIR) dtab = dt + j0;
-        {
-            const int32_t Dp = step_change_max(prm), kint = rebase_interval(Dp);
-            until_rebase = kint;
-            OFF = 0xffff - (kint + 3) * Dp;
-            if (leader()) {
-                cold.Dp = Dp;
-                cold.kint = kint;
-                cold.LOWCHK = (int32_t)U_NEG + (kint + 3) * Dp;
+        constexpr uint32_t M0 = C >= 16 ? 0x55555555u : (C == 8 ? 0x5555u : 0x55u);
+        const uint32_t x0 = W.t[0] ^ W.q[1];
+        const uint32_t n0 = (x0 | (x0 >> 1)) & M0;
+        if constexpr (C == 16) return {n0, 0u};
+        else if constexpr (C == 8) return {n0 * 0x101u, 0u};
+        else if constexpr (C == 4) return {n0 * 0x1001u, 0u};
+        else if constexpr (C > 16) {
+            const uint32_t x1 = W.t[1] ^ W.q[2];
+            const uint32_t n1 = (x1 | (x1 >> 1)) & 0x55555555u;
+            if constexpr (C == 24) return {prmt(n0, n1, 0x4310), prmt(n0, n1, 0x5552)};
+            const uint32_t g = __funnelshift_r(n0, n1, 20);      // slots 10..
+            return {prmt(n0, g, 0x5410), prmt(n0, g, 0x6662)};
+        }
+        else return {0u, 0u};
+    }
+
+    // Store an anti-diagonal's registers at shared address d if slot offset j
+    // is one of the lane's (predicated stores: no divergent branch in the loop).
+    __device__ __forceinline__ static void ring_store(uint32_t d, int32_t j, const uint32_t (&H)[P]) {
+        if constexpr (P % 4 == 0) {
+#pragma unroll
+            for (int p = 0; p < P; p += 4)
+                asm volatile("{\n\t.reg .pred q;\n\tsetp.lt.u32 q, %0, %1;\n\t"
+                             "@q st.shared.v4.b32 [%2], {%3, %4, %5, %6};\n\t}"
+                             :: "r"(j), "n"(C), "r"(d + 4 * p), "r"(H[p]), "r"(H[p + 1]), "r"(H[p + 2]), "r"(H[p + 3])
+                             : "memory");
+        } else {
+#pragma unroll
+            for (int p = 0; p < P; p += 2)
+                asm volatile("{\n\t.reg .pred q;\n\tsetp.lt.u32 q, %0, %1;\n\t"
+                             "@q st.shared.v2.b32 [%2], {%3, %4};\n\t}"
+                             :: "r"(j), "n"(C), "r"(d + 4 * p), "r"(H[p]), "r"(H[p + 1]) : "memory");
+        }
+    }
+    // One anti-diagonal of a lazy block (TWO: two gap pieces).
+    template <bool ODD, bool TWO, int PR>
+    __device__ __forceinline__ void lazy_step(LazyWin &W, const LazyConst &k) {
+        uint32_t (&Hd)[P] = ODD ? Hod : Hev;
+        const uint32_t (&Hx)[P] = ODD ? Hev : Hod;
+        const Comb comb = lazy_mismatch<ODD>(W);
+        uint32_t edge, edge2 = 0;
+        if constexpr (ODD) {
+            edge = prmt(__shfl_up_sync(FULL, Eo[P - 1], 1), Eo[P - 1], 0x5432);
+            if constexpr (TWO) {
+                const uint32_t x = __vmaxu2(E2o[P - 1], Hev[P - 1]);
+                edge2 = prmt(__shfl_up_sync(FULL, x, 1), x, 0x5432);
+            }
+        } else {
+            edge = prmt(Fo[0], __shfl_down_sync(FULL, Fo[0], 1), 0x5432);
+            if constexpr (PR == P) edge = mux(k.top, NEGp, edge);
+            if constexpr (TWO) {
+                const uint32_t x = __vmaxu2(F2o[0], Hod[0]);
+                edge2 = prmt(x, __shfl_down_sync(FULL, x, 1), 0x5432);
+                if constexpr (PR == P) edge2 = mux(k.top, NEGp, edge2);
             }
         }
-        base = 0;
-        last_m = OFF;
-        ovf = false;
-        A2 = ((uint32_t)prm.a & 0xffffu) * 0x10001u;
-        NABs = 0u - (uint32_t)(prm.a + prm.b);
-        OEp = (uint32_t)oe * 0x10001u;
-        DOEp = (uint32_t)(oe2 - oe) * 0x10001u;
-        Ep = (uint32_t)prm.e * 0x10001u;
-        E2p = (uint32_t)prm.e2 * 0x10001u;
-        NEp = ((uint32_t)(-prm.e) & 0xffffu) * 0x10001u;
-        NE2p = ((uint32_t)(-prm.e2) & 0xffffu) * 0x10001u;
-        NEGp = U_NEG * 0x10001u;
-        L0LO = (lane == 0 && wk == 0) ? 0x0000ffffu : 0u;
-        L31HI = (lane == G - 1 && wk == K - 1) ? 0xffff0000u : 0u;
-        xe0 = xe1 = NEGp;
+#pragma unroll
+        for (int i = 0; i < P; ++i) {
+            const int p = ODD ? P - 1 - i : i;
+            const int n = ODD ? p - 1 : p + 1;             // where the moving gap states come from
+            const bool own = ODD ? p > 0 : p < P - 1;      // in a register of this lane
+            const uint32_t Ein = ODD && own ? Eo[own ? n : 0] : (ODD ? edge : Eo[p]);
+            const uint32_t Fin = !ODD && own ? Fo[own ? n : 0] : (!ODD ? edge : Fo[p]);
+            const uint32_t mword = (C <= 16 || p < 8) ? comb.lo : comb.hi;
+            const uint32_t mb = (mword >> (2 * (p & 7))) & 0x10001u;
+            const uint32_t Hs = mb * NABs + Hd[p];
+            const uint32_t X = __viaddmax_u16x2(Hs, k.A, Ein);
+            if constexpr (TWO) {
+                const uint32_t E2in = ODD && own ? E2o[own ? n : 0] : (ODD ? edge2 : E2o[p]);
+                const uint32_t F2in = !ODD && own ? F2o[own ? n : 0] : (!ODD ? edge2 : F2o[p]);
+                const uint32_t H = __vmaxu2(__vimax3_u16x2(X, Fin, E2in), F2in);
+                const uint32_t h = H - k.H2, hoe = H - k.OE;
+                Eo[p] = __viaddmax_u16x2(Ein, k.NE, hoe);
+                Fo[p] = __viaddmax_u16x2(Fin, k.NE, hoe);
+                if constexpr (ODD) E2o[p] = own ? __vimax3_u16x2(E2in, Hx[own ? n : 0], h) : __vmaxu2(E2in, h);
+                else F2o[p] = own ? __vimax3_u16x2(F2in, Hx[own ? n : 0], h) : __vmaxu2(F2in, h);
+                Hd[p] = h;
+            } else {
+                const uint32_t h = __vmaxu2(X, Fin) - k.H2;
+                Eo[p] = __vmaxu2(Ein, h);
+                Fo[p] = __vmaxu2(Fin, h);
+                Hd[p] = h;
+            }
+        }
+        if constexpr (ODD) {
+            constexpr int pr = PR < P ? PR : 0;
+            Eo[0] = mux(L0LO, NEGp, Eo[0]);
+            if constexpr (PR < P) Fo[pr] = mux(k.top, NEGp, Fo[pr]);
+            if constexpr (TWO) {
+                E2o[0] = mux(L0LO, NEGp, E2o[0]);
+                if constexpr (PR < P) {
+                    F2o[pr] = mux(k.top, NEGp, F2o[pr]);
+                    Hod[pr] = mux(k.top, NEGp, Hod[pr]);
+                }
+            }
+        }
+    }
+    template <bool TWO, int PR>
+    __device__ __forceinline__ void lazy_pairs(int32_t n, LazyWin &W, const LazyConst &k, LazyEdge &g) {
+#pragma unroll 1
+        for (; n > 0; --n) {
+            lazy_step<false, TWO, PR>(W, k);
+            lazy_step<true, TWO, PR>(W, k);
+            if (g.on) {
+                // the lanes holding a cell of the last row or column keep the
+                // pair's registers for lazy_edges; the row's slot moved down
+                // before the first anti-diagonal, the column's moves up
+                // before the second
+                --g.dt;
+                ring_store(g.ring, g.dt, Hev);
+                ring_store(g.ring + 2 * RING, g.dq, Hev);
+                ++g.dq;
+                ring_store(g.ring + 4 * P, g.dt, Hod);
+                ring_store(g.ring + 4 * P + 2 * RING, g.dq, Hod);
+                g.ring += 8 * P;
+            }
+        }
+    }
+    template <bool TWO, int PR = 0>
+    __device__ __forceinline__ void lazy_dispatch(int32_t pr, int32_t n, LazyWin &W, const LazyConst &k,
+                                                  LazyEdge &g) {
+        if constexpr (PR == P) {
+            lazy_pairs<TWO, PR>(n, W, k, g);
+        } else {
+            if (pr == PR) lazy_pairs<TWO, PR>(n, W, k, g);
+            else lazy_dispatch<TWO, PR + 1>(pr, n, W, k, g);
+        }
+    }
+
+    // Into the drifting form after anti-diagonal r ((r - w) odd), and back.
+    __device__ __forceinline__ void lazy_enter(const LazyConst &k) {
 #pragma unroll
         for (int p = 0; p < P; ++p) {
-            Hev[p] = Hod[p] = Eo[p] = E2o[p] = Fo[p] = F2o[p] = NEGp;
+            Hod[p] -= k.H2;
+            Hev[p] -= k.H2 + k.D;
+            Eo[p] += k.D;
+            Fo[p] += k.D;
+            E2o[p] += k.D;
+            F2o[p] += k.D;
         }
-        {
-            const int32_t k0 = min(max(w + 1 - j0, 0), C);     // first local slot beyond the band
-            DF2 = (uint32_t)(k0 - 1) * 0x10001u;
-            if constexpr (DMREG) {
+    }
+    // steps: anti-diagonals since lazy_enter
+    __device__ __forceinline__ void lazy_leave(const LazyConst &k, bool two, int32_t steps) {
+        const uint32_t c = k.D * (uint32_t)(steps + 1), lo = NEGp + c;
 #pragma unroll
-                for (int p = 0; p < P; ++p)
-                    DMR[p] = prmt(DF2 - ((uint32_t)p | ((uint32_t)(p + P) << 16)), 0, 0xbb99);
+        for (int p = 0; p < P; ++p) {
+            const uint32_t dm = dead_mask(p), dmr = dead_mask_r<true>(p);
+            const uint32_t f2 = __vmaxu2(F2o[p], Hod[p]);
+            Eo[p] = mux(dmr, NEGp, __vmaxu2(Eo[p], lo) - c);
+            Fo[p] = mux(dmr, NEGp, __vmaxu2(Fo[p], lo) - c);
+            E2o[p] = two ? mux(dmr, NEGp, __vmaxu2(E2o[p], lo) - c) : Eo[p];
+            F2o[p] = two ? mux(dmr, NEGp, __vmaxu2(f2, lo) - c) : Fo[p];
+            Hod[p] = mux(dmr, NEGp, __vmaxu2(Hod[p] + k.H2 + k.D, lo) - c);
+            Hev[p] = mux(dm, NEGp, __vmaxu2(Hev[p] + k.H2 + 2 * k.D, lo) - c);
+        }
+    }
+    // The maximum over the band cells of anti-diagonals r and r - 1 ((r - w)
+    // odd), in the drifting form of r.  inner: every slot of the band is a cell
+    // of the table there.
+    __device__ __forceinline__ int32_t lazy_max(const LazyConst &k, int32_t r, bool inner) const {
+        uint32_t lmax = 0;
+        if (inner) {
+#pragma unroll
+            for (int p = 0; p < P; ++p) {
+                const uint32_t x = __vmaxu2(p == 0 ? Hod[p] & ~L0LO : Hod[p], Hev[p] + k.D);
+                lmax = __vmaxu2(lmax, x & ~dead_mask(p));
+            }
+        } else {
+            const uint32_t b1 = table_bits(r), b0 = table_bits(r - 1);
+#pragma unroll
+            for (int p = 0; p < P; ++p)
+                lmax = __vimax3_u16x2(lmax, half_mask_rt(b1, p) & Hod[p], half_mask_rt(b0, p) & (Hev[p] + k.D));
+        }
+        return __reduce_max_sync(FULL, (int32_t)max(lmax & 0xffffu, lmax >> 16));
+    }
+    // The best score on the last row and column of anti-diagonals r0 + 1 ..
+    // r0 + 2n (lane i takes the i-th of them) from the ring.  off: from a
+    // drifting h of anti-diagonal r0 to its true score.
+    __device__ __forceinline__ void lazy_edges(const uint32_t *ring, int32_t r0, int32_t n, int32_t off, int32_t d) {
+        __syncwarp();
+        const int32_t r = r0 + 1 + lane, B = frame(r);
+        off -= d * (1 + lane);
+        const int32_t lo = max(max(0, r - qlen + 1), ceil_div2(r - w)), hi = min(min(tlen - 1, r), floor_div2(r + w));
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const int32_t t = c == 0 ? tlen - 1 : r - qlen + 1;
+            int32_t v = INT_MIN;
+            if (lane < 2 * n && lo <= t && t <= hi) {
+                const int32_t local = (t - B) % C;
+                v = half_of(ring[c * (RING / 2) + lane * P + local % P], local) + off;
+            }
+            const int32_t m = __reduce_max_sync(FULL, v);
+            if (m > (c == 0 ? cold.mte : cold.mqe)) {
+                const int32_t at = r0 + 1 + __ffs(__ballot_sync(FULL, v == m)) - 1;
+                if (lane == 0) {
+                    if (c == 0) { cold.mte = m; cold.mte_q = at - (tlen - 1); }
+                    else { cold.mqe = m; cold.mqe_t = at - (qlen - 1); }
+                }
             }
         }
-        gmax = 0;
-        pend_r = -3;
-        pend_rb = ~0u;
-        if (leader()) {
-            cold.mqe = K_NEG_OUT; cold.mqe_t = -1; cold.mte = K_NEG_OUT; cold.mte_q = -1;
-            cold.gscore = K_NEG_OUT;
-            cold.gt = -1; cold.gq = -1;
+        __syncwarp();
+    }
+    // Checkpoints: the packed registers of the drifting form.
+    __device__ __forceinline__ uint32_t &lazy_word(int i) {
+        return i < P ? Hev[i] : (i < 2 * P ? Hod[i - P] : (i < 3 * P ? Eo[i - 2 * P]
+               : (i < 4 * P ? Fo[i - 3 * P] : (i < 5 * P ? E2o[i - 4 * P] : F2o[i - 5 * P]))));
+    }
+    __device__ __forceinline__ void lazy_save(int buf, int32_t r, int32_t rs, int32_t u0) {
+        uint4 *d = ck + lane + buf * (CKV * 32);
+#pragma unroll
+        for (int i = 0; i < CKV; ++i)
+            d[i * 32] = make_uint4(lazy_word(4 * i), lazy_word(4 * i + 1), lazy_word(4 * i + 2), lazy_word(4 * i + 3));
+        if (lane == 0) {
+            cold.ck_r[buf] = r;
+            cold.ck_rs[buf] = rs;
+            cold.ck_base[buf] = base;
+            cold.ck_u0[buf] = u0;
         }
-        __syncwarp(gmask());
-        group_sync();
-        zdropped = 0;
+        __syncwarp();
+    }
+    __device__ __forceinline__ void lazy_load(int buf) {
+        const uint4 *d = ck + lane + buf * (CKV * 32);
+#pragma unroll
+        for (int i = 0; i < CKV; ++i) {
+            const uint4 v = d[i * 32];
+            lazy_word(4 * i) = v.x;
+            lazy_word(4 * i + 1) = v.y;
+            lazy_word(4 * i + 2) = v.z;
+            lazy_word(4 * i + 3) = v.w;
+        }
+    }
+    // Pairs of anti-diagonals the next block may hold: n, 8 or 4 (0: none) such
+    // that no anti-diagonal of it can fire the Z-drop test.  g, m, mu: an upper
+    // bound of the global maximum, the maximum of the last two anti-diagonals,
+    // and that maximum with the virtual cells.  k anti-diagonals on, no score is
+    // above mu + a ceil(k/2), and the maximum is at least m - o - c ceil(k/2):
+    // away from the last row and column (c = b, o = min(q+e, q2+e2)) the cell
+    // of m continues along its diagonal, after one gap step if the parity asks
+    // for it; near them (c = max(b, 2e), o = q+e + q + c) it may have to go on
+    // along the edge by a gap, towards the corner, which lies in the band.
+    __device__ __forceinline__ int32_t lazy_span(int32_t n, int32_t g, int32_t m, int32_t mu, int32_t o,
+                                                 int32_t c) const {
+        if (prm.zdrop < 0) return n;
+#pragma unroll 1
+        while (n > 0 && max(g - m, mu - m + prm.a * n) + o + c * n > prm.zdrop)
+            n = n > 8 ? 8 : (n > 4 ? 4 : (n > 2 ? 2 : 0));
+        return n;
+    }
 
-        int32_t r = -2;
-        init_windows(r, tph, qph);
+    // The pair on lazy blocks and, where they may not run, the masked step.
+    // At the end of each block the maximum of its last two anti-diagonals is
+    // taken; a score inside the block is at most U, from that maximum and the
+    // one at the block's start (a up, c down per two anti-diagonals: U weighs
+    // the two bounds so that its place drops out).  A block whose U does not
+    // exceed the largest maximum seen before it cannot hold the global maximum;
+    // one whose U stays below a later maximum does not hold it for good either.
+    // So only the blocks since the last checkpoint that this rules in can hold
+    // it, and when the exact maximum and its cell are wanted (the Z-drop bound
+    // no longer holds, the score has passed a peak, or the table ends) the pair
+    // goes back to that checkpoint and takes the masked step from there up to
+    // exact_until.  Blocks start and end on odd anti-diagonals ((r - w) odd).
+    // The head's last four anti-diagonals (w - 2 .. w + 1), where the virtual
+    // cells leave the band, run the masked step without its test (blind), as a
+    // block of their own; a band that covers the table (cover) has no such
+    // place.  Returns the last anti-diagonal processed.
+    __device__ __forceinline__ int32_t lazy_pair(bool use_fast) {
+        constexpr int32_t NONE = INT_MIN;
+        const bool head = use_fast && w >= 8 && head_bounds_ok();    // lazy blocks in the head too
+        const int32_t L = min(tlen, qlen);
+        const int32_t r_in = max(L - 2, 2 * L - 3 - w);    // no cell of the last row or column up to here
+        // lazy blocks end here at the latest; past r_in only if the corner is in the band
+        const int32_t end = abs(tlen - qlen) <= w ? last_r - 1 : r_in;
+        const int32_t turn = cover ? INT_MAX : w - 3;      // the crossing of the head's end starts after it
+        const int32_t c0 = prm.b, c1 = max(prm.b, 2 * prm.e);
+        const int32_t o0 = min(oe, oe2), o1 = oe + prm.q + c1;
+        const bool two = prm.q2 != prm.q || prm.e2 != prm.e;
+        LazyConst k;
+        const int32_t d = prm.e2, hoff = prm.q2;
+        k.D = (uint32_t)d * 0x10001u;
+        k.H2 = (uint32_t)hoff * 0x10001u;
+        k.A = A2 + k.H2 + 2 * k.D;
+        k.NE = ((uint32_t)(d - prm.e) & 0xffffu) * 0x10001u;
+        k.OE = OEp - k.D;
+        const int32_t s1 = (w + 1) % C;
+        const int32_t pr = w + 1 < NS ? s1 % P : P;
+        k.top = pr == P ? L31HI : (lane == (w + 1) / C ? (s1 >= P ? 0xffff0000u : 0x0000ffffu) : 0u);
+        const float inv0 = 1.0f / (float)max(prm.a + c0, 1), inv1 = 1.0f / (float)max(prm.a + c1, 1);
+        const uint32_t ring = (uint32_t)__cvta_generic_to_shared(ck + 2 * CKV * 32);
+
+        int32_t r = -3;
+        // the masked step runs up to exact_until, first the first r >= 1 with (r - w) odd
+        int32_t exact_until = !use_fast ? INT_MAX : (head ? 1 + (w & 1) : w + 1);
+        // blocks under way: the largest maximum seen, the bound of the blocks not
+        // ruled out (NONE: there are none, the global maximum is best), its value
+        // at the checkpoint, the checkpoint, the one at the block's start
+        bool open = false;
+        int32_t best = 0, upper = NONE, gval = 0, old = 0, last = 0;
+        int32_t m0 = 0, mu = 0, n = 0;                     // the current block: see lazy_span
+        bool block = false, edge = false;
+        for (;;) {
+            if (r < exact_until || !((r - w) & 1)) {
+                if (r >= last_r) return r;
+                ++r;
+                if (r > -2) advance(r);
+                if (head_step(r)) return r;
+                if (until_rebase <= 2 && r >= 0) {
+                    rebase(last_m, r, table_bits(r) | virtual_bits(r), table_bits(r - 1) | virtual_bits(r - 1));
+                    if (ovf) return r;
+                }
+                continue;
+            }
+            if (!open) {
+                if (r <= w && r > turn) { exact_until = w + 1; continue; }
+                if (r + 8 > (r <= w && w + 1 > end ? min(turn, end) : end)) { exact_until = INT_MAX; continue; }
+                if (lazy_span(4, gmax, to_true(last_m), to_true(last_m), o1, c1) != 4) { exact_until = r + 8; continue; }
+            }
+            blind = false;
+            if (until_rebase < 16) {
+                const uint32_t in1 = table_bits(r) | virtual_bits(r), in0 = table_bits(r - 1) | virtual_bits(r - 1);
+                rebase(open ? to_u(m0) : last_m, r, in1, in0);
+                if (ovf) return r;
+            }
+            int32_t rs = r, u0 = until_rebase;
+            lazy_enter(k);
+            for (;;) {
+                const int32_t m1 = lazy_max(k, r, r > w && r <= r_in) + hoff - OFF + base - d * (r - rs);
+                if (!open) {
+                    open = true;
+                    best = gval = gmax;
+                    upper = NONE;
+                    old = 1;
+                } else if (block) {
+                    const int32_t rise = m1 - mu + (edge ? prm.q + c1 * n : c0 * n);
+                    const int32_t U = mu + (int32_t)((float)(prm.a * rise) * (edge ? inv1 : inv0)) + 1;
+                    if (m1 > best && m1 > upper) {
+                        // the blocks before this one are ruled out
+                        gval = upper == NONE ? best : -(1 << 29);
+                        old = last;
+                        upper = U;
+                    } else if (U > best) {
+                        if (upper == NONE) { gval = best; old = last; }
+                        upper = max(upper, U);
+                    }
+                    best = max(best, m1);
+                }
+                block = false;
+                m0 = m1;
+                const bool cross = r == turn;
+                if (r + 2 > end || (cross && w + 1 > end) || (upper != NONE && m0 + prm.a * LAZY_PAIRS <= best)) {
+                    exact_until = r;                       // the end, or past a peak
+                    open = false;
+                    break;
+                }
+                const int32_t left = (u0 - (r - rs) - 4) >> 1;
+                if (left < 4) break;                       // a rebase is due
+                edge = cross || r + 2 > r_in;
+                n = (min(edge ? end : r_in, r < turn ? min(turn, end) : end) - r) >> 1;
+                if (edge && n < 2 * LAZY_PAIRS) n = min(n, max(4, (n + 1) >> 1));   // shorter towards the end
+                n = cross ? 2 : min(min(n, left), LAZY_PAIRS);
+                mu = r < w ? max(m0, -gap_cost(prm, r + 1)) : m0;
+                const int32_t fit = lazy_span(n, max(best, upper), m0, mu, edge ? o1 : o0, edge ? c1 : c0);
+                if (fit == 0 || (cross && fit < n)) {
+                    exact_until = r + 8;
+                    open = false;
+                    break;
+                }
+                n = fit;
+                last = old ^ 1;
+                lazy_save(last, r, rs, u0);
+                block = true;
+                if (cross) {
+                    blind = true;
+                    exact_until = r + 4;
+                    break;
+                }
+                LazyWin W;
+                lazy_windows(W, r);
+                const int32_t B = frame(r);
+                LazyEdge g{__reduce_max_sync(FULL, edge ? 1 : 0), tlen - 1 - B - j0, r - qlen + 1 - B - j0, ring};
+                if (two) lazy_dispatch<true>(pr, n, W, k, g);
+                else lazy_dispatch<false>(pr, n, W, k, g);
+                if (edge)
+                    lazy_edges(reinterpret_cast<const uint32_t *>(ck + 2 * CKV * 32), r, n,
+                               hoff - OFF + base - d * (r - rs), d);
+                r += 2 * n;
+            }
+            if (!open && upper != NONE) {                  // back to the checkpoint
+                lazy_load(old);
+                r = __reduce_max_sync(FULL, cold.ck_r[old]);
+                rs = __reduce_max_sync(FULL, cold.ck_rs[old]);
+                base = __reduce_max_sync(FULL, cold.ck_base[old]);
+                u0 = __reduce_max_sync(FULL, cold.ck_u0[old]);
+                gmax = gval;
+            }
+            lazy_leave(k, two, r - rs);
+            until_rebase = u0 - (r - rs);
+            last_m = to_u(m0);
+            init_windows(r);
+        }
+    }
+
+    // The pair from anti-diagonal r = -2 on the masked and bulk steps (not
+    // LAZY).  Returns the last anti-diagonal processed.
+    __device__ __forceinline__ int32_t steps(int32_t r, bool use_fast) {
         bool stop = head_step(r);
         const int32_t head_end = min(last_r, w + 1);
         // bulk: pairs starting at r = w + 2 ((r - w) even) while every band
@@ -1150,6 +1565,120 @@ struct WarpPair16 {
             advance(r);
             stop = tail_step(r);
         }
+        return r;
+    }
+
+    // ------------------------------------------------------------------ pair
+    // Returns false if the pair must be recomputed with int32 lanes.
+    // DIR (fused): dt is the pair's direction table, one row per anti-diagonal
+    // up to the last one the extension can reach.
+    __device__ __forceinline__ bool run(const DevBatch &Bt, int32_t pair, int32_t lane_, bool use_fast,
+                                        uint8_t *dt = nullptr) {
+        prm = Bt.params;
+        lane = lane_;
+        tlen = Bt.t_len[pair]; qlen = Bt.q_len[pair];
+        if constexpr (LAZY) {
+            // the values that steer the pair, through a warp reduction: the
+            // same in every lane for the compiler too, which then leaves out
+            // the checks for a diverged warp before each shuffle
+            tlen = __reduce_max_sync(FULL, tlen);
+            qlen = __reduce_max_sync(FULL, qlen);
+            int32_t *v = &prm.a;
+#pragma unroll
+            for (int i = 0; i < (int)(sizeof(DevParams) / 4); ++i) v[i] = __reduce_max_sync(FULL, v[i]);
+        }
+        {
+            const int64_t toff = Bt.t_off[pair], qoff = Bt.q_off[pair];
+            const int64_t tw0 = toff >> 4, qw0 = qoff >> 4;
+            tp = Bt.t_packed + tw0;
+            qp = Bt.q_packed + qw0;
+            tph = (int32_t)(toff & 15);
+            qph = (int32_t)(qoff & 15);
+            // the words the pair's bases occupy (inside the stream: checked by prep)
+            tspan = (int32_t)min(Bt.t_words - tw0, (int64_t)((tph + tlen + 15) >> 4));
+            qspan = (int32_t)min(Bt.q_words - qw0, (int64_t)((qph + qlen + 15) >> 4));
+        }
+        agatha_result *out = Bt.out + pair;
+        if constexpr (DIR) { end_t = -1; end_q = -1; }
+        if (tlen <= 0 || qlen <= 0) {
+            if (leader()) write_empty_result(out);
+            return true;
+        }
+        w = effective_w(prm.w, tlen, qlen);
+        if constexpr (LAZY) {
+            // a second piece that is the cheaper one from length one on is
+            // the only one
+            if (prm.q + prm.e > prm.q2 + prm.e2) { prm.q = prm.q2; prm.e = prm.e2; }
+            blind = false;
+            // a band that covers the table may as well be the whole frame: the
+            // virtual cells then never leave it, and all such pairs run the
+            // same copy of the lazy step
+            const int32_t len = max(tlen, qlen);
+            cover = w >= len && len < NS - 1;
+            if (cover) w = NS - 1;
+        }
+        oe = prm.q + prm.e; oe2 = prm.q2 + prm.e2;
+        j0 = (wk * G + lane) * C;
+        last_r = tlen + qlen - 2;
+        if constexpr (DIR) dtab = dt + j0;
+        {
+            int32_t Dp = step_change_max(prm);
+            // the drift of the lazy blocks and half a match per anti-diagonal
+            // stay within the step bound too
+            if constexpr (LAZY) Dp = max(Dp, (prm.a + 1) / 2 + prm.e2);
+            const int32_t kint = rebase_interval(Dp);
+            until_rebase = kint;
+            OFF = 0xffff - (kint + 3) * Dp;
+            if (leader()) {
+                cold.Dp = Dp;
+                cold.kint = kint;
+                cold.LOWCHK = (int32_t)U_NEG + (kint + 3) * Dp;
+            }
+        }
+        base = 0;
+        last_m = OFF;
+        ovf = false;
+        A2 = ((uint32_t)prm.a & 0xffffu) * 0x10001u;
+        NABs = 0u - (uint32_t)(prm.a + prm.b);
+        OEp = (uint32_t)oe * 0x10001u;
+        DOEp = (uint32_t)(oe2 - oe) * 0x10001u;
+        Ep = (uint32_t)prm.e * 0x10001u;
+        E2p = (uint32_t)prm.e2 * 0x10001u;
+        NEp = ((uint32_t)(-prm.e) & 0xffffu) * 0x10001u;
+        NE2p = ((uint32_t)(-prm.e2) & 0xffffu) * 0x10001u;
+        NEGp = U_NEG * 0x10001u;
+        L0LO = (lane == 0 && wk == 0) ? 0x0000ffffu : 0u;
+        L31HI = (lane == G - 1 && wk == K - 1) ? 0xffff0000u : 0u;
+        xe0 = xe1 = NEGp;
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+            Hev[p] = Hod[p] = Eo[p] = E2o[p] = Fo[p] = F2o[p] = NEGp;
+        }
+        {
+            const int32_t k0 = min(max(w + 1 - j0, 0), C);     // first local slot beyond the band
+            DF2 = (uint32_t)(k0 - 1) * 0x10001u;
+            if constexpr (DMREG) {
+#pragma unroll
+                for (int p = 0; p < P; ++p)
+                    DMR[p] = prmt(DF2 - ((uint32_t)p | ((uint32_t)(p + P) << 16)), 0, 0xbb99);
+            }
+        }
+        gmax = 0;
+        pend_r = -3;
+        pend_rb = ~0u;
+        if (leader()) {
+            cold.mqe = K_NEG_OUT; cold.mqe_t = -1; cold.mte = K_NEG_OUT; cold.mte_q = -1;
+            cold.gscore = K_NEG_OUT;
+            cold.gt = -1; cold.gq = -1;
+        }
+        __syncwarp(gmask());
+        group_sync();
+        zdropped = 0;
+
+        init_windows(-2);
+        int32_t r;
+        if constexpr (LAZY) r = lazy_pair(use_fast);
+        else r = steps(-2, use_fast);
         if (ovf) return false;
         locate_pending();
         if constexpr (DIR) {
@@ -1188,7 +1717,6 @@ struct WarpPair16 {
         prm = Bt.params;
         lane = lane_;
         tlen = Bt.t_len[pair]; qlen = Bt.q_len[pair];
-        int32_t tph, qph;
         {
             const int64_t toff = Bt.t_off[pair], qoff = Bt.q_off[pair];
             const int64_t tw0 = toff >> 4, qw0 = qoff >> 4;
@@ -1246,7 +1774,7 @@ struct WarpPair16 {
         __syncwarp(gmask());
         zdropped = 0;
         int32_t r = -2;
-        init_windows(r, tph, qph);
+        init_windows(r);
         bool stop = head_step(r);
         const int32_t head_end = min(last_r, w + 1);
         while (!stop && r < head_end) {
@@ -1279,27 +1807,28 @@ warp16_align_kernel(const DevBatch *__restrict__ d_batch, int32_t use_fast, int3
     __shared__ Cold16 cold[WARP_BLOCK_THREADS / G];
     const DevBatch B = *d_batch;
     const int lane = threadIdx.x & (G - 1);
-    const uint32_t gm = G == 32 ? FULL : 0xffffu << (threadIdx.x & 16);
     const WorkList L = work_list(B, list);
-    // the larger register budget of each slot count: 4 blocks per SM for
-    // 4 slots per lane, 2 for 20 and 24, 3 otherwise
-    constexpr bool HIGH = C == 4 ? MINB == 4 : ((C == 24 || C == 20) ? MINB == 2 : MINB == 3);
-    using Pair = WarpPair16<C, (MINB < 4 && C <= 16) || MINB < 3, true, false, true, 1, HIGH, HIGH, G>;
     if constexpr (G == 32) {
+        using Pair = WarpPair16<C, false, false, false, true, 1, true, false, 32, true>;
+        extern __shared__ uint4 lazy_smem[];
+        const int32_t l_end = __reduce_max_sync(FULL, L.end);
+        uint4 *ck = lazy_smem + (threadIdx.x >> 5) * (2 * Pair::CKV * 32 + Pair::RING / 4);
         for (;;) {
-            int32_t k = 0;
+            int32_t k = INT_MIN;
             if (lane == 0) k = L.begin + atomicAdd(L.head, 1);
-            k = __shfl_sync(gm, k, 0, G);
-            if (k >= L.end) break;
+            k = __reduce_max_sync(FULL, k);
+            if (k >= l_end) break;
             const int32_t pair = L.items ? L.items[k] : k;
-            if (!L.items && (!pair_valid(B, pair) || !warp_takes(B, pair))) continue;
+            if (__any_sync(FULL, !L.items && (!pair_valid(B, pair) || !warp_takes(B, pair)))) continue;
             Pair wp(cold[threadIdx.x / G]);
+            wp.ck = ck;
             if (!wp.run(B, pair, lane, use_fast != 0) && lane == 0) {
                 const int32_t slot = atomicAdd(&B.counters[CTR_NOVF], 1);
                 B.ovf_list[slot] = pair;
             }
         }
     } else {
+        using Pair = WarpPair16<C, MINB < 4, true, false, true, 1, true, true, G>;
         // The warp takes two neighbouring pairs of the longest-first queue at
         // once (about the same length), one per half, and both halves start
         // their next pairs together: the two then pass through the same step
@@ -1375,10 +1904,19 @@ int occupancy_warp16k_c() {
     return nb > 0 ? nb : 1;
 }
 
+// Dynamic shared memory of a block: two checkpoints and the edge ring of every
+// warp.
+template <int C, int G>
+constexpr int warp16_smem() {
+    using Pair = WarpPair16<C, false, false, false, true, 1, false, false, 32, true>;
+    return G == 32 ? (WARP_BLOCK_THREADS / 32) * (2 * Pair::CKV * 32 * 16 + Pair::RING * 4) : 0;
+}
+
 template <int C, int MINB, int G>
 cudaError_t launch_warp16_c(const DevBatch *d_batch, int n_blocks, cudaStream_t s, int use_fast,
                             int list) {
-    warp16_align_kernel<C, MINB, G><<<n_blocks, WARP_BLOCK_THREADS, 0, s>>>(d_batch, use_fast, list);
+    warp16_align_kernel<C, MINB, G><<<n_blocks, WARP_BLOCK_THREADS, warp16_smem<C, G>(), s>>>(d_batch, use_fast,
+                                                                                              list);
     return cudaGetLastError();
 }
 
@@ -1391,7 +1929,7 @@ cudaError_t launch_warp16_prio(const DevBatch *d_batch, int n_blocks, cudaStream
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)n_blocks);
     cfg.blockDim = dim3(WARP_BLOCK_THREADS);
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = warp16_smem<C, 32>();
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributePriority;
@@ -1401,11 +1939,15 @@ cudaError_t launch_warp16_prio(const DevBatch *d_batch, int n_blocks, cudaStream
     return cudaLaunchKernelEx(&cfg, warp16_align_kernel<C, MINB, 32>, d_batch, use_fast, list);
 }
 
+// Resident blocks per SM; also lets the kernel have its shared memory, so a
+// plan is made before the first launch on a device.
 template <int C, int MINB, int G>
 int occupancy_warp16_c() {
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, warp16_align_kernel<C, MINB, G>,
-                                                      WARP_BLOCK_THREADS, 0) != cudaSuccess)
+    if (cudaFuncSetAttribute(warp16_align_kernel<C, MINB, G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             warp16_smem<C, G>()) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, warp16_align_kernel<C, MINB, G>,
+                                                      WARP_BLOCK_THREADS, warp16_smem<C, G>()) != cudaSuccess)
         return 1;
     return nb > 0 ? nb : 1;
 }

@@ -4,10 +4,10 @@
 #include "kernel_tb.cuh"
 
 namespace agatha {
-template cudaError_t launch_warp16_c<8, 4>(const DevBatch *, int, cudaStream_t, int, int);
-template int occupancy_warp16_c<8, 4>();
 template cudaError_t launch_warp16_c<8, 3>(const DevBatch *, int, cudaStream_t, int, int);
 template int occupancy_warp16_c<8, 3>();
+template cudaError_t launch_warp16_c<8, 2>(const DevBatch *, int, cudaStream_t, int, int);
+template int occupancy_warp16_c<8, 2>();
 // two pairs per warp, 16 lanes of 8 slots (the 4-slot band of 128 slots)
 template cudaError_t launch_warp16_c<8, 3, 16>(const DevBatch *, int, cudaStream_t, int, int);
 template int occupancy_warp16_c<8, 3, 16>();

@@ -168,13 +168,12 @@ static cudaError_t launch_warp(int C, const DevBatch *d, int blocks, cudaStream_
 static cudaError_t launch_warp16(int C, int high, const DevBatch *d, int blocks, cudaStream_t s,
                                  int fast, int list) {
     switch (C * 2 + high) {
-        case 8: return launch_warp16_c<4, 6>(d, blocks, s, fast, list);
-        case 9: return launch_warp16_c<4, 4>(d, blocks, s, fast, list);
-        case 16: return launch_warp16_c<8, 4>(d, blocks, s, fast, list);
-        case 17: return launch_warp16_c<8, 3>(d, blocks, s, fast, list);
-        case 32: return launch_warp16_c<16, 4>(d, blocks, s, fast, list);
-        case 33: return launch_warp16_c<16, 3>(d, blocks, s, fast, list);
-        case 48: return launch_warp16_c<24, 3>(d, blocks, s, fast, list);
+        case 8: return launch_warp16_c<4, 4>(d, blocks, s, fast, list);
+        case 9: return launch_warp16_c<4, 3>(d, blocks, s, fast, list);
+        case 16: return launch_warp16_c<8, 3>(d, blocks, s, fast, list);
+        case 17: return launch_warp16_c<8, 2>(d, blocks, s, fast, list);
+        case 32: return launch_warp16_c<16, 3>(d, blocks, s, fast, list);
+        case 33: return launch_warp16_c<16, 2>(d, blocks, s, fast, list);
         default: return launch_warp16_c<24, 2>(d, blocks, s, fast, list);
     }
 }
@@ -218,13 +217,12 @@ cudaError_t launch_overflow_int32(const Slot *sl, const LaunchPlan &lp, cudaStre
 
 int warp16_occupancy(int C, int high) {
     switch (C * 2 + high) {
-        case 8: return occupancy_warp16_c<4, 6>();
-        case 9: return occupancy_warp16_c<4, 4>();
-        case 16: return occupancy_warp16_c<8, 4>();
-        case 17: return occupancy_warp16_c<8, 3>();
-        case 32: return occupancy_warp16_c<16, 4>();
-        case 33: return occupancy_warp16_c<16, 3>();
-        case 48: return occupancy_warp16_c<24, 3>();
+        case 8: return occupancy_warp16_c<4, 4>();
+        case 9: return occupancy_warp16_c<4, 3>();
+        case 16: return occupancy_warp16_c<8, 3>();
+        case 17: return occupancy_warp16_c<8, 2>();
+        case 32: return occupancy_warp16_c<16, 3>();
+        case 33: return occupancy_warp16_c<16, 2>();
         default: return occupancy_warp16_c<24, 2>();
     }
 }
@@ -279,10 +277,8 @@ static cudaError_t enqueue_part(agatha_ctx *ctx, Slot *sl, const LaunchPlan &lp,
             // and the second's fill them as the first's leave
             if ((e = cudaEventRecord(sl->fork, s)) != cudaSuccess) return e;
             if ((e = cudaStreamWaitEvent(sl->aux[0], sl->fork, 0)) != cudaSuccess) return e;
-            e = lp.regs_high ? launch_warp16_prio<24, 2>(d, lp.warp16_blocks[1], s, lp.fast, WARP_LIST_MAIN,
-                                                         ctx->prio_greatest)
-                             : launch_warp16_prio<24, 3>(d, lp.warp16_blocks[0], s, lp.fast, WARP_LIST_MAIN,
-                                                         ctx->prio_greatest);
+            e = launch_warp16_prio<24, 2>(d, lp.warp16_blocks[lp.regs_high], s, lp.fast, WARP_LIST_MAIN,
+                                          ctx->prio_greatest);
             if (e != cudaSuccess) return e;
             if ((e = launch_warp16_prio<20, 2>(d, lp.narrow_blocks, sl->aux[0], lp.fast, WARP_LIST_NARROW,
                                                ctx->prio_least)) != cudaSuccess)

@@ -1,0 +1,84 @@
+"""The 16-bit kernel's lazy blocks against the oracle, every field of every
+pair, where the blocks can go wrong: bands whose edge falls in each register
+of a lane (and in the frame's last slot), tables shorter than the band or
+just longer, tables whose corner leaves the band, ends of every parity,
+divergent tails (the Z-drop bound), long indels (a peak passed and taken
+back), and scorings at the edges of the drift (one piece, the second piece
+always the cheaper, an extension dearer than a match, steep enough for a
+rebase in every block).  Every output is an integer: equality."""
+import numpy as np
+import pytest
+
+from paper_2403_06478_gb300 import agatha as A
+from paper_2403_06478_gb300 import workload as W
+
+pytestmark = pytest.mark.gpu
+
+TWO = W.ONT_SCORING
+ONE = W.BWA_SCORING
+SCORINGS = {
+    "two": TWO,
+    "one": ONE,
+    "second_cheaper": W.Scoring(a=2, b=4, q=4, e=6, q2=5, e2=1, zdrop=200, end_bonus=3),
+    "dear_extension": W.Scoring(a=1, b=1, q=0, e=1, q2=0, e2=1, zdrop=60),
+    "steep": W.Scoring(a=40, b=90, q=60, e=30, q2=200, e2=20, zdrop=3000),
+    "no_zdrop": W.Scoring(a=2, b=4, q=4, e=2, q2=24, e2=1, zdrop=-1),
+    "free_mismatch": W.Scoring(a=1, b=0, q=2, e=1, q2=2, e2=1, zdrop=30),
+}
+
+
+def _pairs(w, scoring, seed, n=72):
+    rng = np.random.default_rng(seed)
+    qs, ts = [], []
+    lens = [1, 2, 3, 7, 33, w // 2, w - 3, w - 1, w, w + 1, w + 2, w + 3, w + 5, w + 9, w + 40, 2 * w, 2 * w + 1,
+            3 * w + 11, 5 * w + 300]
+    for i in range(n):
+        ql = max(1, lens[i % len(lens)] + int(rng.integers(0, 3)))
+        q = rng.integers(0, 4, ql, dtype=np.uint8)
+        em = W.ErrorModel(0.06, 0.03, 0.03, tail_frac=0.3 if i % 3 else 0.0)
+        t, _ = W._mutate_chunk(rng, q, np.array([ql], np.int32), em)
+        if i % 5 == 1 and len(t) > 80:              # a long gap: the maximum falls and recovers
+            k = int(rng.integers(2, max(4, min(60, w))))
+            at = int(rng.integers(10, len(t) - 70))
+            t = np.concatenate([t[:at], t[at + k:]])
+        if i % 7 == 2:                               # the corner off the band, or nearly
+            t = t[:max(1, len(t) - w + int(rng.integers(-2, 3)))]
+        if i % 11 == 3:
+            t = np.concatenate([t, rng.integers(0, 4, w + int(rng.integers(-2, 3)), dtype=np.uint8)])
+        qs.append(q)
+        ts.append(t if len(t) else np.zeros(1, np.uint8))
+    return W.from_pairs(qs, ts, scoring)
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    with A.Context(0) as c:
+        yield c
+
+
+BANDS = [5, 8, 9, 100, 101, 102, 103, 126, 127, 128, 131, 132, 133, 134, 255, 256] + list(range(493, 513)) + \
+        [630, 638, 639, 640, 744, 751, 755, 758, 759, 760, 766, 767]
+
+
+@pytest.mark.parametrize("w", BANDS)
+def test_bands(ctx, w):
+    from oracle import oracle as O
+    scoring = ONE if w % 2 else TWO
+    batch = _pairs(w, W.replace(scoring, w=w), seed=w)
+    ref = O.align_batch(batch)
+    for flags in (0, A.AGATHA_REGS_HIGH):
+        got = A.agatha_align_batch(ctx, batch, flags=flags)
+        bad = A.results_equal(got, ref, O.COMPARE_FIELDS)
+        assert bad.size == 0, f"pairs {bad[:5]}"
+        assert got["lane16"].all()
+
+
+@pytest.mark.parametrize("w", [100, 200, 500, 750])
+@pytest.mark.parametrize("name", sorted(SCORINGS))
+def test_scorings(ctx, name, w):
+    from oracle import oracle as O
+    batch = _pairs(w, W.replace(SCORINGS[name], w=w), seed=1000 + w)
+    ref = O.align_batch(batch)
+    got = A.agatha_align_batch(ctx, batch)
+    bad = A.results_equal(got, ref, O.COMPARE_FIELDS)
+    assert bad.size == 0, f"pairs {bad[:5]}"
