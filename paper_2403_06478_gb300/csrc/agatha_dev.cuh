@@ -187,6 +187,15 @@ __device__ __forceinline__ uint32_t load16(const uint32_t *__restrict__ p, int64
     return __funnelshift_r(lo, hi, sh);
 }
 
+// 16 bases from word-relative base index a of a pair's own words (any a;
+// outside the span words: 0).
+__device__ __forceinline__ uint32_t load_rel(const uint32_t *__restrict__ p, int32_t span, int32_t a) {
+    const int32_t wi = a >> 4;                     // floor for negative a too
+    const uint32_t lo = (uint32_t)wi < (uint32_t)span ? __ldg(p + wi) : 0u;
+    const uint32_t hi = (uint32_t)(wi + 1) < (uint32_t)span ? __ldg(p + wi + 1) : 0u;
+    return __funnelshift_r(lo, hi, (uint32_t)(a & 15) * 2u);
+}
+
 // 32 consecutive bases starting at g.
 __device__ __forceinline__ uint64_t load32(const uint32_t *__restrict__ p, int64_t n_words,
                                            int64_t g) {
@@ -286,10 +295,11 @@ struct TbItem {
 // Launchers (defined in the .cu files).
 cudaError_t launch_prep(const DevBatch *d_batch, int64_t n_pairs, int32_t sort, cudaStream_t s,
                         int n_sm);
-template <int C>
+// The int32 kernel with C slots per lane; K warps share a pair's band (1 or 3).
+template <int C, int K = 1>
 cudaError_t launch_warp_c(const DevBatch *d_batch, int n_blocks, cudaStream_t s, int use_fast,
                           int list = WARP_LIST_MAIN);
-template <int C>
+template <int C, int K = 1>
 int occupancy_warp_c();
 // MINB: resident blocks per SM the 16-bit kernel's registers are cut for.
 // G: lanes per pair (32, or 16 for two pairs per warp).

@@ -184,7 +184,7 @@ tb_kernel(const DevBatch *__restrict__ d_batch, const TbItem *__restrict__ items
         const TbItem it = items[k];
         uint8_t *dt = dir + it.dir_off;
         {
-            WarpPair<C, true> wp;
+            WarpPair<C> wp;
             wp.run_dir(B, it.pair, lane, it.end_t + it.end_q, dt);
         }
         __syncwarp();   // the table rows this warp wrote are read by other lanes

@@ -47,7 +47,7 @@
 //
 // The score path with one warp per pair (LAZY) goes further: nearly all its
 // anti-diagonals, the head's and the tail's too, run in blocks whose step
-// leaves out the maximum, the test and every mask (lazy_step, lazy_pair),
+// leaves out the maximum, the test and every mask (lazy_step, lazy_drive),
 // because the integer ALU pipe bounds this kernel (80% busy) and that step
 // has 75 of its instructions per 16-slot anti-diagonal where the bulk step
 // has 114 and the masked step about 250.  Measured on one GB300, whole calls:
@@ -61,7 +61,7 @@
 #include <climits>
 #include <type_traits>
 
-#include "kernel_warp.cuh"
+#include "lazy_drive.cuh"
 
 namespace agatha {
 
@@ -95,16 +95,6 @@ __device__ __forceinline__ uint32_t half_sign_of_diff(uint32_t a, uint32_t b) {
 __device__ __forceinline__ uint32_t mux(uint32_t m, uint32_t x, uint32_t y) {
     return (m & x) | (~m & y);
 }
-
-struct Cold16 {
-    int32_t mqe, mqe_t, mte, mte_q, gscore;
-    int32_t gt, gq;               // cell of the global maximum
-    int32_t Dp, LOWCHK, kint;     // step bound, lowest allowed score, rebase interval
-    // LAZY: the two checkpoints (their registers lie in dynamic shared memory):
-    // anti-diagonal, start of its drift, base, and the steps then left to the
-    // next rebase
-    int32_t ck_r[2], ck_rs[2], ck_base[2], ck_u0[2];
-};
 
 // What the K warps sharing one pair's band (K > 1) hand each other through
 // shared memory after every anti-diagonal, double-buffered by its parity:
@@ -307,14 +297,6 @@ struct WarpPair16 {
     __device__ __forceinline__ int32_t frame(int32_t r) const { return floor_div2(r - w); }
 
     // ------------------------------------------------------------ windows
-    // 16 bases from word-relative base index a (any a; outside the span: 0)
-    __device__ __forceinline__ static uint32_t load_rel(const uint32_t *__restrict__ p, int32_t span,
-                                                        int32_t a) {
-        const int32_t wi = a >> 4;                     // floor for negative a too
-        const uint32_t lo = (uint32_t)wi < (uint32_t)span ? __ldg(p + wi) : 0u;
-        const uint32_t hi = (uint32_t)(wi + 1) < (uint32_t)span ? __ldg(p + wi + 1) : 0u;
-        return __funnelshift_r(lo, hi, (uint32_t)(a & 15) * 2u);
-    }
     __device__ __forceinline__ static uint64_t load_rel32(const uint32_t *__restrict__ p, int32_t span,
                                                           int32_t a) {
         return (uint64_t)load_rel(p, span, a) | ((uint64_t)load_rel(p, span, a + 16) << 32);
@@ -1002,7 +984,7 @@ struct WarpPair16 {
     // The termination rule needs an anti-diagonal's maximum only where it can
     // change the global maximum for good or end the extension.  Blocks of up
     // to 2 * LAZY_PAIRS anti-diagonals run without it where neither can happen
-    // unseen (lazy_run); this is their step.  Against the exact step it drops
+    // unseen (lazy_drive); this is their step.  Against the exact step it drops
     // the running maximum, the warp reduction and the test, the masks of the
     // slots off the band and the table, and half of the second gap piece's work:
     //  - Scores drift upwards by d per anti-diagonal (d = e2, or e when the
@@ -1025,17 +1007,14 @@ struct WarpPair16 {
     //    column, feed nothing of the table (see step and head_bounds_ok).
     // Minus infinity stays at U_NEG under the drift; every score is then at
     // least U_NEG, because the drifting gap state never falls.
-    static constexpr int LAZY_PAIRS = 16;                // one word of each sequence
     static constexpr int CKV = 6 * P / 4;                // 16-byte words of a checkpoint per lane
-    static constexpr int RING = 2 * 2 * LAZY_PAIRS * P;  // words of the edge ring (row | column)
+    static constexpr int EDGE_PAIRS = LAZY_PAIRS;        // pairs of a block with the last row or column
+    static constexpr int RING = 2 * 2 * EDGE_PAIRS * P;  // words of the edge ring (row | column)
     static constexpr int TW = C <= 16 ? 2 : 3;           // window words: C bases and 16 to come
 
     struct LazyWin { uint32_t t[TW], q[TW]; };
     // packed constants (H2: the offset of h; D: the drift), the slot w + 1 mask
-    struct LazyConst { uint32_t A, NE, OE, H2, D, top; };
-    // where the last row's and column's cells sit, as slots of this lane
-    // (on: the block may hold such cells; uniform) and the ring's shared address
-    struct LazyEdge { int32_t on, dt, dq; uint32_t ring; };
+    struct LazyConst { uint32_t A, NE, OE, H2, D, top; int32_t pr; };
 
     // Windows of anti-diagonal r and the 16 bases after them: t field i is
     // T[B + j0 + i]; q holds the bases in falling order, field 16 + jl of the
@@ -1179,18 +1158,17 @@ struct WarpPair16 {
         }
     }
     template <bool TWO, int PR = 0>
-    __device__ __forceinline__ void lazy_dispatch(int32_t pr, int32_t n, LazyWin &W, const LazyConst &k,
-                                                  LazyEdge &g) {
+    __device__ __forceinline__ void lazy_block(int32_t n, LazyWin &W, const LazyConst &k, LazyEdge &g) {
         if constexpr (PR == P) {
             lazy_pairs<TWO, PR>(n, W, k, g);
         } else {
-            if (pr == PR) lazy_pairs<TWO, PR>(n, W, k, g);
-            else lazy_dispatch<TWO, PR + 1>(pr, n, W, k, g);
+            if (k.pr == PR) lazy_pairs<TWO, PR>(n, W, k, g);
+            else lazy_block<TWO, PR + 1>(n, W, k, g);
         }
     }
 
     // Into the drifting form after anti-diagonal r ((r - w) odd), and back.
-    __device__ __forceinline__ void lazy_enter(const LazyConst &k) {
+    __device__ __forceinline__ void lazy_enter(const LazyConst &k, bool) {
 #pragma unroll
         for (int p = 0; p < P; ++p) {
             Hod[p] -= k.H2;
@@ -1235,33 +1213,6 @@ struct WarpPair16 {
         }
         return __reduce_max_sync(FULL, (int32_t)max(lmax & 0xffffu, lmax >> 16));
     }
-    // The best score on the last row and column of anti-diagonals r0 + 1 ..
-    // r0 + 2n (lane i takes the i-th of them) from the ring.  off: from a
-    // drifting h of anti-diagonal r0 to its true score.
-    __device__ __forceinline__ void lazy_edges(const uint32_t *ring, int32_t r0, int32_t n, int32_t off, int32_t d) {
-        __syncwarp();
-        const int32_t r = r0 + 1 + lane, B = frame(r);
-        off -= d * (1 + lane);
-        const int32_t lo = max(max(0, r - qlen + 1), ceil_div2(r - w)), hi = min(min(tlen - 1, r), floor_div2(r + w));
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            const int32_t t = c == 0 ? tlen - 1 : r - qlen + 1;
-            int32_t v = INT_MIN;
-            if (lane < 2 * n && lo <= t && t <= hi) {
-                const int32_t local = (t - B) % C;
-                v = half_of(ring[c * (RING / 2) + lane * P + local % P], local) + off;
-            }
-            const int32_t m = __reduce_max_sync(FULL, v);
-            if (m > (c == 0 ? cold.mte : cold.mqe)) {
-                const int32_t at = r0 + 1 + __ffs(__ballot_sync(FULL, v == m)) - 1;
-                if (lane == 0) {
-                    if (c == 0) { cold.mte = m; cold.mte_q = at - (tlen - 1); }
-                    else { cold.mqe = m; cold.mqe_t = at - (qlen - 1); }
-                }
-            }
-        }
-        __syncwarp();
-    }
     // Checkpoints: the packed registers of the drifting form.
     __device__ __forceinline__ uint32_t &lazy_word(int i) {
         return i < P ? Hev[i] : (i < 2 * P ? Hod[i - P] : (i < 3 * P ? Eo[i - 2 * P]
@@ -1291,174 +1242,38 @@ struct WarpPair16 {
             lazy_word(4 * i + 3) = v.w;
         }
     }
-    // Pairs of anti-diagonals the next block may hold: n, 8 or 4 (0: none) such
-    // that no anti-diagonal of it can fire the Z-drop test.  g, m, mu: an upper
-    // bound of the global maximum, the maximum of the last two anti-diagonals,
-    // and that maximum with the virtual cells.  k anti-diagonals on, no score is
-    // above mu + a ceil(k/2), and the maximum is at least m - o - c ceil(k/2):
-    // away from the last row and column (c = b, o = min(q+e, q2+e2)) the cell
-    // of m continues along its diagonal, after one gap step if the parity asks
-    // for it; near them (c = max(b, 2e), o = q+e + q + c) it may have to go on
-    // along the edge by a gap, towards the corner, which lies in the band.
-    __device__ __forceinline__ int32_t lazy_span(int32_t n, int32_t g, int32_t m, int32_t mu, int32_t o,
-                                                 int32_t c) const {
-        if (prm.zdrop < 0) return n;
-#pragma unroll 1
-        while (n > 0 && max(g - m, mu - m + prm.a * n) + o + c * n > prm.zdrop)
-            n = n > 8 ? 8 : (n > 4 ? 4 : (n > 2 ? 2 : 0));
-        return n;
-    }
-
-    // The pair on lazy blocks and, where they may not run, the masked step.
-    // At the end of each block the maximum of its last two anti-diagonals is
-    // taken; a score inside the block is at most U, from that maximum and the
-    // one at the block's start (a up, c down per two anti-diagonals: U weighs
-    // the two bounds so that its place drops out).  A block whose U does not
-    // exceed the largest maximum seen before it cannot hold the global maximum;
-    // one whose U stays below a later maximum does not hold it for good either.
-    // So only the blocks since the last checkpoint that this rules in can hold
-    // it, and when the exact maximum and its cell are wanted (the Z-drop bound
-    // no longer holds, the score has passed a peak, or the table ends) the pair
-    // goes back to that checkpoint and takes the masked step from there up to
-    // exact_until.  Blocks start and end on odd anti-diagonals ((r - w) odd).
-    // The head's last four anti-diagonals (w - 2 .. w + 1), where the virtual
-    // cells leave the band, run the masked step without its test (blind), as a
-    // block of their own; a band that covers the table (cover) has no such
-    // place.  Returns the last anti-diagonal processed.
-    __device__ __forceinline__ int32_t lazy_pair(bool use_fast) {
-        constexpr int32_t NONE = INT_MIN;
-        const bool head = use_fast && w >= 8 && head_bounds_ok();    // lazy blocks in the head too
-        const int32_t L = min(tlen, qlen);
-        const int32_t r_in = max(L - 2, 2 * L - 3 - w);    // no cell of the last row or column up to here
-        // lazy blocks end here at the latest; past r_in only if the corner is in the band
-        const int32_t end = abs(tlen - qlen) <= w ? last_r - 1 : r_in;
-        const int32_t turn = cover ? INT_MAX : w - 3;      // the crossing of the head's end starts after it
-        const int32_t c0 = prm.b, c1 = max(prm.b, 2 * prm.e);
-        const int32_t o0 = min(oe, oe2), o1 = oe + prm.q + c1;
-        const bool two = prm.q2 != prm.q || prm.e2 != prm.e;
+    // What lazy_drive asks of the lanes.
+    __device__ __forceinline__ static constexpr bool owns() { return true; }
+    static constexpr bool REBASES = true;
+    __device__ __forceinline__ LazyConst lazy_consts(bool) const {
         LazyConst k;
-        const int32_t d = prm.e2, hoff = prm.q2;
-        k.D = (uint32_t)d * 0x10001u;
-        k.H2 = (uint32_t)hoff * 0x10001u;
+        k.D = (uint32_t)prm.e2 * 0x10001u;
+        k.H2 = (uint32_t)prm.q2 * 0x10001u;
         k.A = A2 + k.H2 + 2 * k.D;
-        k.NE = ((uint32_t)(d - prm.e) & 0xffffu) * 0x10001u;
+        k.NE = ((uint32_t)(prm.e2 - prm.e) & 0xffffu) * 0x10001u;
         k.OE = OEp - k.D;
         const int32_t s1 = (w + 1) % C;
-        const int32_t pr = w + 1 < NS ? s1 % P : P;
-        k.top = pr == P ? L31HI : (lane == (w + 1) / C ? (s1 >= P ? 0xffff0000u : 0x0000ffffu) : 0u);
-        const float inv0 = 1.0f / (float)max(prm.a + c0, 1), inv1 = 1.0f / (float)max(prm.a + c1, 1);
-        const uint32_t ring = (uint32_t)__cvta_generic_to_shared(ck + 2 * CKV * 32);
-
-        int32_t r = -3;
-        // the masked step runs up to exact_until, first the first r >= 1 with (r - w) odd
-        int32_t exact_until = !use_fast ? INT_MAX : (head ? 1 + (w & 1) : w + 1);
-        // blocks under way: the largest maximum seen, the bound of the blocks not
-        // ruled out (NONE: there are none, the global maximum is best), its value
-        // at the checkpoint, the checkpoint, the one at the block's start
-        bool open = false;
-        int32_t best = 0, upper = NONE, gval = 0, old = 0, last = 0;
-        int32_t m0 = 0, mu = 0, n = 0;                     // the current block: see lazy_span
-        bool block = false, edge = false;
-        for (;;) {
-            if (r < exact_until || !((r - w) & 1)) {
-                if (r >= last_r) return r;
-                ++r;
-                if (r > -2) advance(r);
-                if (head_step(r)) return r;
-                if (until_rebase <= 2 && r >= 0) {
-                    rebase(last_m, r, table_bits(r) | virtual_bits(r), table_bits(r - 1) | virtual_bits(r - 1));
-                    if (ovf) return r;
-                }
-                continue;
-            }
-            if (!open) {
-                if (r <= w && r > turn) { exact_until = w + 1; continue; }
-                if (r + 8 > (r <= w && w + 1 > end ? min(turn, end) : end)) { exact_until = INT_MAX; continue; }
-                if (lazy_span(4, gmax, to_true(last_m), to_true(last_m), o1, c1) != 4) { exact_until = r + 8; continue; }
-            }
-            blind = false;
-            if (until_rebase < 16) {
-                const uint32_t in1 = table_bits(r) | virtual_bits(r), in0 = table_bits(r - 1) | virtual_bits(r - 1);
-                rebase(open ? to_u(m0) : last_m, r, in1, in0);
-                if (ovf) return r;
-            }
-            int32_t rs = r, u0 = until_rebase;
-            lazy_enter(k);
-            for (;;) {
-                const int32_t m1 = lazy_max(k, r, r > w && r <= r_in) + hoff - OFF + base - d * (r - rs);
-                if (!open) {
-                    open = true;
-                    best = gval = gmax;
-                    upper = NONE;
-                    old = 1;
-                } else if (block) {
-                    const int32_t rise = m1 - mu + (edge ? prm.q + c1 * n : c0 * n);
-                    const int32_t U = mu + (int32_t)((float)(prm.a * rise) * (edge ? inv1 : inv0)) + 1;
-                    if (m1 > best && m1 > upper) {
-                        // the blocks before this one are ruled out
-                        gval = upper == NONE ? best : -(1 << 29);
-                        old = last;
-                        upper = U;
-                    } else if (U > best) {
-                        if (upper == NONE) { gval = best; old = last; }
-                        upper = max(upper, U);
-                    }
-                    best = max(best, m1);
-                }
-                block = false;
-                m0 = m1;
-                const bool cross = r == turn;
-                if (r + 2 > end || (cross && w + 1 > end) || (upper != NONE && m0 + prm.a * LAZY_PAIRS <= best)) {
-                    exact_until = r;                       // the end, or past a peak
-                    open = false;
-                    break;
-                }
-                const int32_t left = (u0 - (r - rs) - 4) >> 1;
-                if (left < 4) break;                       // a rebase is due
-                edge = cross || r + 2 > r_in;
-                n = (min(edge ? end : r_in, r < turn ? min(turn, end) : end) - r) >> 1;
-                if (edge && n < 2 * LAZY_PAIRS) n = min(n, max(4, (n + 1) >> 1));   // shorter towards the end
-                n = cross ? 2 : min(min(n, left), LAZY_PAIRS);
-                mu = r < w ? max(m0, -gap_cost(prm, r + 1)) : m0;
-                const int32_t fit = lazy_span(n, max(best, upper), m0, mu, edge ? o1 : o0, edge ? c1 : c0);
-                if (fit == 0 || (cross && fit < n)) {
-                    exact_until = r + 8;
-                    open = false;
-                    break;
-                }
-                n = fit;
-                last = old ^ 1;
-                lazy_save(last, r, rs, u0);
-                block = true;
-                if (cross) {
-                    blind = true;
-                    exact_until = r + 4;
-                    break;
-                }
-                LazyWin W;
-                lazy_windows(W, r);
-                const int32_t B = frame(r);
-                LazyEdge g{__reduce_max_sync(FULL, edge ? 1 : 0), tlen - 1 - B - j0, r - qlen + 1 - B - j0, ring};
-                if (two) lazy_dispatch<true>(pr, n, W, k, g);
-                else lazy_dispatch<false>(pr, n, W, k, g);
-                if (edge)
-                    lazy_edges(reinterpret_cast<const uint32_t *>(ck + 2 * CKV * 32), r, n,
-                               hoff - OFF + base - d * (r - rs), d);
-                r += 2 * n;
-            }
-            if (!open && upper != NONE) {                  // back to the checkpoint
-                lazy_load(old);
-                r = __reduce_max_sync(FULL, cold.ck_r[old]);
-                rs = __reduce_max_sync(FULL, cold.ck_rs[old]);
-                base = __reduce_max_sync(FULL, cold.ck_base[old]);
-                u0 = __reduce_max_sync(FULL, cold.ck_u0[old]);
-                gmax = gval;
-            }
-            lazy_leave(k, two, r - rs);
-            until_rebase = u0 - (r - rs);
-            last_m = to_u(m0);
-            init_windows(r);
-        }
+        k.pr = w + 1 < NS ? s1 % P : P;
+        k.top = k.pr == P ? L31HI : (lane == (w + 1) / C ? (s1 >= P ? 0xffff0000u : 0x0000ffffu) : 0u);
+        return k;
+    }
+    // from a drifting h of the anti-diagonal lazy_enter followed to its true score
+    __device__ __forceinline__ int32_t lazy_off() const { return prm.q2 - OFF + base; }
+    __device__ __forceinline__ int32_t lazy_drift() const { return prm.e2; }
+    __device__ __forceinline__ int32_t last_max() const { return to_true(last_m); }
+    __device__ __forceinline__ void set_last_max(int32_t m) { last_m = to_u(m); }
+    __device__ __forceinline__ void lazy_rebase(int32_t m, int32_t r) {
+        rebase(to_u(m), r, table_bits(r) | virtual_bits(r), table_bits(r - 1) | virtual_bits(r - 1));
+    }
+    __device__ __forceinline__ bool lazy_head_ok() const { return head_bounds_ok(); }
+    __device__ __forceinline__ uint32_t ring_address() const {
+        return (uint32_t)__cvta_generic_to_shared(ck + 2 * CKV * 32);
+    }
+    // the value of slot j of the i-th anti-diagonal kept in the ring (c: 0 row, 1 column)
+    __device__ __forceinline__ int32_t ring_value(int c, int32_t i, int32_t j) const {
+        const uint32_t *ring = reinterpret_cast<const uint32_t *>(ck + 2 * CKV * 32);
+        const int32_t local = j % C;
+        return half_of(ring[c * (RING / 2) + i * P + local % P], local);
     }
 
     // The pair from anti-diagonal r = -2 on the masked and bulk steps (not
@@ -1677,7 +1492,7 @@ struct WarpPair16 {
 
         init_windows(-2);
         int32_t r;
-        if constexpr (LAZY) r = lazy_pair(use_fast);
+        if constexpr (LAZY) r = lazy_drive(*this, use_fast);
         else r = steps(-2, use_fast);
         if (ovf) return false;
         locate_pending();

@@ -77,16 +77,6 @@ int setup_current_device(DeviceSetup **out) {
     return AGATHA_OK;
 }
 
-cudaError_t launch_warp_any(int C, const agatha::DevBatch *d, int blocks, cudaStream_t s) {
-    switch (C) {
-        case 4: return agatha::launch_warp_c<4>(d, blocks, s, 1);
-        case 8: return agatha::launch_warp_c<8>(d, blocks, s, 1);
-        case 16: return agatha::launch_warp_c<16>(d, blocks, s, 1);
-        case 24: return agatha::launch_warp_c<24>(d, blocks, s, 1);
-        default: return agatha::launch_warp_c<32>(d, blocks, s, 1);
-    }
-}
-
 }  // namespace
 
 extern "C" int agatha_align_batch_noalloc(const agatha_batch *batch, const agatha_params *params,
@@ -117,7 +107,8 @@ extern "C" int agatha_align_batch_noalloc(const agatha_batch *batch, const agath
         wide_w = p.w < 0 ? plain_kernel_max_w() : p.w;
         if (wide_w > plain_kernel_max_w()) return AGATHA_ENOTSUP;
     }
-    const int blocks = ds->n_sm * warp_occupancy(C);
+    const Shape32 shape = pick_shape32(w_plan < warp_w_max ? w_plan : warp_w_max);
+    const int blocks = ds->n_sm * warp32_occupancy(shape);
 
     DevBatch desc;
     desc.q_packed = batch->q_packed;
@@ -146,7 +137,7 @@ extern "C" int agatha_align_batch_noalloc(const agatha_batch *batch, const agath
     if (e == cudaSuccess) e = cudaMemsetAsync(desc.counters, 0, CTR_COUNT * sizeof(int32_t), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(desc.bucket_hist, 0, 256 * sizeof(int64_t), s);
     if (e == cudaSuccess) e = launch_prep(d_desc, batch->n_pairs, 1, s, ds->n_sm);
-    if (e == cudaSuccess) e = launch_warp_any(C, d_desc, blocks, s);
+    if (e == cudaSuccess) e = launch_warp32(shape, d_desc, blocks, s, 1, WARP_LIST_MAIN);
     if (e == cudaSuccess && wide_w > 0) e = launch_plain_kernel(d_desc, (int64_t)ds->n_sm * 2, wide_w, 1, s);
     int32_t ctr[CTR_COUNT] = {0};
     if (e == cudaSuccess)

@@ -152,14 +152,35 @@ int pick_slots_per_lane(int32_t w) {
     return 32;
 }
 
-static cudaError_t launch_warp(int C, const DevBatch *d, int blocks, cudaStream_t s, int fast,
-                               int list) {
-    switch (C) {
-        case 4: return launch_warp_c<4>(d, blocks, s, fast, list);
-        case 8: return launch_warp_c<8>(d, blocks, s, fast, list);
-        case 16: return launch_warp_c<16>(d, blocks, s, fast, list);
-        case 24: return launch_warp_c<24>(d, blocks, s, fast, list);
-        default: return launch_warp_c<32>(d, blocks, s, fast, list);
+// The int32 score kernel's shape for a band of half-width w: slots per lane
+// and warps per pair.  One warp does the least work per cell as long as 16
+// slots per lane hold the band (20,000 pairs of 1,500 bp at w = 500: 17.8 ms
+// against 33.6 with three warps of 8 slots, and even 2,500 ONT-like pairs,
+// which the longest pair bounds, 23.7 against 30.9 ms).  Beyond that its six
+// arrays do not fit the registers any more, and three warps share the band
+// (1,000 ONT-like pairs at w = 1,000: 120 ms on one warp of 32 slots, 30 ms).
+Shape32 pick_shape32(int32_t w) {
+    if (w <= 511) return {w <= 127 ? 4 : (w <= 255 ? 8 : 16), 1};
+    return {w <= 734 ? 8 : 12, 3};
+}
+
+cudaError_t launch_warp32(Shape32 k, const DevBatch *d, int blocks, cudaStream_t s, int fast, int list) {
+    switch (k.C * 4 + k.K) {
+        case 4 * 4 + 1: return launch_warp_c<4, 1>(d, blocks, s, fast, list);
+        case 8 * 4 + 1: return launch_warp_c<8, 1>(d, blocks, s, fast, list);
+        case 16 * 4 + 1: return launch_warp_c<16, 1>(d, blocks, s, fast, list);
+        case 8 * 4 + 3: return launch_warp_c<8, 3>(d, blocks, s, fast, list);
+        default: return launch_warp_c<12, 3>(d, blocks, s, fast, list);
+    }
+}
+
+int warp32_occupancy(Shape32 k) {
+    switch (k.C * 4 + k.K) {
+        case 4 * 4 + 1: return occupancy_warp_c<4, 1>();
+        case 8 * 4 + 1: return occupancy_warp_c<8, 1>();
+        case 16 * 4 + 1: return occupancy_warp_c<16, 1>();
+        case 8 * 4 + 3: return occupancy_warp_c<8, 3>();
+        default: return occupancy_warp_c<12, 3>();
     }
 }
 
@@ -212,7 +233,7 @@ int warp16k_occupancy(int C16, int K) {
 }
 
 cudaError_t launch_overflow_int32(const Slot *sl, const LaunchPlan &lp, cudaStream_t s) {
-    return launch_warp(lp.C, sl->d_desc, lp.warp_blocks, s, lp.fast, WARP_LIST_OVERFLOW);
+    return launch_warp32(lp.shape32, sl->d_desc, lp.warp_blocks, s, lp.fast, WARP_LIST_OVERFLOW);
 }
 
 int warp16_occupancy(int C, int high) {
@@ -234,16 +255,6 @@ int pick_slots16(int32_t w) {
     if (w <= 32 * 16 - 1) return 16;
     if (w <= 32 * 24 - 1) return 24;
     return 0;
-}
-
-int warp_occupancy(int C) {
-    switch (C) {
-        case 4: return occupancy_warp_c<4>();
-        case 8: return occupancy_warp_c<8>();
-        case 16: return occupancy_warp_c<16>();
-        case 24: return occupancy_warp_c<24>();
-        default: return occupancy_warp_c<32>();
-    }
 }
 
 // Enqueue the device work of one batch whose descriptor is already in the
@@ -298,7 +309,7 @@ static cudaError_t enqueue_part(agatha_ctx *ctx, Slot *sl, const LaunchPlan &lp,
                               WARP_LIST_MAIN);
             any16 = true;
         } else {
-            e = launch_warp(lp.C, d, lp.warp_blocks, s, lp.fast, WARP_LIST_MAIN);
+            e = launch_warp32(lp.shape32, d, lp.warp_blocks, s, lp.fast, WARP_LIST_MAIN);
         }
         if (e != cudaSuccess) return e;
     } else {
@@ -310,7 +321,7 @@ static cudaError_t enqueue_part(agatha_ctx *ctx, Slot *sl, const LaunchPlan &lp,
             if ((e = cudaStreamWaitEvent(sc, sl->fork, 0)) != cudaSuccess) return e;
             const int v = lp.cls_var[c];
             if (v == VAR_32) {
-                e = launch_warp(lp.C, d, lp.warp_blocks, sc, lp.fast, WARP_LIST_CLASS + c);
+                e = launch_warp32(lp.shape32, d, lp.warp_blocks, sc, lp.fast, WARP_LIST_CLASS + c);
             } else if (v == VAR_16_HALF) {
                 e = launch_warp16h(lp.C16, d, lp.warp16h_blocks, sc, lp.fast, WARP_LIST_CLASS + c);
                 any16 = true;
@@ -329,7 +340,7 @@ static cudaError_t enqueue_part(agatha_ctx *ctx, Slot *sl, const LaunchPlan &lp,
         }
     }
     // pairs whose scores left the 16-bit range, recomputed on int32 lanes
-    if (any16 && (e = launch_warp(lp.C, d, lp.warp_blocks, s, lp.fast, WARP_LIST_OVERFLOW)) != cudaSuccess)
+    if (any16 && (e = launch_warp32(lp.shape32, d, lp.warp_blocks, s, lp.fast, WARP_LIST_OVERFLOW)) != cudaSuccess)
         return e;
     if (lp.wide_w > 0) e = launch_plain_kernel(d, (int64_t)ctx->n_sm * 2, lp.wide_w, 1, s);
     return e;
@@ -467,8 +478,8 @@ int make_plan(agatha_ctx *ctx, const DevParams &p, const BatchShape &shape, uint
     if (lp->wide_w > pmax)
         return set_error(ctx, AGATHA_ENOTSUP, "band of %d cells is wider than supported (%d)",
                          lp->wide_w, pmax);
-    const int occ = warp_occupancy(lp->C);
-    lp->warp_blocks = ctx->n_sm * occ;
+    lp->shape32 = pick_shape32(std::min(shape.max_w_all, lp->warp_w_max));
+    lp->warp_blocks = ctx->n_sm * warp32_occupancy(lp->shape32);
     // 16-bit packed lanes when the band fits and one anti-diagonal changes a
     // score by at most 255 (the 16-bit kernel then still rebases at least
     // every 50 anti-diagonals)

@@ -70,10 +70,16 @@ struct TuneChoice {
     int8_t split = 0;
 };
 
+// Shape of the int32 score kernel: slots per lane, warps per pair.
+struct Shape32 {
+    int C, K;
+};
+
 struct LaunchPlan {
     int64_t n = 0;
     int plain = 0, sort = 1, fast = 1, use_graph = 1;
-    int C = 16;                 // slots per lane of the int32 kernel
+    int C = 16;                 // slots per lane that hold the widest band on one warp
+    Shape32 shape32 = {16, 1};  // the int32 score kernel's
     int32_t warp_w_max = 0;
     int warp_blocks = 0;
     int lane16 = 0, C16 = 0;    // 16-bit lanes allowed; their slots per lane
@@ -92,7 +98,7 @@ struct LaunchPlan {
     int32_t plain_w = 0;
     int64_t plain_blocks = 0;
     PlanKey key() const {
-        return {plain, C, C16 * lane16, regs_high, sort, fast, wide_w, warp_blocks, split,
+        return {plain, C | (shape32.C << 8) | (shape32.K << 16), C16 * lane16, regs_high, sort, fast, wide_w, warp_blocks, split,
                 split ? cls_var[0] | (cls_var[1] << 4) | (cls_var[2] << 8) | (cls_var[3] << 12) : 0,
                 split ? 1 : groupk, (split ? 0 : half) | (narrow_w > 0 ? 2 : 0)};
     }
@@ -128,7 +134,9 @@ int normalise_params(const agatha_params *in, DevParams *out);
 int validate_host_batch(agatha_ctx *ctx, const agatha_batch *b, const DevParams &p, BatchShape *shape);
 int pick_slots_per_lane(int32_t w);
 int pick_slots16(int32_t w);
-int warp_occupancy(int C);
+Shape32 pick_shape32(int32_t w);
+cudaError_t launch_warp32(Shape32 k, const DevBatch *d, int blocks, cudaStream_t s, int fast, int list);
+int warp32_occupancy(Shape32 k);
 int warp16_occupancy(int C, int high);
 int warp16h_occupancy(int C16);   // two pairs per warp; 0 where none exists
 void apply_narrow(agatha_ctx *ctx, LaunchPlan *lp, uint32_t flags);

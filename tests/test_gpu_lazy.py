@@ -1,4 +1,4 @@
-"""The 16-bit kernel's lazy blocks against the oracle, every field of every
+"""The lazy blocks of the 16-bit and int32 kernels against the oracle, every field of every
 pair, where the blocks can go wrong: bands whose edge falls in each register
 of a lane (and in the frame's last slot), tables shorter than the band or
 just longer, tables whose corner leaves the band, ends of every parity,
@@ -73,11 +73,36 @@ def test_bands(ctx, w):
         assert got["lane16"].all()
 
 
+@pytest.mark.parametrize("w", [5, 8, 100, 127, 128, 200, 255, 500, 511, 512, 750, 767, 768] +
+                         list(range(990, 1024)))
+def test_bands_int32(ctx, w):
+    from oracle import oracle as O
+    batch = _pairs(w, W.replace(ONE if w % 2 else TWO, w=w), seed=5000 + w)
+    ref = O.align_batch(batch)
+    got = A.agatha_align_batch(ctx, batch, flags=A.AGATHA_FORCE32)
+    bad = A.results_equal(got, ref, O.COMPARE_FIELDS)
+    assert bad.size == 0, f"pairs {bad[:5]}"
+    assert not got["lane16"].any()
+
+
 @pytest.mark.parametrize("w", [100, 200, 500, 750])
 @pytest.mark.parametrize("name", sorted(SCORINGS))
 def test_scorings(ctx, name, w):
     from oracle import oracle as O
     batch = _pairs(w, W.replace(SCORINGS[name], w=w), seed=1000 + w)
+    ref = O.align_batch(batch)
+    for flags in (0, A.AGATHA_FORCE32):
+        got = A.agatha_align_batch(ctx, batch, flags=flags)
+        bad = A.results_equal(got, ref, O.COMPARE_FIELDS)
+        assert bad.size == 0, f"flags {flags}: pairs {bad[:5]}"
+
+
+@pytest.mark.parametrize("w", [100, 500, 1000])
+def test_int32_large_scores(ctx, w):
+    """Scores near the int32 headroom the library admits (2^28 for the
+    pair's anti-diagonals), far beyond 16-bit lanes."""
+    from oracle import oracle as O
+    batch = _pairs(w, W.Scoring(a=4000, b=7000, q=1500, e=1200, q2=7000, e2=600, w=w, zdrop=200000), seed=77 + w)
     ref = O.align_batch(batch)
     got = A.agatha_align_batch(ctx, batch)
     bad = A.results_equal(got, ref, O.COMPARE_FIELDS)
