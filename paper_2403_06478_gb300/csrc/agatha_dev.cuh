@@ -171,6 +171,16 @@ __host__ __device__ inline int32_t step_change_max(const DevParams &p) {
     return d > 0 ? d : 1;
 }
 
+// The step bound of the 16-bit lazy blocks: their drift (e2) and half a match
+// per anti-diagonal stay within it too.
+__host__ __device__ inline int32_t lazy_step_max(const DevParams &p) {
+    const int32_t d = step_change_max(p), g = (p.a + 1) / 2 + p.e2;
+    return d > g ? d : g;
+}
+// The 16-bit traceback recomputes up to 36 anti-diagonals between two rebases,
+// which steps of at most this admit (rebase_interval: 44).
+constexpr int32_t TRACE_STEP_MAX = 300;
+
 // One packed word of a stream, zero outside it (reads are clamped).
 __device__ __forceinline__ uint32_t load_word(const uint32_t *__restrict__ p, int64_t n_words,
                                               int64_t i) {

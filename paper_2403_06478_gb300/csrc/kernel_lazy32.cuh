@@ -36,7 +36,7 @@ struct LazyPair32 {
     static_assert(C % 4 == 0 && C <= 32, "4 to 32 slots per lane");
     static constexpr int32_t NS = K == 1 ? 32 * C : (30 * K + 2) * C;
     static constexpr int HALO = 2 * K * 2 * 6 * C;        // words of the halo exchange (double-buffered)
-    static constexpr bool REBASES = false;
+    static constexpr bool REBASES = false, TRACE = false;
     static constexpr int TW = C <= 16 ? 2 : 3;            // window words: C bases and 16 to come
     static constexpr int V = C / 4;                       // 16-byte words of a lane's array
     static constexpr int EDGE_PAIRS = 8;                  // pairs of a block with the last row or column

@@ -1,12 +1,13 @@
 // Traceback kernels: the CIGAR of each extension, after the score path has
 // found its end cell.
 //
-// One warp takes one pair from a device queue (longest first, like the score
-// kernels).  It recomputes anti-diagonals 0..r_end of the pair's band with
-// the warp step of a score kernel in its DIR variant, which writes one
+// Two forms.  tbf16_kernel aligns and traces in one launch (below: "Fused").
+// The others run after the score path: one warp takes one pair from a device
+// queue (longest first, like the score kernels).  It recomputes anti-diagonals
+// 0..r_end of the pair's band with a DIR variant of a score step, which writes one
 // direction byte per band slot: lane L stores its C bytes of anti-diagonal r
 // at table[r * 32C + L*C] with one vector store, so a warp writes a 32C-byte
-// row per step, coalesced.  Two kernels share the walk:
+// row per step, coalesced.  Two such kernels share the walk:
 //   tb16_kernel  the 16-bit packed-lane step (kernel_warp16.cuh): two cells
 //                per instruction, its slot frame B(r) = floor((r-w)/2), bytes
 //                2p and 2p+1 of a lane from the halves of register p; a pair
@@ -99,9 +100,9 @@ struct TbRuns {
     uint32_t *ops;
     int32_t cap, n;
     uint32_t op, len;
-    __device__ __forceinline__ void push(uint32_t o, uint32_t l) {
+    __device__ __forceinline__ void push(uint32_t o, uint32_t l, int32_t lane = 0) {
         if (len > 0 && op == o) { len += l; return; }
-        if (len > 0 && n < cap) ops[n] = (len << 4) | op;
+        if (len > 0 && n < cap && lane == 0) ops[n] = (len << 4) | op;
         if (len > 0) ++n;
         op = o;
         len = l;
@@ -229,55 +230,293 @@ tb16_kernel(const DevBatch *__restrict__ d_batch, const TbItem *__restrict__ ite
     }
 }
 
-// Fused score path and traceback on 16-bit lanes: each warp aligns a pair
-// exactly as warp16_align_kernel does (results, termination, hand-back of
-// pairs that leave the 16-bit range to the int32 score kernel's list) while
-// writing the direction bytes of every anti-diagonal it computes, then walks
-// back from the end cell it found.  The table of an item has room for every
-// anti-diagonal of the pair (tlen + qlen - 1 rows) and its run scratch for
-// tlen + qlen runs; a handed-back pair gets n = -1.
+// Fused score path and traceback on 16-bit lanes.
+//
+// Each warp aligns a pair exactly as warp16_align_kernel does, on lazy blocks,
+// and keeps the band's state of every 32nd anti-diagonal in memory (TRACE).
+// Then it goes back over the segments between those states: it recomputes a
+// segment on the same lazy step, holds the scores of the 34 to 36 anti-diagonals
+// of the few lanes the path can reach in it in shared memory, and follows the
+// path through them.  No direction byte is computed or stored.
+//
+// What bounds it: the integer ALU pipe, twice the score kernel's work (and for
+// a few thousand pairs the longest one).  The form before wrote a direction
+// byte per cell from a step of 36 lane-instructions per cell (against 8 to 9 of
+// the lazy step, twice) and walked back through the table one cell at a time.
+// One GB300, kernel time: 20,000 ONT-like pairs 155 -> 95 ms, 2,000 56 -> 36
+// ms, 20,000 reads of 150 bp 2.4 -> 1.6 ms.
+//
+// The path from scores alone (the rules at the top of this file): a diagonal
+// step is taken wherever H equals the diagonal's H plus the substitution, so
+// the lanes test the coming diagonal cells at once and the run is as long as
+// the first that fails.  There, H came from E iff some cell l steps back in t
+// has H - (q + e l) equal to it, from F iff one l steps back in q, from E2, F2
+// the same with the second piece; the gap's length is the smallest such l
+// (opening is preferred to extending on ties), found by the lanes at once.
+// Past the segment's start the state E (F, E2, F2) kept there stands for all
+// longer gaps: a gap that equals only that one continues in the segment
+// before, where the smallest l is looked for that opens it.
+template <class S>
+struct TraceWin {
+    static constexpr int C = S::P * 2, P = S::P;
+    // lanes that hold 39 neighbouring slots wherever they start: a path and
+    // the gaps from it move at most one slot per two anti-diagonals
+    static constexpr int NL = (39 + C - 1 + C - 1) / C;
+    static constexpr int ROWS = 38;               // the first segment starts at -2
+    static constexpr int WORDS = NL * (ROWS + 4) * P + ROWS;
+    uint32_t *rows;                               // [lane - la][row][register]
+    uint32_t *st;                                 // [E, F, E2, F2][lane - la][register] leaving row rk
+    int32_t *off;                                 // from a row's stored value to the score
+    int32_t la, rk, st_off;
+    __device__ __forceinline__ explicit TraceWin(uint4 *mem)
+        : rows(reinterpret_cast<uint32_t *>(mem)), st(rows + NL * ROWS * P),
+          off(reinterpret_cast<int32_t *>(st + 4 * NL * P)) {}
+    __device__ __forceinline__ int32_t score(const S &s, int32_t t, int32_t r) const {
+        const int32_t j = t - s.frame(r), local = j % C, i = r - rk + 1;
+        return S::half_of(rows[((j / C - la) * ROWS + i) * P + local % P], local) + off[i];
+    }
+    // the gap state k (0 E, 1 F, 2 E2, 3 F2) leaving cell (t, rk - t)
+    __device__ __forceinline__ int32_t state(const S &s, int k, int32_t t) const {
+        const int32_t j = t - s.frame(rk), local = j % C;
+        return S::half_of(st[k * (NL * P) + (j / C - la) * P + local % P], local) + st_off;
+    }
+    __device__ __forceinline__ void keep(const S &s, int32_t r, const uint32_t (&H)[P], int32_t o) {
+        const int32_t l = s.lane - la;
+        if (l >= 0 && l < NL) {
+#pragma unroll
+            for (int p = 0; p < P; ++p) rows[(l * ROWS + r - rk + 1) * P + p] = H[p];
+        }
+        if (s.lane == 0) off[r - rk + 1] = o;
+    }
+};
+
+// Recompute anti-diagonals rk + 1 .. target (or one more) from state seg into
+// the window.
+template <class S>
+__device__ __forceinline__ void trace_segment(S &s, TraceWin<S> &W, int32_t seg, int32_t target,
+                                              const typename S::LazyConst &k, bool two, bool head, int32_t end) {
+    using TW = TraceWin<S>;
+    constexpr int P = S::P;
+    const int32_t w = s.w, d = s.lazy_drift();
+    const int32_t turn = s.cover ? INT_MAX : w - 3;
+    int32_t r, rs = 0;
+    bool drifting = false;
+    if (seg == 0) {
+#pragma unroll
+        for (int p = 0; p < P; ++p)
+            s.Hev[p] = s.Hod[p] = s.Eo[p] = s.E2o[p] = s.Fo[p] = s.F2o[p] = s.NEGp;
+        s.base = 0;
+        r = -3;
+    } else {
+        r = W.rk;
+        drifting = s.trace_load(seg, rs);
+        if (!drifting) {
+            s.lazy_enter(k, two);
+            rs = r;
+            drifting = true;
+        }
+        W.keep(s, r - 1, s.Hev, s.lazy_off() - d * (r - 1 - rs));
+        W.keep(s, r, s.Hod, s.lazy_off() - d * (r - rs));
+        W.st_off = s.base - s.OFF - d * (r + 1 - rs);
+        const int32_t l = s.lane - W.la;
+        if (l >= 0 && l < TW::NL) {
+#pragma unroll
+            for (int p = 0; p < P; ++p) {
+                W.st[l * P + p] = s.Eo[p];
+                W.st[TW::NL * P + l * P + p] = s.Fo[p];
+                W.st[2 * TW::NL * P + l * P + p] = two ? s.E2o[p] : s.Eo[p];
+                W.st[3 * TW::NL * P + l * P + p] = two ? __vmaxu2(s.F2o[p], s.Hod[p]) : s.Fo[p];
+            }
+        }
+    }
+    while (r < target) {
+        // the lazy step wherever it holds (lazy_drive), else the masked one
+        const int32_t limit = r <= w ? (head ? min(turn, end) : INT_MIN) : end;
+        if (r >= s.first_r() && ((r - w) & 1) && limit >= r + 2) {
+            if (!drifting) {
+                s.lazy_enter(k, two);
+                rs = r;
+                drifting = true;
+            }
+            const int32_t n = min((min(target + 1, limit) - r) >> 1, LAZY_PAIRS);
+            typename S::LazyWin B;
+            s.lazy_windows(B, r);
+            const int32_t l = s.lane - W.la;
+            const bool in = l >= 0 && l < TW::NL;
+            const uint32_t *first = W.rows + ((in ? l : 0) * TW::ROWS + r + 1 - W.rk + 1) * P;
+            LazyEdge g{__reduce_max_sync(FULL, 1), in ? 0 : -1, -(1 << 20),
+                       (uint32_t)__cvta_generic_to_shared(first), 0};
+            if (two) s.template lazy_block<true>(n, B, k, g);
+            else s.template lazy_block<false>(n, B, k, g);
+            if (s.lane < 2 * n) W.off[r + 1 + s.lane - W.rk + 1] = s.lazy_off() - d * (r + 1 + s.lane - rs);
+            r += 2 * n;
+        } else {
+            if (drifting) {
+                s.lazy_leave(k, two, r - rs);
+                s.init_windows(r);
+                drifting = false;
+            }
+            ++r;
+            if (r == -2) s.init_windows(r);
+            else s.advance(r);
+            s.head_step(r);
+            W.keep(s, r, ((r - w) & 1) ? s.Hod : s.Hev, s.base - s.OFF);
+        }
+    }
+    __syncwarp();
+}
+
+// Walk back from (s.end_t, s.end_q).  Returns the number of runs.
+template <class S>
+__device__ __forceinline__ int32_t tb_trace(S &s, uint32_t *ops, int32_t cap) {
+    using TW = TraceWin<S>;
+    TW W(s.ck);
+    TbRuns runs{ops, cap, 0, 0u, 0u};
+    const DevParams &prm = s.prm;
+    const int32_t w = s.w, g0 = s.first_r(), lane = s.lane;
+    const bool two = prm.q2 != prm.q || prm.e2 != prm.e;
+    const bool head = w >= 8 && s.lazy_head_ok();
+    const int32_t L = min(s.tlen, s.qlen);
+    const int32_t end = abs(s.tlen - s.qlen) <= w ? s.last_r - 1 : max(L - 2, 2 * L - 3 - w);
+    const auto k = s.lazy_consts(two);
+    s.blind = true;
+    s.ovf = false;
+    int32_t t = s.end_t, q = s.end_q;
+    int32_t kind = -1, tau = 0;               // a gap of this kind under way (-1: none): see below
+    while (t >= 0 && q >= 0) {
+        const int32_t rc = t + q;
+        const int32_t seg = rc <= g0 + 32 ? 0 : (rc - g0 - 1) >> 5;
+        W.rk = seg ? g0 + 32 * seg : -2;
+        W.la = min(max(t - s.frame(rc) - 19, 0) / TW::C, 32 - TW::NL);
+        trace_segment(s, W, seg, rc, k, two, head, end);
+        while (t >= 0 && q >= 0 && t + q > W.rk) {
+            int32_t r = t + q;
+            if (kind < 0) {
+                // lane i: whether cell (t - i, q - i) took the diagonal
+                const int32_t ti = t - lane, qi = q - lane, ri = r - 2 * lane;
+                bool ok = false;
+                if (ti >= 0 && qi >= 0 && ri > W.rk) {
+                    const int32_t tb = ti + s.tph, qb = qi + s.qph;
+                    const uint32_t x = (__ldg(s.tp + (tb >> 4)) >> (2 * (tb & 15))) ^
+                                       (__ldg(s.qp + (qb >> 4)) >> (2 * (qb & 15)));
+                    const int32_t m = max(ti, qi);
+                    const int32_t from = ti && qi ? W.score(s, ti - 1, ri - 2) : (m ? -gap_cost(prm, m) : 0);
+                    ok = W.score(s, ti, ri) == from + ((x & 3u) ? -prm.b : prm.a);
+                }
+                const uint32_t miss = ~__ballot_sync(FULL, ok);
+                const int32_t n = miss ? __ffs(miss) - 1 : 32;
+                if (n > 0) {
+                    runs.push(TB_OP_M, (uint32_t)n, lane);
+                    t -= n;
+                    q -= n;
+                    r -= 2 * n;
+                    if (t < 0 || q < 0 || r <= W.rk) break;
+                }
+            }
+            // a gap: H (or, under way, its state one step on) equals the score
+            // l steps back less the gap's cost
+            const int32_t want = kind < 0 ? W.score(s, t, r) : tau;
+            const int32_t D = r - W.rk;
+            uint64_t hit[4] = {0, 0, 0, 0};       // bit l - 1: the gap of length l
+            for (int32_t l = lane + 1;; l += 32) {
+                // (only the first segment has more than 32 anti-diagonals)
+                constexpr int32_t OUT = -(1 << 29);
+                const int32_t rl = r - l, te = t - l, qf = q - l;
+                int32_t he = OUT, hf = OUT;
+                if (rl >= W.rk) {
+                    if (te >= 0) { if (te - q >= -w) he = W.score(s, te, rl); }
+                    else if (te == -1 && q <= w) he = -gap_cost(prm, q + 1);
+                    if (qf >= 0) { if (t - qf <= w) hf = W.score(s, t, rl); }
+                    else if (qf == -1 && t <= w) hf = -gap_cost(prm, t + 1);
+                }
+                const int32_t c1 = want + prm.q + prm.e * l, c2 = want + prm.q2 + prm.e2 * l;
+                const int sh = l > 32 ? 32 : 0;
+                hit[0] |= (uint64_t)__ballot_sync(FULL, he == c1) << sh;
+                hit[1] |= (uint64_t)__ballot_sync(FULL, hf == c1) << sh;
+                hit[2] |= (uint64_t)__ballot_sync(FULL, he == c2) << sh;
+                hit[3] |= (uint64_t)__ballot_sync(FULL, hf == c2) << sh;
+                if (sh || D <= 32) break;
+            }
+            int32_t at = 0, pick = -1, value = 0;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                if (pick >= 0 || (kind >= 0 && kind != c)) continue;
+                if (hit[c]) {
+                    pick = c;
+                    at = __ffsll((long long)hit[c]);
+                } else if (W.rk > 0) {
+                    // the state leaving the segment's first anti-diagonal, if
+                    // the gap reaches it inside the table and the band
+                    const int32_t ts = (c & 1) ? t : t - D, qs = W.rk - ts;
+                    if (ts >= 0 && qs >= 0 && ts - qs <= w && qs - ts <= w) {
+                        value = W.state(s, c, ts);
+                        if (__any_sync(FULL, value - (c < 2 ? prm.e : prm.e2) * (D - 1) == want)) pick = c;
+                    }
+                }
+            }
+            const int32_t n = at ? at : D;
+            if (pick < 0) {                       // (cannot be; keeps the walk moving)
+                runs.push(TB_OP_M, 1u, lane);
+                --t;
+                --q;
+                kind = -1;
+                continue;
+            }
+            runs.push((pick & 1) ? TB_OP_I : TB_OP_D, (uint32_t)n, lane);
+            if (pick & 1) q -= n;
+            else t -= n;
+            kind = at ? -1 : pick;
+            tau = value + (pick < 2 ? prm.e : prm.e2);
+        }
+        __syncwarp();                             // the window is written again
+    }
+    if (t < 0 && q >= 0) runs.push(TB_OP_I, (uint32_t)(q + 1), lane);
+    if (q < 0 && t >= 0) runs.push(TB_OP_D, (uint32_t)(t + 1), lane);
+    runs.push(0xfu, 1u, lane);                    // flush the last run
+    return runs.n;
+}
+
+// The memory of an item has room for the direction table of every
+// anti-diagonal of the pair (tlen + qlen - 1 rows of 32 C bytes), of which the
+// states take three eighths, and its run scratch for tlen + qlen runs.  A pair
+// that leaves the 16-bit range goes to the int32 score kernel's list and gets
+// n = -1.
+template <int C>
+using TracePair = WarpPair16<C, false, false, false, 1, true, false, 32, true, true>;
+template <int C>
+__host__ __device__ constexpr int tbf16_warp_smem() {                 // 16-byte words of a warp
+    using S = TracePair<C>;
+    constexpr int a = 2 * S::CKV * 32 + S::RING / 4, b = (TraceWin<S>::WORDS + 3) / 4;
+    return a > b ? a : b;
+}
+
 template <int C, int MINB>
 __global__ void __launch_bounds__(WARP_BLOCK_THREADS, MINB)
 tbf16_kernel(const DevBatch *__restrict__ d_batch, const TbItem *__restrict__ items, int32_t n_items,
-             int32_t *head, uint8_t *dir, uint32_t *ops, int32_t *n_cigar) {
+             int32_t *head, uint8_t *states, uint32_t *ops, int32_t *n_cigar) {
     __shared__ Cold16 cold[WARP_BLOCK_THREADS / 32];
-    __shared__ __align__(16) uint8_t win[WARP_BLOCK_THREADS / 32][TB_WIN_ROWS * TbLayout<C, true>::WB];
+    extern __shared__ uint4 lazy_smem[];
     const DevBatch B = *d_batch;
     const int lane = threadIdx.x & 31;
-    uint8_t *my_win = win[threadIdx.x >> 5];
     for (;;) {
-        int32_t k = 0;
+        int32_t k = INT_MIN;
         if (lane == 0) k = atomicAdd(head, 1);
-        k = __shfl_sync(FULL, k, 0);
+        k = __reduce_max_sync(FULL, k);
         if (k >= n_items) break;
         const TbItem it = items[k];
-        uint8_t *dt = dir + it.dir_off;
-        bool ok;
-        int32_t et, eq;
-        {
-            // without the deferred arg-max (DEFER): its saved registers cost
-            // more here, beside the direction bits, than the searches they save
-            // (measured on the ONT-like batch: 171 against 179 ms)
-            WarpPair16<C, (MINB < 4 && C <= 16) || MINB < 3, false, true, true> wp(cold[threadIdx.x >> 5]);
-            ok = wp.run(B, it.pair, lane, true, dt);
-            et = wp.end_t;
-            eq = wp.end_q;
-        }
-        if (!ok) {                                  // the int32 score kernel takes it
+        TracePair<C> wp(cold[threadIdx.x >> 5]);
+        wp.ck = lazy_smem + (threadIdx.x >> 5) * tbf16_warp_smem<C>();
+        int32_t n = -1;
+        if (!wp.run(B, it.pair, lane, true, states + it.dir_off)) {    // the int32 score kernel takes it
             if (lane == 0) {
                 const int32_t slot = atomicAdd(&B.counters[CTR_NOVF], 1);
                 B.ovf_list[slot] = it.pair;
-                n_cigar[it.pair] = -1;
             }
-            continue;
+        } else {
+            __syncwarp();
+            n = wp.end_t < 0 || wp.end_q < 0 ? 0      // the maximum is the origin
+                                             : tb_trace(wp, ops + it.ops_off, wp.end_t + wp.end_q + 2);
         }
-        if (et < 0 || eq < 0) {                     // the maximum is the origin
-            if (lane == 0) n_cigar[it.pair] = 0;
-            continue;
-        }
-        __syncwarp();
-        const int32_t w = effective_w(B.params.w, B.t_len[it.pair], B.q_len[it.pair]);
-        const int32_t n = tb_walk<C, true>(my_win, dt, ops + it.ops_off, et + eq + 2, et, eq, w, lane);
         if (lane == 0) n_cigar[it.pair] = n;
     }
 }
@@ -285,16 +524,19 @@ tbf16_kernel(const DevBatch *__restrict__ d_batch, const TbItem *__restrict__ it
 template <int C, int MINB>
 cudaError_t launch_tbf16_c(const DevBatch *d_batch, const TbItem *items, int32_t n_items, int32_t *head,
                            uint8_t *dir, uint32_t *ops, int32_t *n_cigar, int n_blocks, cudaStream_t s) {
-    tbf16_kernel<C, MINB><<<n_blocks, WARP_BLOCK_THREADS, 0, s>>>(d_batch, items, n_items, head, dir, ops,
-                                                                  n_cigar);
+    tbf16_kernel<C, MINB><<<n_blocks, WARP_BLOCK_THREADS, (WARP_BLOCK_THREADS / 32) * 16 * tbf16_warp_smem<C>(),
+                            s>>>(d_batch, items, n_items, head, dir, ops, n_cigar);
     return cudaGetLastError();
 }
 
 template <int C, int MINB>
 int occupancy_tbf16_c() {
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, tbf16_kernel<C, MINB>, WARP_BLOCK_THREADS, 0) !=
-        cudaSuccess)
+    constexpr int smem = (WARP_BLOCK_THREADS / 32) * 16 * tbf16_warp_smem<C>();
+    if (cudaFuncSetAttribute(tbf16_kernel<C, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
+            cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, tbf16_kernel<C, MINB>, WARP_BLOCK_THREADS, smem) !=
+            cudaSuccess)
         return 1;
     return nb > 0 ? nb : 1;
 }

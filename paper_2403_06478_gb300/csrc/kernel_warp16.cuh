@@ -125,11 +125,7 @@ struct Xchg16 {
 //   bits 4-7  Eo, Fo, E2o, F2o leaving the cell extend the cell's own gap
 //             state (strictly better than opening from H)
 // Each bit is one 16x2 minimum of an exclusive or (0 or 1 per half).
-// SCORE: the termination test and the result (the score path).  DIR with
-// SCORE is the fused traceback variant: the score path itself writes the
-// direction bytes of every anti-diagonal it computes, so the traceback needs
-// no second pass over the band; without SCORE (run_dir) the end anti-diagonal
-// is given and nothing else is tracked.
+// With DIR (run_dir) the end anti-diagonal is given and nothing else is tracked.
 // K: warps sharing one pair's band (1, 2 or 4).  Warp k of the group holds
 // slots 32kC .. 32(k+1)C - 1 of the frame; after every anti-diagonal the warps
 // exchange their edge gap states and anti-diagonal maxima through shared
@@ -138,9 +134,12 @@ struct Xchg16 {
 // the edge steps defer their arg-max search like the bulk.  (The larger
 // register budget only: the extra state does not fit the smaller one
 // without spills.)
-// LAZY: blocks of anti-diagonals without a maximum (see lazy_run).
-template <int C, bool DMREG, bool DEFER = false, bool DIR = false, bool SCORE = !DIR, int K = 1,
-          bool FHEAD = false, bool EDEFER = false, int G = 32, bool LAZY = false>
+// LAZY: blocks of anti-diagonals without a maximum (see lazy_drive).
+// TRACE (with LAZY): the score path also keeps the band's state of every 32nd
+// anti-diagonal in memory, from which the traceback recomputes its way back
+// (tb_trace in kernel_tb.cuh).
+template <int C, bool DMREG, bool DEFER = false, bool DIR = false, int K = 1,
+          bool FHEAD = false, bool EDEFER = false, int G = 32, bool LAZY = false, bool TRACE_ = false>
 struct WarpPair16 {
     static_assert(C == 4 || C == 6 || C == 8 || C == 12 || C == 16 || C == 20 || C == 24,
                   "16-bit lanes use 4, 6, 8, 12, 16, 20 or 24 slots per lane");
@@ -189,7 +188,8 @@ struct WarpPair16 {
     uint32_t DMR[DMREG ? P : 1];   // DMREG: dead_mask(p), computed once per pair
     uint32_t Hsave[DEFER ? P : 1]; // DEFER: H of the pending maximum's anti-diagonal
     uint8_t *dtab;                 // DIR: this lane's bytes of anti-diagonal 0
-    int32_t end_t, end_q;          // DIR and SCORE: where the traceback starts (-1: empty)
+    uint4 *gck;                    // TRACE: the pair's states in memory
+    int32_t end_t, end_q;          // TRACE: where the traceback starts (-1: empty)
     int32_t pend_r, pend_m, pend_lm;   // its anti-diagonal (-3: none), maximum, lane maximum
     uint32_t pend_rb;              // lane bits of its band slots (~0: every slot of the bulk)
     bool in_head;                  // FHEAD: the pair loop is running head anti-diagonals
@@ -715,10 +715,7 @@ struct WarpPair16 {
             else if (i == P - 1) lmax = __vmaxu2(lmax, mx);
             else pend = mx;
         }
-        if constexpr (DIR && !SCORE) return dir_finish<ODD, MODE>(r, lmax, rb, vb, dbits);
-        if constexpr (DIR && SCORE) {
-            if (r >= 0) store_row(r, dbits);
-        }
+        if constexpr (DIR) return dir_finish<ODD, MODE>(r, lmax, rb, vb, dbits);
         const int32_t lm = (int32_t)max(lmax & 0xffffu, lmax >> 16);
         int32_t m_grp = 0;
         if constexpr (K > 1) m_grp = exchange<!ODD, MODE != BULK>(r, lm);
@@ -804,7 +801,7 @@ struct WarpPair16 {
         }
     }
 
-    // DIR without SCORE: end of a step.  Store the row, then what the rebase
+    // DIR: end of a step.  Store the row, then what the rebase
     // needs: the anti-diagonal maximum (only when a rebase follows) and the
     // rebase.
     template <bool ODD, int MODE>
@@ -1147,10 +1144,10 @@ struct WarpPair16 {
                 // pair's registers for lazy_edges; the row's slot moved down
                 // before the first anti-diagonal, the column's moves up
                 // before the second
-                --g.dt;
+                g.dt -= g.step;
                 ring_store(g.ring, g.dt, Hev);
                 ring_store(g.ring + 2 * RING, g.dq, Hev);
-                ++g.dq;
+                g.dq += g.step;
                 ring_store(g.ring + 4 * P, g.dt, Hod);
                 ring_store(g.ring + 4 * P + 2 * RING, g.dq, Hod);
                 g.ring += 8 * P;
@@ -1242,9 +1239,46 @@ struct WarpPair16 {
             lazy_word(4 * i + 3) = v.w;
         }
     }
+    // TRACE: state k >= 1 is that after anti-diagonal first_r() + 32k, in the
+    // drifting form (rs: its start) or, from the masked step, the plain one.
+    // An entry is the checkpoint's words and one of {rs, base, drifting}.
+    static constexpr int TRACE_ENTRY = CKV * 32 + 1;     // 16-byte words
+    __device__ __forceinline__ int32_t first_r() const { return 1 + (w & 1); }
+    __device__ __forceinline__ bool trace_mark(int32_t r) const {
+        return r > first_r() && ((r - first_r()) & 31) == 0;
+    }
+    // pairs of anti-diagonals from r to the next state kept
+    __device__ __forceinline__ int32_t trace_room(int32_t r) const { return (32 - ((r - first_r()) & 31)) >> 1; }
+    __device__ __forceinline__ uint4 *trace_entry(int32_t k) const { return gck + (int64_t)(k - 1) * TRACE_ENTRY; }
+    __device__ __forceinline__ void trace_save(int32_t r, int32_t rs, bool drifting) {
+        uint4 *d = trace_entry((r - first_r()) >> 5);
+#pragma unroll
+        for (int i = 0; i < CKV; ++i)
+            d[i * 32 + lane] =
+                make_uint4(lazy_word(4 * i), lazy_word(4 * i + 1), lazy_word(4 * i + 2), lazy_word(4 * i + 3));
+        if (lane == 0) d[CKV * 32] = make_uint4((uint32_t)rs, (uint32_t)base, drifting ? 1u : 0u, 0u);
+    }
+    // Load state k; returns whether it is in the drifting form.
+    __device__ __forceinline__ bool trace_load(int32_t k, int32_t &rs) {
+        const uint4 *d = trace_entry(k);
+#pragma unroll
+        for (int i = 0; i < CKV; ++i) {
+            const uint4 v = d[i * 32 + lane];
+            lazy_word(4 * i) = v.x;
+            lazy_word(4 * i + 1) = v.y;
+            lazy_word(4 * i + 2) = v.z;
+            lazy_word(4 * i + 3) = v.w;
+        }
+        uint4 m = make_uint4(0x80000000u, 0x80000000u, 0u, 0u);
+        if (lane == 0) m = d[CKV * 32];
+        rs = __reduce_max_sync(FULL, (int32_t)m.x);
+        base = __reduce_max_sync(FULL, (int32_t)m.y);
+        return __any_sync(FULL, m.z != 0u);
+    }
+
     // What lazy_drive asks of the lanes.
     __device__ __forceinline__ static constexpr bool owns() { return true; }
-    static constexpr bool REBASES = true;
+    static constexpr bool REBASES = true, TRACE = TRACE_;
     __device__ __forceinline__ LazyConst lazy_consts(bool) const {
         LazyConst k;
         k.D = (uint32_t)prm.e2 * 0x10001u;
@@ -1385,10 +1419,9 @@ struct WarpPair16 {
 
     // ------------------------------------------------------------------ pair
     // Returns false if the pair must be recomputed with int32 lanes.
-    // DIR (fused): dt is the pair's direction table, one row per anti-diagonal
-    // up to the last one the extension can reach.
+    // TRACE: states is the memory for the pair's states.
     __device__ __forceinline__ bool run(const DevBatch &Bt, int32_t pair, int32_t lane_, bool use_fast,
-                                        uint8_t *dt = nullptr) {
+                                        uint8_t *states = nullptr) {
         prm = Bt.params;
         lane = lane_;
         tlen = Bt.t_len[pair]; qlen = Bt.q_len[pair];
@@ -1414,7 +1447,11 @@ struct WarpPair16 {
             qspan = (int32_t)min(Bt.q_words - qw0, (int64_t)((qph + qlen + 15) >> 4));
         }
         agatha_result *out = Bt.out + pair;
-        if constexpr (DIR) { end_t = -1; end_q = -1; }
+        if constexpr (TRACE) {
+            end_t = -1;
+            end_q = -1;
+            gck = reinterpret_cast<uint4 *>(states);
+        }
         if (tlen <= 0 || qlen <= 0) {
             if (leader()) write_empty_result(out);
             return true;
@@ -1435,12 +1472,8 @@ struct WarpPair16 {
         oe = prm.q + prm.e; oe2 = prm.q2 + prm.e2;
         j0 = (wk * G + lane) * C;
         last_r = tlen + qlen - 2;
-        if constexpr (DIR) dtab = dt + j0;
         {
-            int32_t Dp = step_change_max(prm);
-            // the drift of the lazy blocks and half a match per anti-diagonal
-            // stay within the step bound too
-            if constexpr (LAZY) Dp = max(Dp, (prm.a + 1) / 2 + prm.e2);
+            const int32_t Dp = LAZY ? lazy_step_max(prm) : step_change_max(prm);
             const int32_t kint = rebase_interval(Dp);
             until_rebase = kint;
             OFF = 0xffff - (kint + 3) * Dp;
@@ -1496,11 +1529,11 @@ struct WarpPair16 {
         else r = steps(-2, use_fast);
         if (ovf) return false;
         locate_pending();
-        if constexpr (DIR) {
+        if constexpr (TRACE) {
             // the traceback's start: the query end when reached, else the maximum
             const bool reach = !zdropped && cold.mqe != K_NEG_OUT && cold.mqe + prm.end_bonus > gmax;
-            end_t = reach ? cold.mqe_t : cold.gt;
-            end_q = reach ? qlen - 1 : cold.gq;
+            end_t = __reduce_max_sync(FULL, reach ? cold.mqe_t : cold.gt);
+            end_q = __reduce_max_sync(FULL, reach ? qlen - 1 : cold.gq);
         }
         group_sync();           // K > 1: every warp's last writes to cold are in
         if (leader()) {
@@ -1624,7 +1657,7 @@ warp16_align_kernel(const DevBatch *__restrict__ d_batch, int32_t use_fast, int3
     const int lane = threadIdx.x & (G - 1);
     const WorkList L = work_list(B, list);
     if constexpr (G == 32) {
-        using Pair = WarpPair16<C, false, false, false, true, 1, true, false, 32, true>;
+        using Pair = WarpPair16<C, false, false, false, 1, true, false, 32, true>;
         extern __shared__ uint4 lazy_smem[];
         const int32_t l_end = __reduce_max_sync(FULL, L.end);
         uint4 *ck = lazy_smem + (threadIdx.x >> 5) * (2 * Pair::CKV * 32 + Pair::RING / 4);
@@ -1643,7 +1676,7 @@ warp16_align_kernel(const DevBatch *__restrict__ d_batch, int32_t use_fast, int3
             }
         }
     } else {
-        using Pair = WarpPair16<C, MINB < 4, true, false, true, 1, true, true, G>;
+        using Pair = WarpPair16<C, MINB < 4, true, false, 1, true, true, G>;
         // The warp takes two neighbouring pairs of the longest-first queue at
         // once (about the same length), one per half, and both halves start
         // their next pairs together: the two then pass through the same step
@@ -1687,7 +1720,7 @@ warp16k_align_kernel(const DevBatch *__restrict__ d_batch, int32_t use_fast, int
     const int32_t bar = 1 + g;                           // named barrier of the group
     const WorkList L = work_list(B, list);
     for (;;) {
-        WarpPair16<C, (MINB < 4 && C <= 16) || MINB < 3, true, false, true, K> wp(cold[g], &xch[g], wk, bar);
+        WarpPair16<C, (MINB < 4 && C <= 16) || MINB < 3, true, false, K> wp(cold[g], &xch[g], wk, bar);
         if (wk == 0 && lane == 0) xch[g].pair = L.begin + atomicAdd(L.head, 1);
         wp.group_sync();
         const int32_t k = xch[g].pair;
@@ -1723,7 +1756,7 @@ int occupancy_warp16k_c() {
 // warp.
 template <int C, int G>
 constexpr int warp16_smem() {
-    using Pair = WarpPair16<C, false, false, false, true, 1, false, false, 32, true>;
+    using Pair = WarpPair16<C, false, false, false, 1, true, false, 32, true>;
     return G == 32 ? (WARP_BLOCK_THREADS / 32) * (2 * Pair::CKV * 32 * 16 + Pair::RING * 4) : 0;
 }
 

@@ -12,7 +12,7 @@ template int occupancy_warp16_c<4, 3>();
 template cudaError_t launch_tb16_c<4, 6>(const DevBatch *, const TbItem *, int32_t, int32_t *, uint8_t *,
                                           uint32_t *, int32_t *, int, cudaStream_t);
 template int occupancy_tb16_c<4, 6>();
-template cudaError_t launch_tbf16_c<4, 6>(const DevBatch *, const TbItem *, int32_t, int32_t *, uint8_t *,
+template cudaError_t launch_tbf16_c<4, 4>(const DevBatch *, const TbItem *, int32_t, int32_t *, uint8_t *,
                                            uint32_t *, int32_t *, int, cudaStream_t);
-template int occupancy_tbf16_c<4, 6>();
+template int occupancy_tbf16_c<4, 4>();
 }  // namespace agatha

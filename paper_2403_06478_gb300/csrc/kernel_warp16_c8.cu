@@ -15,7 +15,7 @@ template int occupancy_warp16_c<8, 3, 16>();
 template cudaError_t launch_tb16_c<8, 4>(const DevBatch *, const TbItem *, int32_t, int32_t *, uint8_t *,
                                           uint32_t *, int32_t *, int, cudaStream_t);
 template int occupancy_tb16_c<8, 4>();
-template cudaError_t launch_tbf16_c<8, 4>(const DevBatch *, const TbItem *, int32_t, int32_t *, uint8_t *,
+template cudaError_t launch_tbf16_c<8, 3>(const DevBatch *, const TbItem *, int32_t, int32_t *, uint8_t *,
                                            uint32_t *, int32_t *, int, cudaStream_t);
-template int occupancy_tbf16_c<8, 4>();
+template int occupancy_tbf16_c<8, 3>();
 }  // namespace agatha

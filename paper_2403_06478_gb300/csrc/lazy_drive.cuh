@@ -24,7 +24,8 @@ struct Cold16 {
 
 // Where the last row's and column's cells sit, as slots of this lane (on: the
 // block may hold such cells; uniform), and the ring's shared address.
-struct LazyEdge { int32_t on, dt, dq; uint32_t ring; };
+// step: 1 (0: the same lanes keep every anti-diagonal, for the traceback).
+struct LazyEdge { int32_t on, dt, dq; uint32_t ring; int32_t step; };
 
 // Pairs of anti-diagonals the next block may hold: n, 8, 4 or 2 (0: none) such
 // that no anti-diagonal of it can fire the Z-drop test.  g, m, mu: an upper
@@ -123,11 +124,16 @@ __device__ __forceinline__ int32_t lazy_drive(S &s, bool use_fast) {
             ++r;
             if (r > -2) s.advance(r);
             if (s.head_step(r)) return r;
+            bool mark = false;
+            if constexpr (S::TRACE) mark = s.trace_mark(r);
             if constexpr (S::REBASES) {
-                if (s.until_rebase <= 2 && r >= 0) {
+                if (s.until_rebase <= (mark ? 36 : 2) && r >= 0) {
                     s.lazy_rebase(s.last_max(), r);
                     if (s.ovf) return r;
                 }
+            }
+            if constexpr (S::TRACE) {
+                if (mark) s.trace_save(r, r, false);
             }
             continue;
         }
@@ -139,7 +145,7 @@ __device__ __forceinline__ int32_t lazy_drive(S &s, bool use_fast) {
         }
         s.blind = false;
         if constexpr (S::REBASES) {
-            if (s.until_rebase < 16) {
+            if (s.until_rebase < (S::TRACE ? 40 : 16)) {
                 s.lazy_rebase(open ? m0 : s.last_max(), r);
                 if (s.ovf) return r;
             }
@@ -171,6 +177,12 @@ __device__ __forceinline__ int32_t lazy_drive(S &s, bool use_fast) {
             }
             block = false;
             m0 = m1;
+            if constexpr (S::TRACE) {
+                if (s.trace_mark(r)) {
+                    if (u0 - (r - rs) < 36) break;     // a rebase first: none within 32 anti-diagonals of it
+                    s.trace_save(r, rs, true);
+                }
+            }
             const bool cross = r == turn;
             if (r + 2 > end || (cross && w + 1 > end) || (upper != NONE && m0 + prm.a * LAZY_PAIRS <= best)) {
                 exact_until = r;                       // the end, or past a peak
@@ -180,12 +192,15 @@ __device__ __forceinline__ int32_t lazy_drive(S &s, bool use_fast) {
             int32_t left = LAZY_PAIRS;
             if constexpr (S::REBASES) {
                 left = (u0 - (r - rs) - 4) >> 1;
-                if (left < 4) break;                   // a rebase is due
+                if (left < (S::TRACE ? 2 : 4)) break;  // a rebase is due
             }
             edge = cross || r + 2 > r_in;
             n = (min(edge ? end : r_in, r < turn ? min(turn, end) : end) - r) >> 1;
             if (edge && n < 2 * LAZY_PAIRS) n = min(n, max(4, (n + 1) >> 1));   // shorter towards the end
             n = cross ? 2 : min(min(n, left), edge ? S::EDGE_PAIRS : LAZY_PAIRS);
+            if constexpr (S::TRACE) {
+                if (!cross) n = min(n, s.trace_room(r));
+            }
             mu = r < w ? max(m0, -gap_cost(prm, r + 1)) : m0;
             const int32_t fit = lazy_span(prm, n, max(best, upper), m0, mu, edge ? o1 : o0, edge ? c1 : c0);
             if (fit == 0 || (cross && fit < n)) {
@@ -205,7 +220,7 @@ __device__ __forceinline__ int32_t lazy_drive(S &s, bool use_fast) {
             typename S::LazyWin W;
             s.lazy_windows(W, r);
             const int32_t B = floor_div2(r - w);
-            LazyEdge g{__reduce_max_sync(FULL, edge ? 1 : 0), tlen - 1 - B - s.j0, r - qlen + 1 - B - s.j0, ring};
+            LazyEdge g{__reduce_max_sync(FULL, edge ? 1 : 0), tlen - 1 - B - s.j0, r - qlen + 1 - B - s.j0, ring, 1};
             if (!s.owns()) g.dt = g.dq = -(1 << 20);
             if (two) s.template lazy_block<true>(n, W, k, g);
             else s.template lazy_block<false>(n, W, k, g);

@@ -85,8 +85,8 @@ cudaError_t launch_tb16(int C, const DevBatch *d, const TbItem *items, int32_t n
 cudaError_t launch_tbf16(int C, const DevBatch *d, const TbItem *items, int32_t n, int32_t *head,
                          uint8_t *dir, uint32_t *ops, int32_t *ncig, int blocks, cudaStream_t s) {
     switch (C) {
-        case 4: return launch_tbf16_c<4, 6>(d, items, n, head, dir, ops, ncig, blocks, s);
-        case 8: return launch_tbf16_c<8, 4>(d, items, n, head, dir, ops, ncig, blocks, s);
+        case 4: return launch_tbf16_c<4, 4>(d, items, n, head, dir, ops, ncig, blocks, s);
+        case 8: return launch_tbf16_c<8, 3>(d, items, n, head, dir, ops, ncig, blocks, s);
         case 16: return launch_tbf16_c<16, 3>(d, items, n, head, dir, ops, ncig, blocks, s);
         default: return launch_tbf16_c<24, 2>(d, items, n, head, dir, ops, ncig, blocks, s);
     }
@@ -94,8 +94,8 @@ cudaError_t launch_tbf16(int C, const DevBatch *d, const TbItem *items, int32_t 
 
 int tbf16_occupancy(int C) {
     switch (C) {
-        case 4: return occupancy_tbf16_c<4, 6>();
-        case 8: return occupancy_tbf16_c<8, 4>();
+        case 4: return occupancy_tbf16_c<4, 4>();
+        case 8: return occupancy_tbf16_c<8, 3>();
         case 16: return occupancy_tbf16_c<16, 3>();
         default: return occupancy_tbf16_c<24, 2>();
     }
@@ -183,7 +183,8 @@ extern "C" int agatha_align_cigar(agatha_ctx *ctx, const agatha_batch *batch, co
     const int C32 = pick_slots_per_lane(std::max<int32_t>(shape.max_w_all, 1));
     const int C16 = pick_slots16(std::max<int32_t>(shape.max_w_all, 1));
     const bool use16 = C16 > 0 && step_change_max(p) <= STEP16_MAX && !(flags & AGATHA_FORCE32);
-    const bool fused = use16 && lp.lane16 && !lp.wide_w && !(flags & (AGATHA_PLAIN | AGATHA_TB_TWO_PASS));
+    const bool fused = use16 && lp.lane16 && !lp.wide_w && !(flags & (AGATHA_PLAIN | AGATHA_TB_TWO_PASS)) &&
+                       lazy_step_max(p) <= TRACE_STEP_MAX;
     Slot *sl = &ctx->main;
     if (fused) {
         if ((rc = stage_batch(ctx, batch, p, out, flags, s, lp))) return rc;

@@ -107,3 +107,40 @@ def test_int32_large_scores(ctx, w):
     got = A.agatha_align_batch(ctx, batch)
     bad = A.results_equal(got, ref, O.COMPARE_FIELDS)
     assert bad.size == 0, f"pairs {bad[:5]}"
+
+
+def _gap_pairs(w, scoring, seed, n=48):
+    """Pairs whose paths hold gaps of up to several segments of the
+    traceback's recomputation, in either sequence, and leading gaps."""
+    rng = np.random.default_rng(seed)
+    qs, ts = [], []
+    for i in range(n):
+        x = rng.integers(0, 4, int(rng.integers(60, 900)), dtype=np.uint8)
+        y, _ = W._mutate_chunk(rng, x, np.array([len(x)], np.int32), W.ErrorModel(0.03, 0.02, 0.02))
+        for _ in range(2):
+            k = int(rng.integers(1, max(2, min(200, w))))
+            at = int(rng.integers(0, max(1, len(y) - k))) if i % 4 else 0
+            y = np.concatenate([y[:at], y[at + k:]])
+        if not len(y):
+            y = x[:1]
+        if i % 3 == 0:                          # repeats: ties between gap places
+            y = np.concatenate([y, np.tile(x[:7], 9)])
+        qs.append(x if i % 2 else y)
+        ts.append(y if i % 2 else x)
+    return W.from_pairs(qs, ts, scoring)
+
+
+@pytest.mark.parametrize("w", [5, 8, 33, 100, 127, 128, 200, 255, 500, 511, 630, 750, 767])
+@pytest.mark.parametrize("name", sorted(SCORINGS))
+def test_cigars(ctx, name, w):
+    from oracle import oracle as O
+    for make, seed in ((_gap_pairs, 31), (_pairs, 32)):
+        batch = make(w, W.replace(SCORINGS[name], w=w), seed + w, n=40)
+        ref = O.align_batch(batch)
+        want, _ = O.traceback_batch(batch, ref)
+        res, off, cig = ctx.align_cigar(A.pack_batch(batch), batch.scoring)
+        bad = A.results_equal(res, ref, O.COMPARE_FIELDS)
+        assert bad.size == 0, f"results of pairs {bad[:5]}"
+        for i in range(batch.n_pairs):
+            got = cig[off[i]:off[i + 1]]
+            assert np.array_equal(got, want[i]), (i, A.cigar_string(got), A.cigar_string(want[i]))
