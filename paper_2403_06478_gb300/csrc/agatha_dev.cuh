@@ -348,8 +348,7 @@ cudaError_t launch_cigar_gather(const TbItem *items, int32_t n_items, const int3
 cudaError_t launch_plain_kernel(const DevBatch *d_batch, int64_t n_blocks, int32_t w_max,
                                 int use_wide_list, cudaStream_t s);
 // The local extension (kernel_local.cu), C slots per lane of int32 lanes.
-cudaError_t launch_local(int C, const DevBatch *d_batch, int n_blocks, cudaStream_t s);
-int local_occupancy(int C);
+cudaError_t launch_local(int C, const DevBatch *d_batch, int n_sm, cudaStream_t s);
 int plain_kernel_max_w();
 cudaError_t plain_kernel_prepare();
 

@@ -78,7 +78,7 @@ extern "C" int agatha_align_batch_local(agatha_ctx *ctx, const agatha_batch *bat
         (e = launch_prep(d, n, lp.sort, s, ctx->n_sm)) != cudaSuccess)
         return cuda_fail(ctx, e, "prep");
     if (ctx->timing && (e = cudaEventRecord(ctx->ev_k0, s)) != cudaSuccess) return cuda_fail(ctx, e, "event");
-    if ((e = launch_local(lp.C, d, ctx->n_sm * local_occupancy(lp.C), s)) != cudaSuccess)
+    if ((e = launch_local(lp.C, d, ctx->n_sm, s)) != cudaSuccess)
         return cuda_fail(ctx, e, "launch local");
     if (ctx->timing && (e = cudaEventRecord(ctx->ev_k1, s)) != cudaSuccess) return cuda_fail(ctx, e, "event");
     if ((e = cudaMemcpyAsync(sl->h_counters, sl->counters.ptr, CTR_COUNT * sizeof(int32_t),

@@ -144,3 +144,21 @@ def test_cigars(ctx, name, w):
         for i in range(batch.n_pairs):
             got = cig[off[i]:off[i + 1]]
             assert np.array_equal(got, want[i]), (i, A.cigar_string(got), A.cigar_string(want[i]))
+
+
+@pytest.mark.parametrize("w", [4, 5, 8, 13, 33, 100, 101, 102, 126, 127, 128, 200, 255, 256, 300, 500, 510, 511])
+@pytest.mark.parametrize("name", ["one", "two", "second_cheaper", "dear_extension", "no_zdrop", "free_mismatch"])
+def test_local(ctx, name, w):
+    """The local extension's row blocks: initial scores that die before, at and
+    after the band's corner (the last take the per-cell step), rows that end
+    with the band and with the table, and scores too large for the row keys."""
+    from oracle import oracle as O
+    rng = np.random.default_rng(900 + w)
+    for make in (_pairs, _gap_pairs):
+        batch = make(w, W.replace(SCORINGS[name], w=w), 77 + w, n=60)
+        edge = [1, 2, 7, 20, 40, 60, w, w + 7, 2 * w + 9, 1000, (1 << 20) - 3, 1 << 24]
+        h0 = rng.choice(edge, batch.n_pairs).astype(np.int32)
+        ref = O.align_batch(batch, h0=h0)
+        got = ctx.align_local(A.pack_batch(batch), batch.scoring, h0)
+        bad = A.results_equal(got, ref, O.COMPARE_FIELDS)
+        assert bad.size == 0, (bad[:5], h0[bad[:5]], got[bad[:2]], ref[bad[:2]])
