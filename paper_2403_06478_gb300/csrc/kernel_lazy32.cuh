@@ -39,6 +39,7 @@ struct LazyPair32 {
     static constexpr bool REBASES = false, TRACE = false;
     static constexpr int TW = C <= 16 ? 2 : 3;            // window words: C bases and 16 to come
     static constexpr int V = C / 4;                       // 16-byte words of a lane's array
+    static constexpr int BLOCK_PAIRS = C <= 4 ? 16 : 32;  // most pairs of a block (see WarpPair16)
     static constexpr int EDGE_PAIRS = 8;                  // pairs of a block with the last row or column
     static constexpr int RING = 2 * 2 * EDGE_PAIRS * C;   // words of the edge ring (row | column)
     static constexpr int CKV = 6 * V;                     // 16-byte words of a checkpoint per lane
@@ -54,7 +55,6 @@ struct LazyPair32 {
     // H(r) overwrites H(r-2) in the array of its parity; gap states leaving the
     // last anti-diagonal (on lazy blocks: see lazy_step)
     int32_t Hev[C], Hod[C], Eo[C], Fo[C], E2o[C], F2o[C];
-    LazyWin Wx;                   // windows of the last masked anti-diagonal
     int32_t gmax, zdropped, lastm, until_rebase;
     bool cover, blind;
     Cold16 &cold;
@@ -112,8 +112,6 @@ struct LazyPair32 {
             W.q[i] = rev2_32(load_rel(qp, qspan, qb - 16 * i));
         }
     }
-    __device__ __forceinline__ void init_windows(int32_t r) { lazy_windows(Wx, r); }
-    __device__ __forceinline__ void advance(int32_t r) { lazy_windows(Wx, r); }
     // bit 2 (p mod 16) of word p / 16: slot p's bases differ
     __device__ __forceinline__ static uint2 mismatch(const LazyWin &W) {
         const uint32_t x0 = W.t[0] ^ W.q[1];
@@ -139,9 +137,10 @@ struct LazyPair32 {
     // table keeps its value, a virtual row or column cell (in the head) gets
     // its own, anything else is minus infinity.  Then the last row and column,
     // the maximum and the termination test (Eq. 4-7).
-    template <bool ODD>
+    // (One copy for both parities: it runs on few anti-diagonals, and the
+    // instruction cache is what the pair's other steps need.)
     __device__ __forceinline__ bool masked_step(int32_t r) {
-        int32_t (&Hd)[C] = ODD ? Hod : Hev;
+        const bool odd = ((r - w) & 1) != 0;
         const int32_t B = floor_div2(r - w);
         int32_t st = 0, en = -1;
         if constexpr (K > 1) {
@@ -160,44 +159,49 @@ struct LazyPair32 {
             if (r >= -1 && r + 1 < tlen) v2 = r + 1 - B - j0;  // (r + 1, -1)
         }
         const int32_t vv = r == -2 ? 0 : -gap_cost(prm, r + 2);
-        int32_t edge, edge2;
-        if constexpr (ODD) {
-            edge = __shfl_up_sync(FULL, Eo[C - 1], 1);
-            edge2 = __shfl_up_sync(FULL, E2o[C - 1], 1);
-            if (lane == 0 && wk == 0) edge = edge2 = K_NEG;
-        } else {
-            edge = __shfl_down_sync(FULL, Fo[0], 1);
-            edge2 = __shfl_down_sync(FULL, F2o[0], 1);
-            if (lane == 31 && wk == K - 1) {
-                // slot NS of r - 1: the virtual column cell (t, -1) when q == -1 there
-                edge = edge2 = K_NEG;
-                const int32_t ts = floor_div2(r - 1 - w) + NS, qs = r - 1 - ts;
-                if (qs == -1 && ts >= 0 && ts < tlen && r <= w + 1) {
-                    const int32_t v = -gap_cost(prm, ts + 1);
-                    edge = v - oe;
-                    edge2 = v - oe2;
-                }
+        int32_t eL = __shfl_up_sync(FULL, Eo[C - 1], 1), e2L = __shfl_up_sync(FULL, E2o[C - 1], 1);
+        int32_t fR = __shfl_down_sync(FULL, Fo[0], 1), f2R = __shfl_down_sync(FULL, F2o[0], 1);
+        if (lane == 0 && wk == 0) eL = e2L = K_NEG;
+        if (lane == 31 && wk == K - 1) {
+            // slot NS of r - 1: the virtual column cell (t, -1) when q == -1 there
+            fR = f2R = K_NEG;
+            const int32_t ts = floor_div2(r - 1 - w) + NS, qs = r - 1 - ts;
+            if (qs == -1 && ts >= 0 && ts < tlen && r <= w + 1) {
+                const int32_t v = -gap_cost(prm, ts + 1);
+                fR = v - oe;
+                f2R = v - oe2;
             }
         }
+        LazyWin Wx;
+        lazy_windows(Wx, r);
         const uint2 nm = mismatch(Wx);
         int32_t lm = INT_MIN;
+        int32_t nE[C], nE2[C], nF[C], nF2[C], Hd[C];
 #pragma unroll
-        for (int i = 0; i < C; ++i) {
-            const int p = ODD ? C - 1 - i : i;
-            const int32_t Ein = ODD ? (p ? Eo[p - 1] : edge) : Eo[p];
-            const int32_t E2in = ODD ? (p ? E2o[p - 1] : edge2) : E2o[p];
-            const int32_t Fin = ODD ? Fo[p] : (p < C - 1 ? Fo[p + 1] : edge);
-            const int32_t F2in = ODD ? F2o[p] : (p < C - 1 ? F2o[p + 1] : edge2);
+        for (int p = 0; p < C; ++p) {
+            const int32_t Ein = odd ? (p ? Eo[p - 1] : eL) : Eo[p];
+            const int32_t E2in = odd ? (p ? E2o[p - 1] : e2L) : E2o[p];
+            const int32_t Fin = odd ? Fo[p] : (p < C - 1 ? Fo[p + 1] : fR);
+            const int32_t F2in = odd ? F2o[p] : (p < C - 1 ? F2o[p + 1] : f2R);
             const int32_t s = mismatch_of(nm, p) ? -prm.b : prm.a;
-            const int32_t H = max(max(Hd[p] + s, Ein), max(max(Fin, E2in), F2in));
+            const int32_t H = max(max((odd ? Hod[p] : Hev[p]) + s, Ein), max(max(Fin, E2in), F2in));
             const bool real = p >= lo && p <= hi;
             const int32_t Hm = real ? H : (p == v1 || p == v2 ? vv : K_NEG);
-            Eo[p] = max(Ein - prm.e, Hm - oe);
-            Fo[p] = max(Fin - prm.e, Hm - oe);
-            E2o[p] = max(E2in - prm.e2, Hm - oe2);
-            F2o[p] = max(F2in - prm.e2, Hm - oe2);
+            nE[p] = max(Ein - prm.e, Hm - oe);
+            nF[p] = max(Fin - prm.e, Hm - oe);
+            nE2[p] = max(E2in - prm.e2, Hm - oe2);
+            nF2[p] = max(F2in - prm.e2, Hm - oe2);
             Hd[p] = Hm;
             lm = real ? max(lm, Hm) : lm;
+        }
+#pragma unroll
+        for (int p = 0; p < C; ++p) {
+            Eo[p] = nE[p];
+            Fo[p] = nF[p];
+            E2o[p] = nE2[p];
+            F2o[p] = nF2[p];
+            Hod[p] = odd ? Hd[p] : Hod[p];
+            Hev[p] = odd ? Hev[p] : Hd[p];
         }
         if (r < 0) return false;
         // the lane that owns the last row's (column's) cell looks at it
@@ -252,9 +256,6 @@ struct LazyPair32 {
         }
         if (set_gs) cold.gscore = gs;
         return false;
-    }
-    __device__ __forceinline__ bool head_step(int32_t r) {
-        return ((r - w) & 1) ? masked_step<true>(r) : masked_step<false>(r);
     }
 
     // --------------------------------------------------------- lazy blocks
@@ -443,6 +444,49 @@ struct LazyPair32 {
         x[4 * i + 2] = v.z;
         x[4 * i + 3] = v.w;
     }
+    // The cell of the maximum m (drifting form of r) of the pair r - 1, r whose
+    // state checkpoint buf holds: the first anti-diagonal's first.
+    __device__ __forceinline__ void lazy_locate(const LazyConst &k, int buf, int32_t r, int32_t m) {
+        const int4 *d = ck + buf * (CKV * 32);
+        int32_t t[2];
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const int32_t rr = r - 1 + c, B = floor_div2(rr - w);
+            const int32_t lo = max(max(0, rr - qlen + 1), ceil_div2(rr - w)) - B - j0;
+            const int32_t hi = min(min(tlen - 1, rr), floor_div2(rr + w)) - B - j0;
+            int32_t at = INT_MAX;
+#pragma unroll
+            for (int i = V - 1; i >= 0; --i) {
+                const int4 v = d[(c * V + i) * 32];
+                const int32_t h[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int x = 3; x >= 0; --x) {
+                    const int p = 4 * i + x;
+                    if (p >= lo && p <= hi && h[x] + (c ? 0 : k.D) == m) at = B + j0 + p;
+                }
+            }
+            t[c] = __reduce_min_sync(FULL, owns() ? at : INT_MAX);
+        }
+        if constexpr (K > 1) {
+            int32_t *x = xch + HALO;                  // 2 K words: both halves of the maxima
+            __syncthreads();
+            if (lane == 0) { x[2 * wk] = t[0]; x[2 * wk + 1] = t[1]; }
+            __syncthreads();
+#pragma unroll
+            for (int i = 0; i < K; ++i) {
+                t[0] = min(t[0], x[2 * i]);
+                t[1] = min(t[1], x[2 * i + 1]);
+            }
+            __syncthreads();
+        }
+        if (leader()) {
+            const bool first = t[0] != INT_MAX;
+            cold.gt = first ? t[0] : t[1];
+            cold.gq = (first ? r - 1 : r) - cold.gt;
+        }
+        __syncwarp();
+        group_sync();
+    }
     // A lane's state as 16-byte words, at d[0], d[stride] ...
     __device__ __forceinline__ void put(int4 *d, int stride) const {
 #pragma unroll
@@ -527,7 +571,6 @@ struct LazyPair32 {
         }
         __syncwarp();
         group_sync();
-        init_windows(-2);
         const int32_t r = lazy_drive(*this, use_fast);
         __syncwarp();
         group_sync();                 // every warp's last writes to cold are in

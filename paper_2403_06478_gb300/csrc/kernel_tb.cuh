@@ -353,13 +353,10 @@ __device__ __forceinline__ void trace_segment(S &s, TraceWin<S> &W, int32_t seg,
         } else {
             if (drifting) {
                 s.lazy_leave(k, two, r - rs);
-                s.init_windows(r);
                 drifting = false;
             }
             ++r;
-            if (r == -2) s.init_windows(r);
-            else s.advance(r);
-            s.head_step(r);
+            s.masked_step(r);
             W.keep(s, r, ((r - w) & 1) ? s.Hod : s.Hev, s.base - s.OFF);
         }
     }
@@ -375,7 +372,7 @@ __device__ __forceinline__ int32_t tb_trace(S &s, uint32_t *ops, int32_t cap) {
     const DevParams &prm = s.prm;
     const int32_t w = s.w, g0 = s.first_r(), lane = s.lane;
     const bool two = prm.q2 != prm.q || prm.e2 != prm.e;
-    const bool head = w >= 8 && s.lazy_head_ok();
+    const bool head = __any_sync(FULL, w >= 8 && s.lazy_head_ok());
     const int32_t L = min(s.tlen, s.qlen);
     const int32_t end = abs(s.tlen - s.qlen) <= w ? s.last_r - 1 : max(L - 2, 2 * L - 3 - w);
     const auto k = s.lazy_consts(two);

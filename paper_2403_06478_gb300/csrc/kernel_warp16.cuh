@@ -518,8 +518,7 @@ struct WarpPair16 {
                 group_sync();
                 tstar = xch->t[r & 1];
             }
-            const bool drop = max_and_zdrop(mt, tstar, r);
-            if (LAZY ? __any_sync(FULL, drop) : drop) { zdropped = 1; return true; }
+            if (max_and_zdrop(mt, tstar, r)) { zdropped = 1; return true; }
         }
         return false;
     }
@@ -596,12 +595,8 @@ struct WarpPair16 {
             rb = range_bits(st - B - j0, en - B - j0);
         }
         if constexpr (MODE == HEAD) {
-            // (LAZY runs it past the head as well, where no virtual cell is in
-            // the band)
-            if (!LAZY || r <= w + 1) {
-                if (r + 1 < qlen) vb |= slot_bit(-1 - B - j0);                 // (-1, r+1)
-                if (r >= -1 && r + 1 < tlen) vb |= slot_bit(r + 1 - B - j0);  // (r+1, -1)
-            }
+            if (r + 1 < qlen) vb |= slot_bit(-1 - B - j0);                 // (-1, r+1)
+            if (r >= -1 && r + 1 < tlen) vb |= slot_bit(r + 1 - B - j0);  // (r+1, -1)
             const int32_t vv = to_u(r == -2 ? 0 : -gap_cost(prm, r + 2));
             if (__any_sync(gmask(), vb != 0u) && (vv < cold.LOWCHK || vv > 0xffff - cold.Dp)) ovf = true;
             VVp = (uint32_t)vv * 0x10001u;
@@ -624,7 +619,7 @@ struct WarpPair16 {
             uint32_t f2R = __shfl_down_sync(gmask(), F2o[0], 1, G);
             if (K > 1 && wk < K - 1 && lane == 31) { fR = xe0; f2R = xe1; }
             uint32_t inj = NEGp, inj2 = NEGp;
-            if (MODE == HEAD && lane == G - 1 && (K == 1 || wk == K - 1) && (!LAZY || r <= w + 1)) {
+            if (MODE == HEAD && lane == G - 1 && (K == 1 || wk == K - 1)) {
                 // beyond the last lane: slot NS of r-1, the virtual column
                 // cell (t, -1) when q == -1 there
                 const int32_t ts = frame(r - 1) + NS, qs = r - 1 - ts;
@@ -749,16 +744,9 @@ struct WarpPair16 {
                 }
             }
             __syncwarp(gmask());
-            if constexpr (LAZY) {
-                if (blind) { --until_rebase; return false; }
-            }
             if (anti_diagonal_max<ODD>(r, B, lm, m_grp, Hd, [&](int p) { return ~half_mask_rt(rb, p); }, rb))
                 return true;
             if (set_gs && lane == 0) cold.gscore = gs;
-            if constexpr (LAZY) {
-                --until_rebase;
-                return false;
-            }
             if (--until_rebase <= 2) {
                 // slots off the table (past its end, or holding NEG) are
                 // reset; the virtual cells' values are kept
@@ -1005,6 +993,12 @@ struct WarpPair16 {
     // Minus infinity stays at U_NEG under the drift; every score is then at
     // least U_NEG, because the drifting gap state never falls.
     static constexpr int CKV = 6 * P / 4;                // 16-byte words of a checkpoint per lane
+    // Most pairs of a block: what a block costs besides its steps (its maximum,
+    // bounds and checkpoint, about 250 instructions) against what is taken again
+    // at a pair's end and the instruction cache.  On 4 slots per lane, whose
+    // pairs are short, 16 (200,000 reads of 150 bp 4.5 ms, with 32 4.7); on
+    // more 32 (20,000 ONT-like pairs 37.2 ms, with 16 38.5).
+    static constexpr int BLOCK_PAIRS = C <= 4 ? 16 : 32;
     static constexpr int EDGE_PAIRS = LAZY_PAIRS;        // pairs of a block with the last row or column
     static constexpr int RING = 2 * 2 * EDGE_PAIRS * P;  // words of the edge ring (row | column)
     static constexpr int TW = C <= 16 ? 2 : 3;           // window words: C bases and 16 to come
@@ -1026,7 +1020,7 @@ struct WarpPair16 {
         }
     }
     template <bool ODD>
-    __device__ __forceinline__ Comb lazy_mismatch(LazyWin &W) const {
+    __device__ __forceinline__ static void lazy_slide(LazyWin &W) {
         if constexpr (!ODD) {
 #pragma unroll
             for (int i = 0; i + 1 < TW; ++i) W.t[i] = __funnelshift_r(W.t[i], W.t[i + 1], 2);
@@ -1036,6 +1030,8 @@ struct WarpPair16 {
             for (int i = TW - 1; i > 0; --i) W.q[i] = __funnelshift_l(W.q[i - 1], W.q[i], 2);
             W.q[0] <<= 2;
         }
+    }
+    __device__ __forceinline__ static Comb window_mismatch(const LazyWin &W) {
         constexpr uint32_t M0 = C >= 16 ? 0x55555555u : (C == 8 ? 0x5555u : 0x55u);
         const uint32_t x0 = W.t[0] ^ W.q[1];
         const uint32_t n0 = (x0 | (x0 >> 1)) & M0;
@@ -1075,7 +1071,8 @@ struct WarpPair16 {
     __device__ __forceinline__ void lazy_step(LazyWin &W, const LazyConst &k) {
         uint32_t (&Hd)[P] = ODD ? Hod : Hev;
         const uint32_t (&Hx)[P] = ODD ? Hev : Hod;
-        const Comb comb = lazy_mismatch<ODD>(W);
+        lazy_slide<ODD>(W);
+        const Comb comb = window_mismatch(W);
         uint32_t edge, edge2 = 0;
         if constexpr (ODD) {
             edge = prmt(__shfl_up_sync(FULL, Eo[P - 1], 1), Eo[P - 1], 0x5432);
@@ -1164,6 +1161,116 @@ struct WarpPair16 {
         }
     }
 
+    // One anti-diagonal with every case handled by masks, as HEAD and TAIL in
+    // one (see step): a band cell of the table keeps its value, a virtual row or
+    // column cell (in the head) gets its own, anything else is minus infinity;
+    // then the last row and column, the maximum and the termination test.
+    // (One copy for both parities: it runs on few anti-diagonals, and the
+    // instruction cache is what the pair's other steps need.)
+    __device__ __forceinline__ bool masked_step(int32_t r) {
+        const bool odd = ((r - w) & 1) != 0;
+        const int32_t B = frame(r);
+        int32_t st = 0, en = -1;
+        if (r >= 0) {
+            st = max(max(0, r - qlen + 1), ceil_div2(r - w));
+            en = min(min(tlen - 1, r), floor_div2(r + w));
+            if (st > en) { zdropped = 1; return true; }    // the band left the table
+        }
+        const uint32_t rb = range_bits(st - B - j0, en - B - j0);
+        uint32_t vb = 0;
+        if (r <= w + 1) {
+            if (r + 1 < qlen) vb |= slot_bit(-1 - B - j0);                 // (-1, r+1)
+            if (r >= -1 && r + 1 < tlen) vb |= slot_bit(r + 1 - B - j0);  // (r+1, -1)
+        }
+        const int32_t vv = to_u(r == -2 ? 0 : -gap_cost(prm, r + 2));
+        if (vb != 0u && (vv < cold.LOWCHK || vv > 0xffff - cold.Dp)) ovf = true;
+        const uint32_t VVp = (uint32_t)vv * 0x10001u;
+        // the edge words (see step)
+        uint32_t inj = NEGp, inj2 = NEGp;
+        if (lane == 31) {
+            const int32_t ts = frame(r - 1) + NS, qs = r - 1 - ts;
+            if (qs == -1 && ts >= 0 && ts < tlen && r <= w + 1) {
+                const int32_t v = to_u(-gap_cost(prm, ts + 1));
+                if (v < cold.LOWCHK || v > 0xffff - cold.Dp) ovf = true;
+                inj = ((uint32_t)(v - oe) << 16) | (NEGp & 0xffffu);
+                inj2 = ((uint32_t)(v - oe2) << 16) | (NEGp & 0xffffu);
+            }
+        }
+        const uint32_t eL = mux(L0LO, NEGp, prmt(__shfl_up_sync(FULL, Eo[P - 1], 1), Eo[P - 1], 0x5432));
+        const uint32_t e2L = mux(L0LO, NEGp, prmt(__shfl_up_sync(FULL, E2o[P - 1], 1), E2o[P - 1], 0x5432));
+        const uint32_t fR = mux(L31HI, inj, prmt(Fo[0], __shfl_down_sync(FULL, Fo[0], 1), 0x5432));
+        const uint32_t f2R = mux(L31HI, inj2, prmt(F2o[0], __shfl_down_sync(FULL, F2o[0], 1), 0x5432));
+        LazyWin W;
+        lazy_windows(W, r);
+        const Comb comb = window_mismatch(W);
+        uint32_t lmax = 0, Hn[P], nE[P], nE2[P], nF[P], nF2[P];
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+            const uint32_t Ein = odd ? (p ? Eo[p - 1] : eL) : Eo[p];
+            const uint32_t E2in = odd ? (p ? E2o[p - 1] : e2L) : E2o[p];
+            const uint32_t Fin = odd ? Fo[p] : (p < P - 1 ? Fo[p + 1] : fR);
+            const uint32_t F2in = odd ? F2o[p] : (p < P - 1 ? F2o[p + 1] : f2R);
+            const uint32_t mword = (C <= 16 || p < 8) ? comb.lo : comb.hi;
+            const uint32_t mb = (mword >> (2 * (p & 7))) & 0x10001u;
+            const uint32_t Hs = mb * NABs + (odd ? Hod[p] : Hev[p]);
+            const uint32_t H = __vmaxu2(__vimax3_u16x2(__viaddmax_u16x2(Hs, A2, Ein), Fin, E2in), F2in);
+            const uint32_t rm = half_mask_rt(rb, p), vm = half_mask_rt(vb, p);
+            const uint32_t Hm = mux(rm, H, mux(vm, VVp, NEGp));
+            const uint32_t hoe = Hm - OEp, hoe2 = hoe - DOEp;
+            nE[p] = __viaddmax_u16x2(Ein, NEp, hoe);
+            nF[p] = __viaddmax_u16x2(Fin, NEp, hoe);
+            nE2[p] = __viaddmax_u16x2(E2in, NE2p, hoe2);
+            nF2[p] = __viaddmax_u16x2(F2in, NE2p, hoe2);
+            Hn[p] = Hm;
+            lmax = __vmaxu2(lmax, rm & hoe);
+        }
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+            Eo[p] = nE[p];
+            Fo[p] = nF[p];
+            E2o[p] = nE2[p];
+            F2o[p] = nF2[p];
+            Hod[p] = odd ? Hn[p] : Hod[p];
+            Hev[p] = odd ? Hev[p] : Hn[p];
+        }
+        if (__any_sync(FULL, ovf)) { ovf = true; return true; }
+        if (r < 0) return false;
+        --until_rebase;
+        // the lane that owns the last row's (column's) cell looks at it
+        bool set_gs = false;
+        int32_t gs = K_NEG_OUT;
+        const int32_t jt = tlen - 1 - B - j0, jq = r - qlen + 1 - B - j0;
+        if (st <= tlen - 1 && tlen - 1 <= en && (uint32_t)jt < (uint32_t)C) {
+            const int32_t v = to_true(half_of(reg_select(Hn, jt % P), jt));
+            if (v > cold.mte) { cold.mte = v; cold.mte_q = r - (tlen - 1); }
+            if (r == last_r) { gs = v; set_gs = true; }    // kept unless Z-drop stops r
+        }
+        if (st <= r - qlen + 1 && r - qlen + 1 <= en && (uint32_t)jq < (uint32_t)C) {
+            const int32_t v = to_true(half_of(reg_select(Hn, jq % P), jq));
+            if (v > cold.mqe) { cold.mqe = v; cold.mqe_t = r - (qlen - 1); }
+        }
+        __syncwarp();
+        if (blind) return false;
+        const int32_t lm = (int32_t)max(lmax & 0xffffu, lmax >> 16);
+        const int32_t m = __reduce_max_sync(FULL, lm), mt = to_true(m + oe);
+        last_m = m + oe;
+        if (mt > gmax || (prm.zdrop >= 0 && gmax - mt > prm.zdrop)) {
+            // its lowest slot
+            const uint32_t m2 = (uint32_t)(m + oe) * 0x10001u;
+            uint32_t ne = 0;
+#pragma unroll
+            for (int p = 0; p < P; ++p) ne += __vminu2((Hn[p] ^ m2) | ~half_mask_rt(rb, p), 0x10001u) << p;
+            const uint32_t eq = ~ne & ((((1u << P) - 1) << 16) | ((1u << P) - 1));
+            const uint32_t lo_eq = eq & 0xffffu, hi_eq = eq >> 16;
+            const int32_t jl = lo_eq ? __ffs(lo_eq) - 1 : P + __ffs(hi_eq) - 1;
+            const int32_t tstar =
+                __shfl_sync(FULL, B + j0 + jl, __ffs(__ballot_sync(FULL, lm == m)) - 1);
+            if (__any_sync(FULL, max_and_zdrop(mt, tstar, r))) { zdropped = 1; return true; }
+        }
+        if (set_gs) cold.gscore = gs;
+        return false;
+    }
+
     // Into the drifting form after anti-diagonal r ((r - w) odd), and back.
     __device__ __forceinline__ void lazy_enter(const LazyConst &k, bool) {
 #pragma unroll
@@ -1209,6 +1316,35 @@ struct WarpPair16 {
                 lmax = __vimax3_u16x2(lmax, half_mask_rt(b1, p) & Hod[p], half_mask_rt(b0, p) & (Hev[p] + k.D));
         }
         return __reduce_max_sync(FULL, (int32_t)max(lmax & 0xffffu, lmax >> 16));
+    }
+    // The cell of the maximum m (drifting form of r) of the pair r - 1, r whose
+    // state checkpoint buf holds: the first anti-diagonal's first.
+    __device__ __forceinline__ void lazy_locate(const LazyConst &k, int buf, int32_t r, int32_t m) {
+        const uint32_t m2 = (uint32_t)m * 0x10001u;
+        const uint32_t *d = reinterpret_cast<const uint32_t *>(ck + lane + buf * (CKV * 32));
+        int32_t j[2];
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const uint32_t bits = table_bits(r - 1 + c), add = c ? 0u : k.D;
+            uint32_t ne = 0;
+#pragma unroll
+            for (int p = 0; p < P; ++p) {
+                const int i = c * P + p;
+                const uint32_t h = d[(i / 4) * 128 + i % 4] + add;
+                ne += __vminu2((h ^ m2) | ~half_mask_rt(bits, p), 0x10001u) << p;
+            }
+            const uint32_t eq = ~ne & ((((1u << P) - 1) << 16) | ((1u << P) - 1));
+            const uint32_t lo = eq & 0xffffu, hi = eq >> 16;
+            j[c] = lo ? __ffs(lo) - 1 : (hi ? P + __ffs(hi) - 1 : -1);
+        }
+        const uint32_t b0 = __ballot_sync(FULL, j[0] >= 0), b1 = __ballot_sync(FULL, j[1] >= 0);
+        const int32_t at = b0 ? r - 1 : r;
+        const int32_t src = __ffs(b0 ? b0 : b1) - 1;
+        if (lane == src) {
+            cold.gt = frame(at) + j0 + (b0 ? j[0] : j[1]);
+            cold.gq = at - cold.gt;
+        }
+        __syncwarp();
     }
     // Checkpoints: the packed registers of the drifting form.
     __device__ __forceinline__ uint32_t &lazy_word(int i) {
@@ -1523,10 +1659,13 @@ struct WarpPair16 {
         group_sync();
         zdropped = 0;
 
-        init_windows(-2);
         int32_t r;
-        if constexpr (LAZY) r = lazy_drive(*this, use_fast);
-        else r = steps(-2, use_fast);
+        if constexpr (LAZY) {
+            r = lazy_drive(*this, use_fast);
+        } else {
+            init_windows(-2);
+            r = steps(-2, use_fast);
+        }
         if (ovf) return false;
         locate_pending();
         if constexpr (TRACE) {

@@ -4,15 +4,15 @@
 #include "kernel_tb.cuh"
 
 namespace agatha {
-template cudaError_t launch_warp16_c<16, 3>(const DevBatch *, int, cudaStream_t, int, int);
-template int occupancy_warp16_c<16, 3>();
 template cudaError_t launch_warp16_c<16, 2>(const DevBatch *, int, cudaStream_t, int, int);
 template int occupancy_warp16_c<16, 2>();
+template cudaError_t launch_warp16_c<16, 3>(const DevBatch *, int, cudaStream_t, int, int);
+template int occupancy_warp16_c<16, 3>();
 // the traceback variants (two-pass and fused) at one budget (no spills)
 template cudaError_t launch_tb16_c<16, 3>(const DevBatch *, const TbItem *, int32_t, int32_t *, uint8_t *,
                                           uint32_t *, int32_t *, int, cudaStream_t);
 template int occupancy_tb16_c<16, 3>();
-template cudaError_t launch_tbf16_c<16, 3>(const DevBatch *, const TbItem *, int32_t, int32_t *, uint8_t *,
+template cudaError_t launch_tbf16_c<16, 2>(const DevBatch *, const TbItem *, int32_t, int32_t *, uint8_t *,
                                            uint32_t *, int32_t *, int, cudaStream_t);
-template int occupancy_tbf16_c<16, 3>();
+template int occupancy_tbf16_c<16, 2>();
 }  // namespace agatha

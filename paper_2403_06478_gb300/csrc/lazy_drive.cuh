@@ -11,7 +11,7 @@
 
 namespace agatha {
 
-constexpr int LAZY_PAIRS = 16;      // anti-diagonal pairs of a block: one word of each sequence
+constexpr int LAZY_PAIRS = 16;      // anti-diagonal pairs of one word of each sequence
 
 struct Cold16 {
     int32_t mqe, mqe_t, mte, mte_q, gscore;
@@ -27,7 +27,7 @@ struct Cold16 {
 // step: 1 (0: the same lanes keep every anti-diagonal, for the traceback).
 struct LazyEdge { int32_t on, dt, dq; uint32_t ring; int32_t step; };
 
-// Pairs of anti-diagonals the next block may hold: n, 8, 4 or 2 (0: none) such
+// Pairs of anti-diagonals the next block may hold: n, 16, 8, 4 or 2 (0: none) such
 // that no anti-diagonal of it can fire the Z-drop test.  g, m, mu: an upper
 // bound of the global maximum, the maximum of the last two anti-diagonals,
 // and that maximum with the virtual cells.  k anti-diagonals on, no score is
@@ -41,7 +41,7 @@ __device__ __forceinline__ int32_t lazy_span(const DevParams &prm, int32_t n, in
     if (prm.zdrop < 0) return n;
 #pragma unroll 1
     while (n > 0 && max(g - m, mu - m + prm.a * n) + o + c * n > prm.zdrop)
-        n = n > 8 ? 8 : (n > 4 ? 4 : (n > 2 ? 2 : 0));
+        n = n > 16 ? 16 : (n > 8 ? 8 : (n > 4 ? 4 : (n > 2 ? 2 : 0)));
     return n;
 }
 
@@ -83,8 +83,9 @@ __device__ __forceinline__ void lazy_edges(S &s, int32_t r0, int32_t n, int32_t 
 // So only the blocks since the last checkpoint that this rules in can hold
 // it, and when the exact maximum and its cell are wanted (the Z-drop bound
 // no longer holds, the score has passed a peak, or the table ends) the pair
-// goes back to that checkpoint and takes the masked step from there up to
-// exact_until.  Blocks start and end on odd anti-diagonals ((r - w) odd).
+// goes back to that checkpoint and takes the lazy step again from there, with
+// the maximum of every pair of anti-diagonals (the masked step, up to
+// exact_until, where a rebase or the head's end lies between).  Blocks start and end on odd anti-diagonals ((r - w) odd).
 // The head's last four anti-diagonals (w - 2 .. w + 1), where the virtual
 // cells leave the band, run the masked step without its test (blind), as a
 // block of their own; a band that covers the table (cover) has no such
@@ -94,7 +95,9 @@ __device__ __forceinline__ int32_t lazy_drive(S &s, bool use_fast) {
     constexpr int32_t NONE = INT_MIN;
     const DevParams &prm = s.prm;
     const int32_t w = s.w, tlen = s.tlen, qlen = s.qlen, last_r = s.last_r;
-    const bool head = use_fast && w >= 8 && s.lazy_head_ok();    // lazy blocks in the head too
+    // lazy blocks in the head too (by a vote: shared memory's values are not
+    // uniform for the compiler, see WarpPair16::run)
+    const bool head = __any_sync(FULL, use_fast && w >= 8 && s.lazy_head_ok());
     const int32_t L = min(tlen, qlen);
     const int32_t r_in = max(L - 2, 2 * L - 3 - w);    // no cell of the last row or column up to here
     // lazy blocks end here at the latest; past r_in only if the corner is in the band
@@ -119,21 +122,19 @@ __device__ __forceinline__ int32_t lazy_drive(S &s, bool use_fast) {
     int32_t m0 = 0, mu = 0, n = 0;                     // the current block: see lazy_span
     bool block = false, edge = false;
     for (;;) {
+        if constexpr (S::REBASES) {
+            // (one place for it: a second copy costs the instruction cache)
+            if (s.until_rebase < (S::TRACE ? 40 : 16) && r >= 0) {
+                s.lazy_rebase(open ? m0 : s.last_max(), r);
+                if (s.ovf) return r;
+            }
+        }
         if (r < exact_until || !((r - w) & 1)) {
             if (r >= last_r) return r;
             ++r;
-            if (r > -2) s.advance(r);
-            if (s.head_step(r)) return r;
-            bool mark = false;
-            if constexpr (S::TRACE) mark = s.trace_mark(r);
-            if constexpr (S::REBASES) {
-                if (s.until_rebase <= (mark ? 36 : 2) && r >= 0) {
-                    s.lazy_rebase(s.last_max(), r);
-                    if (s.ovf) return r;
-                }
-            }
+            if (s.masked_step(r)) return r;
             if constexpr (S::TRACE) {
-                if (mark) s.trace_save(r, r, false);
+                if (s.trace_mark(r)) s.trace_save(r, r, false);
             }
             continue;
         }
@@ -144,17 +145,29 @@ __device__ __forceinline__ int32_t lazy_drive(S &s, bool use_fast) {
             if (lazy_span(prm, 4, s.gmax, m, m, o1, c1) != 4) { exact_until = r + 8; continue; }
         }
         s.blind = false;
-        if constexpr (S::REBASES) {
-            if (s.until_rebase < (S::TRACE ? 40 : 16)) {
-                s.lazy_rebase(open ? m0 : s.last_max(), r);
-                if (s.ovf) return r;
-            }
-        }
         int32_t rs = r, u0 = s.until_rebase;
         s.lazy_enter(k, two);
+        int32_t target = NONE, seen = NONE, fresh = 0;     // taking blocks again: see below
+        typename S::LazyWin W;
         for (;;) {
             const int32_t m1 = s.lazy_max(k, r, r > w && r <= r_in) + s.lazy_off() - d * (r - rs);
-            if (!open) {
+            if (target != NONE) {
+                // the blocks since the checkpoint once more, pair by pair: the
+                // state of the pair with the highest maximum is kept, which
+                // holds the cell
+                if (m1 > s.gmax) {
+                    s.gmax = m1;
+                    s.lazy_save(old ^ 1, r, rs, u0);
+                    seen = r;
+                }
+                if (r >= target) {
+                    if (seen != NONE) s.lazy_locate(k, old ^ 1, seen, s.gmax - s.lazy_off() + d * (seen - rs));
+                    target = NONE;
+                    best = gval = s.gmax;
+                    upper = NONE;
+                    old = 1;
+                }
+            } else if (!open) {
                 open = true;
                 best = gval = s.gmax;
                 upper = NONE;
@@ -177,70 +190,101 @@ __device__ __forceinline__ int32_t lazy_drive(S &s, bool use_fast) {
             }
             block = false;
             m0 = m1;
-            if constexpr (S::TRACE) {
-                if (s.trace_mark(r)) {
-                    if (u0 - (r - rs) < 36) break;     // a rebase first: none within 32 anti-diagonals of it
-                    s.trace_save(r, rs, true);
+            if (target == NONE) {
+                if constexpr (S::TRACE) {
+                    if (s.trace_mark(r)) {
+                        if (u0 - (r - rs) < 36) break; // a rebase first: none within 32 anti-diagonals of it
+                        s.trace_save(r, rs, true);
+                    }
+                }
+                const bool cross = r == turn;
+                bool close = false;                    // the Z-drop bound leaves no block
+                // the end, or past a peak
+                bool stop = r + 2 > end || (cross && w + 1 > end) ||
+                            (upper != NONE && m0 + prm.a * LAZY_PAIRS <= best);
+                if (!stop) {
+                    int32_t left = S::BLOCK_PAIRS;
+                    if constexpr (S::REBASES) {
+                        left = (u0 - (r - rs) - 4) >> 1;
+                        if (left < (S::TRACE ? 2 : 4)) break;  // a rebase is due
+                    }
+                    edge = cross || r + 2 > r_in;
+                    n = (min(edge ? end : r_in, r < turn ? min(turn, end) : end) - r) >> 1;
+                    if (edge && n < 2 * LAZY_PAIRS) n = min(n, max(4, (n + 1) >> 1));   // shorter towards the end
+                    n = cross ? 2 : min(min(n, left), edge ? S::EDGE_PAIRS : S::BLOCK_PAIRS);
+                    if constexpr (S::TRACE) {
+                        if (!cross) n = min(n, s.trace_room(r));
+                    }
+                    mu = r < w ? max(m0, -gap_cost(prm, r + 1)) : m0;
+                    const int32_t fit =
+                        lazy_span(prm, n, max(best, upper), m0, mu, edge ? o1 : o0, edge ? c1 : c0);
+                    close = fit == 0 || (cross && fit < n);
+                    stop = close;
+                    n = fit;
+                }
+                if (stop) {
+                    const int32_t to = r;
+                    bool again = upper != NONE;
+                    if (again) {                       // back to the checkpoint
+                        s.lazy_load(old);
+                        r = __reduce_max_sync(FULL, s.cold.ck_r[old]);
+                        rs = __reduce_max_sync(FULL, s.cold.ck_rs[old]);
+                        again = !(r <= turn && to > turn);
+                        if constexpr (S::REBASES) {
+                            s.base = __reduce_max_sync(FULL, s.cold.ck_base[old]);
+                            u0 = __reduce_max_sync(FULL, s.cold.ck_u0[old]);
+                            again = again && to - rs <= u0 - 4;
+                        }
+                        s.gmax = gval;
+                    }
+                    if (!again) {                      // on the masked step, if at all
+                        exact_until = to + (close ? 8 : 0);
+                        open = false;
+                        break;
+                    }
+                    target = to;
+                    seen = NONE;
+                    fresh = 0;
+                } else {
+                    last = old ^ 1;
+                    s.lazy_save(last, r, rs, u0);
+                    block = true;
+                    fresh = 0;                         // (the bases are read again)
+                    if (cross) {
+                        s.blind = true;
+                        exact_until = r + 4;
+                        break;
+                    }
                 }
             }
-            const bool cross = r == turn;
-            if (r + 2 > end || (cross && w + 1 > end) || (upper != NONE && m0 + prm.a * LAZY_PAIRS <= best)) {
-                exact_until = r;                       // the end, or past a peak
-                open = false;
-                break;
+            int32_t run = n;
+            if (target != NONE) {
+                if (r >= target) continue;             // (a checkpoint at the place itself)
+                run = 1;
             }
-            int32_t left = LAZY_PAIRS;
-            if constexpr (S::REBASES) {
-                left = (u0 - (r - rs) - 4) >> 1;
-                if (left < (S::TRACE ? 2 : 4)) break;  // a rebase is due
-            }
-            edge = cross || r + 2 > r_in;
-            n = (min(edge ? end : r_in, r < turn ? min(turn, end) : end) - r) >> 1;
-            if (edge && n < 2 * LAZY_PAIRS) n = min(n, max(4, (n + 1) >> 1));   // shorter towards the end
-            n = cross ? 2 : min(min(n, left), edge ? S::EDGE_PAIRS : LAZY_PAIRS);
-            if constexpr (S::TRACE) {
-                if (!cross) n = min(n, s.trace_room(r));
-            }
-            mu = r < w ? max(m0, -gap_cost(prm, r + 1)) : m0;
-            const int32_t fit = lazy_span(prm, n, max(best, upper), m0, mu, edge ? o1 : o0, edge ? c1 : c0);
-            if (fit == 0 || (cross && fit < n)) {
-                exact_until = r + 8;
-                open = false;
-                break;
-            }
-            n = fit;
-            last = old ^ 1;
-            s.lazy_save(last, r, rs, u0);
-            block = true;
-            if (cross) {
-                s.blind = true;
-                exact_until = r + 4;
-                break;
-            }
-            typename S::LazyWin W;
-            s.lazy_windows(W, r);
+            const bool rim = edge && target == NONE;
             const int32_t B = floor_div2(r - w);
-            LazyEdge g{__reduce_max_sync(FULL, edge ? 1 : 0), tlen - 1 - B - s.j0, r - qlen + 1 - B - s.j0, ring, 1};
+            LazyEdge g{__reduce_max_sync(FULL, rim ? 1 : 0), tlen - 1 - B - s.j0, r - qlen + 1 - B - s.j0, ring, 1};
             if (!s.owns()) g.dt = g.dq = -(1 << 20);
-            if (two) s.template lazy_block<true>(n, W, k, g);
-            else s.template lazy_block<false>(n, W, k, g);
-            if (edge) lazy_edges(s, r, n, s.lazy_off() - d * (r - rs), d);
-            r += 2 * n;
-        }
-        if (!open && upper != NONE) {                  // back to the checkpoint
-            s.lazy_load(old);
-            r = __reduce_max_sync(FULL, s.cold.ck_r[old]);
-            rs = __reduce_max_sync(FULL, s.cold.ck_rs[old]);
-            if constexpr (S::REBASES) {
-                s.base = __reduce_max_sync(FULL, s.cold.ck_base[old]);
-                u0 = __reduce_max_sync(FULL, s.cold.ck_u0[old]);
+#pragma unroll 1
+            for (int32_t done = 0;;) {
+                if (fresh == 0) {
+                    s.lazy_windows(W, r + 2 * done);
+                    fresh = LAZY_PAIRS;
+                }
+                const int32_t m = min(run - done, fresh);
+                if (two) s.template lazy_block<true>(m, W, k, g);
+                else s.template lazy_block<false>(m, W, k, g);
+                fresh -= m;
+                done += m;
+                if (S::BLOCK_PAIRS <= LAZY_PAIRS || done >= run) break;
             }
-            s.gmax = gval;
+            if (rim) lazy_edges(s, r, run, s.lazy_off() - d * (r - rs), d);
+            r += 2 * run;
         }
         s.lazy_leave(k, two, r - rs);
         if constexpr (S::REBASES) s.until_rebase = u0 - (r - rs);
         s.set_last_max(m0);
-        s.init_windows(r);
     }
 }
 

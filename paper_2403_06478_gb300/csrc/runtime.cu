@@ -184,8 +184,14 @@ int warp32_occupancy(Shape32 k) {
     }
 }
 
-// 16-bit kernel with C slots per lane; high: the larger register budget
-// (one resident block per SM fewer).
+// 16-bit kernel with C slots per lane at its default budget of registers or
+// (high) the second one, which the autotuner tries too.  The defaults are the
+// faster ones on the workloads: with 16 slots two blocks per SM of up to 255
+// registers, whose lazy loop has no register moves and whose longest pairs
+// have the SM to themselves sooner (20,000 ONT-like pairs 37.2 ms, three blocks
+// of 168 41.3; 5,000 HiFi-like 22.8 and 23.8); with 8 slots three blocks (20,000
+// pairs of 2 kbp at w = 200: 7.3 ms, two 8.4); with 4 slots four (200,000 reads
+// of 150 bp: 4.8 ms, three 5.4); with 24 only two fit.
 static cudaError_t launch_warp16(int C, int high, const DevBatch *d, int blocks, cudaStream_t s,
                                  int fast, int list) {
     switch (C * 2 + high) {
@@ -193,8 +199,8 @@ static cudaError_t launch_warp16(int C, int high, const DevBatch *d, int blocks,
         case 9: return launch_warp16_c<4, 3>(d, blocks, s, fast, list);
         case 16: return launch_warp16_c<8, 3>(d, blocks, s, fast, list);
         case 17: return launch_warp16_c<8, 2>(d, blocks, s, fast, list);
-        case 32: return launch_warp16_c<16, 3>(d, blocks, s, fast, list);
-        case 33: return launch_warp16_c<16, 2>(d, blocks, s, fast, list);
+        case 32: return launch_warp16_c<16, 2>(d, blocks, s, fast, list);
+        case 33: return launch_warp16_c<16, 3>(d, blocks, s, fast, list);
         default: return launch_warp16_c<24, 2>(d, blocks, s, fast, list);
     }
 }
@@ -242,8 +248,8 @@ int warp16_occupancy(int C, int high) {
         case 9: return occupancy_warp16_c<4, 3>();
         case 16: return occupancy_warp16_c<8, 3>();
         case 17: return occupancy_warp16_c<8, 2>();
-        case 32: return occupancy_warp16_c<16, 3>();
-        case 33: return occupancy_warp16_c<16, 2>();
+        case 32: return occupancy_warp16_c<16, 2>();
+        case 33: return occupancy_warp16_c<16, 3>();
         default: return occupancy_warp16_c<24, 2>();
     }
 }

@@ -83,7 +83,7 @@ struct LaunchPlan {
     int32_t warp_w_max = 0;
     int warp_blocks = 0;
     int lane16 = 0, C16 = 0;    // 16-bit lanes allowed; their slots per lane
-    int regs_high = 0;          // 16-bit kernel at its larger register budget
+    int regs_high = 0;          // 16-bit kernel at its second register budget
     int warp16_blocks[2] = {0, 0};   // grid of the 16-bit kernel per budget
     int groupk = 1;             // warps per pair of the single launch (1, 2, 4)
     int warp16k_blocks[2] = {0, 0};  // grids of the 2- and 4-warp kernels (0: none)

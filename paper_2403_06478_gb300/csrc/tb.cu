@@ -87,7 +87,7 @@ cudaError_t launch_tbf16(int C, const DevBatch *d, const TbItem *items, int32_t 
     switch (C) {
         case 4: return launch_tbf16_c<4, 4>(d, items, n, head, dir, ops, ncig, blocks, s);
         case 8: return launch_tbf16_c<8, 3>(d, items, n, head, dir, ops, ncig, blocks, s);
-        case 16: return launch_tbf16_c<16, 3>(d, items, n, head, dir, ops, ncig, blocks, s);
+        case 16: return launch_tbf16_c<16, 2>(d, items, n, head, dir, ops, ncig, blocks, s);
         default: return launch_tbf16_c<24, 2>(d, items, n, head, dir, ops, ncig, blocks, s);
     }
 }
@@ -96,7 +96,7 @@ int tbf16_occupancy(int C) {
     switch (C) {
         case 4: return occupancy_tbf16_c<4, 4>();
         case 8: return occupancy_tbf16_c<8, 3>();
-        case 16: return occupancy_tbf16_c<16, 3>();
+        case 16: return occupancy_tbf16_c<16, 2>();
         default: return occupancy_tbf16_c<24, 2>();
     }
 }
