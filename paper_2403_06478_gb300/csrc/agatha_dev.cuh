@@ -13,6 +13,7 @@
 //   (t, q-1) [F, F2 input] sits in slot j   on r-1 if (r-w) is even, else j+1.
 #pragma once
 
+#include <climits>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -59,7 +60,8 @@ struct DevBatch {
 
 enum : int32_t { CTR_HEAD = 0, CTR_NWARP = 1, CTR_NWIDE = 2, CTR_ERR = 3, CTR_WIDE_HEAD = 4,
                  CTR_NOVF = 5, CTR_OVF_HEAD = 6, CTR_CLS_HEAD = 8, CTR_T_BEGIN = 12, CTR_T_END = 14,
-                 CTR_COUNT = 16 };
+                 CTR_PART = 16, CTR_COUNT = 64 };
+// (the heads of a list's later parts: head + CTR_PART, + 2 CTR_PART ..., see TierQueue)
 
 // Device clock of a step's kernels, in nanoseconds of the GPU's global timer
 // (one clock for every SM): counters[CTR_T_BEGIN..+1] holds when the first
@@ -295,6 +297,89 @@ __device__ __forceinline__ WorkList work_list(const DevBatch &B, int32_t list) {
     return L;
 }
 
+// Whether a list's pairs come longest first.
+__device__ __forceinline__ bool list_sorted(const WorkList &L, int32_t list) {
+    return L.items != nullptr && list != WARP_LIST_NARROW && list != WARP_LIST_OVERFLOW;
+}
+
+// A launch's pairs, handed out so that the longest get most of an SM.  A block
+// fills its SM: its first tier of warps is one per scheduler (or one group of
+// warps per SM), and each further tier shares the schedulers with it.  A lone
+// warp of the 16-slot 16-bit kernel takes 102 ns per anti-diagonal, two on a
+// scheduler 181 each; with 4 slots 70, and 159 for four.  So the list is cut
+// into parts: `units` pairs, the longest, of which each first tier takes one,
+// then as many for the second tiers, then for the third, and the rest.  Tier t
+// starts with part t and goes on to the next ones; of a batch that fits the
+// first tiers the others take nothing.  And before a later tier starts, it asks
+// whether its scheduler's first pair is one that bounds the launch
+// (tier_crowded), and then leaves it alone for good.  One GB300, kernel time
+// against one queue for all warps (which pile up on the SMs that start first):
+// 256 pairs of 1 kbp 0.32 -> 0.19 ms, 2,500 ONT-like pairs 14.0 -> 11.0 (int32
+// lanes 23.7 -> 20.4), 1,000 of them at w = 1,000 28.7 -> 20.6, 100,000 pairs of
+// Pareto lengths 71 -> 65; of the batches that no long pair bounds, 20,000 reads
+// -1%, ONT-like and HiFi-like ones +1% (two blocks on an SM share it less evenly,
+// which ends a batch less raggedly).
+// The state lives in shared memory (the loops over pairs have no registers to
+// spare): one TierQueue per block, one place per warp that asks.
+struct TierQueue {
+    static constexpr int PARTS = 4;
+    int32_t *head;               // of part p: head[CTR_PART * p]
+    int32_t at[PARTS + 1];       // where the parts start
+
+    __device__ __forceinline__ void open(int32_t *head_, int32_t begin, int32_t end, int32_t units) {
+        head = head_;
+        for (int p = 0; p < PARTS; ++p) at[p] = min((int64_t)end, begin + (int64_t)p * units);
+        at[PARTS] = end;
+    }
+    __device__ __forceinline__ static int32_t start(int32_t tier) { return min(tier, PARTS - 1); }
+    // The next pair's place in the list, INT_MAX if there is none (one lane
+    // asks).  place: the part, the first one (start(tier)) and whether the warp
+    // has had a pair: a tier that has had one also helps with the parts before
+    // its own, whose blocks another launch may keep from starting.
+    // (Out of line: the loops over pairs are tight for the instruction cache.)
+    __device__ __noinline__ int32_t next(int32_t &place) {
+        int32_t v = place;
+        for (;;) {
+            const int32_t p = v & 3, k = at[p] + atomicAdd(head + CTR_PART * p, 1);
+            if (k < at[p + 1]) {
+                place = v | 16;
+                return k;
+            }
+            const int32_t to = (p + 1) & 3;
+            if (to == (v >> 2 & 3) || (to == 0 && !(v & 16))) return INT_MAX;
+            v = (v & ~3) | to;
+        }
+    }
+    __device__ __forceinline__ static int32_t first_place(int32_t tier) { return start(tier) * 5; }
+};
+
+// Whether warps of tier `tier` (1, 2 ..) would hold up the launch by sharing
+// the scheduler of the list's pair `mine`, or have nothing to do.  With them a
+// step of that pair takes tier + 1 of the time that a step costs on a full SM;
+// alone it takes `lone` of it.  The launch cannot end before its longest pair
+// run alone, nor much before the average load of the `units` schedulers; the
+// pair is crowded if it would take longer than both.  steps(k): anti-diagonals
+// of the list's k-th pair, which fall with k (32 samples give the sum).
+template <class Steps>
+__device__ __noinline__ bool tier_crowded(const TierQueue &q, int32_t mine, int32_t tier, int32_t units, float lone,
+                                          Steps steps) {
+    const int32_t begin = q.at[0], end = q.at[TierQueue::PARTS], n = end - begin, lane = threadIdx.x & 31;
+    if (mine >= end || q.at[q.start(tier)] >= end) return true;
+    const uint32_t x = (uint32_t)steps(begin + (int32_t)((int64_t)(2 * lane + 1) * n / 64));
+    const float load = (float)__reduce_add_sync(0xffffffffu, x) * ((float)n / 32.0f) / (float)units;
+    const float t = fmaxf(load + lone * (float)steps(q.at[1]), lone * (float)steps(begin));
+    return (float)steps(mine) * (float)(tier + 1) > t;
+}
+
+// Steps of the sorted list of a score launch.
+struct ListSteps {
+    const int32_t *items, *t_len, *q_len;
+    __device__ __forceinline__ int32_t operator()(int32_t k) const {
+        const int32_t i = items[k];
+        return t_len[i] + q_len[i];
+    }
+};
+
 // One pair of a traceback launch: its end cell (from the score path) and
 // where its direction table (bytes) and run scratch (uint32) start.
 struct TbItem {
@@ -311,7 +396,8 @@ cudaError_t launch_warp_c(const DevBatch *d_batch, int n_blocks, cudaStream_t s,
                           int list = WARP_LIST_MAIN);
 template <int C, int K = 1>
 int occupancy_warp_c();
-// MINB: resident blocks per SM the 16-bit kernel's registers are cut for.
+// MINB: warps per scheduler the 16-bit kernel's registers are cut for (one
+// block per SM holds them; with G = 16 that many blocks of four).
 // G: lanes per pair (32, or 16 for two pairs per warp).
 template <int C, int MINB, int G = 32>
 cudaError_t launch_warp16_c(const DevBatch *d_batch, int n_blocks, cudaStream_t s, int use_fast,
@@ -337,8 +423,8 @@ cudaError_t launch_tb16_c(const DevBatch *d_batch, const TbItem *items, int32_t 
 template <int C, int MINB>
 int occupancy_tb16_c();
 template <int C, int MINB>
-cudaError_t launch_tbf16_c(const DevBatch *d_batch, const TbItem *items, int32_t n_items, int32_t *head,
-                           uint8_t *dir, uint32_t *ops, int32_t *n_cigar, int n_blocks, cudaStream_t s);
+cudaError_t launch_tbf16_c(const DevBatch *d_batch, const TbItem *items, int32_t n_items, uint8_t *dir,
+                           uint32_t *ops, int32_t *n_cigar, int n_blocks, cudaStream_t s);
 template <int C, int MINB>
 int occupancy_tbf16_c();
 // Copy each pair's runs (written end first) to dense[dst_off[pair]..] in order.

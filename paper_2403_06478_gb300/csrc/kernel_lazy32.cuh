@@ -22,7 +22,7 @@
 
 namespace agatha {
 
-// K warps (a block of its own when K > 1) share one pair's band: warp k holds
+// K warps share one pair's band: warp k holds
 // lanes 30k .. 30k + 31 of the frame, so that neighbouring warps have two lanes
 // in common.  Lane 0 of every warp but the first and lane 31 of every one but
 // the last are halos, copies of the neighbour's lanes 30 and 1: whatever enters
@@ -60,15 +60,21 @@ struct LazyPair32 {
     Cold16 &cold;
     int32_t *ring;
     int32_t wk;                   // this warp's place in the group
-    int32_t *xch;                 // K > 1: the halo exchange, then two maxima and one place per warp
+    int32_t *xch0;                // K > 1: of group 0, the halo exchange, then two maxima and one place per
+                                  // warp, and the next pair
     int32_t age, flip, mflip;     // anti-diagonals since the halo was fresh; buffer halves
     int4 *ck;                     // this lane's words of the warp's two checkpoints
 
-    __device__ explicit LazyPair32(Cold16 &c, int32_t *rg, int4 *ck_, int32_t wk_ = 0, int32_t *x = nullptr)
-        : cold(c), ring(rg), wk(wk_), xch(x), flip(0), mflip(0), ck(ck_) {}
+    __device__ explicit LazyPair32(Cold16 &c, int32_t *rg, int4 *ck_, int32_t wk_, int32_t *x)
+        : cold(c), ring(rg), wk(wk_), xch0(x), flip(0), mflip(0), ck(ck_) {}
 
+    static constexpr int XCH = K > 1 ? (HALO + 3 * K + 4) / 4 * 4 : 4;
+    // the group's exchange and barrier, from the thread's place each time: no
+    // registers to keep them in
+    __device__ __forceinline__ static int32_t group() { return (int32_t)(threadIdx.x / (32 * K)); }
+    __device__ __forceinline__ int32_t *xch() const { return xch0 + group() * XCH; }
     __device__ __forceinline__ static void group_sync() {
-        if constexpr (K > 1) __syncthreads();
+        if constexpr (K > 1) asm volatile("bar.sync %0, %1;" :: "r"(1 + group()), "n"(32 * K) : "memory");
     }
     __device__ __forceinline__ bool leader() const { return lane == 0 && wk == 0; }
     // not a halo lane
@@ -78,10 +84,10 @@ struct LazyPair32 {
     __device__ __forceinline__ int32_t group_max(int32_t v) {
         int32_t m = __reduce_max_sync(FULL, v);
         if constexpr (K > 1) {
-            int32_t *x = xch + HALO + mflip * K;
+            int32_t *x = xch() + HALO + mflip * K;
             mflip ^= 1;
             if (lane == 0) x[wk] = m;
-            __syncthreads();
+            group_sync();
 #pragma unroll
             for (int i = 0; i < K; ++i) m = max(m, x[i]);
             m = __reduce_max_sync(FULL, m);
@@ -91,10 +97,10 @@ struct LazyPair32 {
     // The halo lanes from the neighbours' own lanes.
     __device__ __forceinline__ void refresh() {
         if constexpr (K > 1) {
-            int4 *x = reinterpret_cast<int4 *>(xch) + flip * (K * 2 * CKV);
+            int4 *x = reinterpret_cast<int4 *>(xch()) + flip * (K * 2 * CKV);
             flip ^= 1;
             if (lane == 1 || lane == 30) put(x + (wk * 2 + (lane == 30 ? 1 : 0)) * CKV, 1);
-            __syncthreads();
+            group_sync();
             if (!owns()) get(x + (lane == 0 ? (wk - 1) * 2 + 1 : (wk + 1) * 2) * CKV, 1);
             __syncwarp();
             age = 0;
@@ -233,13 +239,13 @@ struct LazyPair32 {
             int32_t tstar = __shfl_sync(FULL, B + j0 + li, ball ? __ffs(ball) - 1 : 0);
             if constexpr (K > 1) {
                 // of the first warp that has it
-                int32_t *x = xch + HALO + 2 * K;
+                int32_t *x = xch() + HALO + 2 * K;
                 if (lane == 0) x[wk] = ball ? tstar : INT_MAX;
-                __syncthreads();
+                group_sync();
                 tstar = x[0];
 #pragma unroll
                 for (int i = 1; i < K; ++i) tstar = min(tstar, x[i]);
-                __syncthreads();
+                group_sync();
             }
             const int32_t qstar = r - tstar;
             if (m > gmax) {
@@ -468,16 +474,16 @@ struct LazyPair32 {
             t[c] = __reduce_min_sync(FULL, owns() ? at : INT_MAX);
         }
         if constexpr (K > 1) {
-            int32_t *x = xch + HALO;                  // 2 K words: both halves of the maxima
-            __syncthreads();
+            int32_t *x = xch() + HALO;                  // 2 K words: both halves of the maxima
+            group_sync();
             if (lane == 0) { x[2 * wk] = t[0]; x[2 * wk + 1] = t[1]; }
-            __syncthreads();
+            group_sync();
 #pragma unroll
             for (int i = 0; i < K; ++i) {
                 t[0] = min(t[0], x[2 * i]);
                 t[1] = min(t[1], x[2 * i + 1]);
             }
-            __syncthreads();
+            group_sync();
         }
         if (leader()) {
             const bool first = t[0] != INT_MAX;
@@ -595,48 +601,75 @@ struct LazyPair32 {
     }
 };
 
-// Resident blocks per SM the registers are cut for: six arrays of C values and
+// Warps per scheduler (K > 1: groups per SM) the registers are cut for: six arrays of C values and
 // no spills in the lazy loop, within what the checkpoints' shared memory admits.
 template <int C, int K>
-constexpr int warp32_blocks() {
+__host__ __device__ constexpr int warp32_blocks() {
     return K > 1 ? (C <= 8 ? 5 : 3) : (C <= 4 ? 5 : (C <= 8 ? 4 : 2));
 }
+template <int C, int K>
+__host__ __device__ constexpr int warp32_threads() { return (K == 1 ? WARP_BLOCK_THREADS : 32 * K) * warp32_blocks<C, K>(); }
 // Dynamic shared memory of a block: two checkpoints of every warp.
 template <int C, int K>
 constexpr int warp32_smem() {
-    return (K == 1 ? WARP_BLOCK_THREADS / 32 : K) * 2 * LazyPair32<C, K>::CKV * 32 * 16;
+    return warp32_threads<C, K>() / 32 * 2 * LazyPair32<C, K>::CKV * 32 * 16;
 }
 
+// What a lone warp (group) takes per anti-diagonal of what one costs on a full SM.
 template <int C, int K>
-__global__ void __launch_bounds__(K == 1 ? WARP_BLOCK_THREADS : 32 * K, warp32_blocks<C, K>())
+__host__ __device__ constexpr float warp32_lone() {
+    return K > 1 ? (C <= 8 ? 1.8f : 1.5f) : (C <= 4 ? 1.6f : (C <= 8 ? 1.4f : 1.15f));
+}
+
+// One block per SM; see TierQueue.
+template <int C, int K>
+__global__ void __launch_bounds__(warp32_threads<C, K>(), 1)
 warp_align_kernel(const DevBatch *__restrict__ d_batch, int32_t use_fast, int32_t list) {
-    constexpr int G = K == 1 ? WARP_BLOCK_THREADS / 32 : 1;      // pairs at a time
+    constexpr int G = warp32_threads<C, K>() / (32 * K);         // pairs at a time
+    constexpr int U = K == 1 ? 4 : 1;                            // of the first tier
     using Pair = LazyPair32<C, K>;
     __shared__ Cold16 cold[G];
     __shared__ __align__(16) int32_t ring[G][Pair::RING];
-    __shared__ __align__(16) int32_t xch[K > 1 ? Pair::HALO + 3 * K + 1 : 1];
+    __shared__ __align__(16) int32_t xch[K > 1 ? G : 1][Pair::XCH];
+    __shared__ TierQueue q;
+    __shared__ int32_t first[U], place[G];
     extern __shared__ int4 lazy32_smem[];
     const DevBatch B = *d_batch;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int g = K == 1 ? warp : 0, wk = K == 1 ? 0 : warp;
+    const int g = warp / K, wk = warp - g * K, tier = g / U;
+    const bool asks = lane == 0 && wk == 0;
     const WorkList L = work_list(B, list);
     const int32_t l_end = __reduce_max_sync(FULL, L.end);
+    if (threadIdx.x == 0) q.open(L.head, L.begin, l_end, U * (int32_t)gridDim.x);
+    if (asks) place[g] = q.first_place(tier);
+    __syncthreads();
+    int32_t k = INT_MAX;
+    if (tier == 0 && asks) first[g] = k = q.next(place[g]);
+    __syncthreads();
+    if (tier > 0) {
+        if (list_sorted(L, list) &&
+            tier_crowded(q, first[g % U], tier, U * (int32_t)gridDim.x, warp32_lone<C, K>(),
+                         ListSteps{L.items, B.t_len, B.q_len}))
+            k = l_end;
+        else if (asks) k = q.next(place[g]);
+    }
     for (;;) {
-        int32_t k = INT_MIN;
-        if (lane == 0 && wk == 0) k = L.begin + atomicAdd(L.head, 1);
         if constexpr (K > 1) {
-            int32_t &next = xch[Pair::HALO + 3 * K];
-            if (threadIdx.x == 0) next = k;
-            __syncthreads();
+            int32_t &next = xch[g][Pair::HALO + 3 * K];
+            if (asks) next = k;
+            Pair::group_sync();
             k = next;
-            __syncthreads();
+            Pair::group_sync();
         }
-        k = __reduce_max_sync(FULL, k);
+        k = __reduce_min_sync(FULL, k);
         if (k >= l_end) break;
         const int32_t pair = L.items ? L.items[k] : k;
-        if (__any_sync(FULL, !L.items && (!pair_valid(B, pair) || !warp_takes(B, pair)))) continue;
-        Pair wp(cold[g], ring[g], lazy32_smem + warp * (2 * Pair::CKV * 32) + lane, wk, xch);
-        wp.run(B, pair, lane, use_fast != 0);
+        k = INT_MAX;
+        if (__any_sync(FULL, L.items || (pair_valid(B, pair) && warp_takes(B, pair)))) {
+            Pair wp(cold[g], ring[g], lazy32_smem + warp * (2 * Pair::CKV * 32) + lane, wk, xch[0]);
+            wp.run(B, pair, lane, use_fast != 0);
+        }
+        if (asks) k = q.next(place[g]);
     }
     if (lane == 0) mark_step_end(B.counters);
 }
@@ -644,8 +677,7 @@ warp_align_kernel(const DevBatch *__restrict__ d_batch, int32_t use_fast, int32_
 template <int C, int K>
 cudaError_t launch_warp_c(const DevBatch *d_batch, int n_blocks, cudaStream_t s, int use_fast,
                           int list) {
-    warp_align_kernel<C, K><<<n_blocks, K == 1 ? WARP_BLOCK_THREADS : 32 * K, warp32_smem<C, K>(), s>>>(
-        d_batch, use_fast, list);
+    warp_align_kernel<C, K><<<n_blocks, warp32_threads<C, K>(), warp32_smem<C, K>(), s>>>(d_batch, use_fast, list);
     return cudaGetLastError();
 }
 
@@ -657,7 +689,7 @@ int occupancy_warp_c() {
     if (cudaFuncSetAttribute(warp_align_kernel<C, K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              warp32_smem<C, K>()) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, warp_align_kernel<C, K>,
-                                                      K == 1 ? WARP_BLOCK_THREADS : 32 * K,
+                                                      warp32_threads<C, K>(),
                                                       warp32_smem<C, K>()) != cudaSuccess)
         return 1;
     return nb > 0 ? nb : 1;

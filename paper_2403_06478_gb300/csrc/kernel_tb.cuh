@@ -487,22 +487,37 @@ __host__ __device__ constexpr int tbf16_warp_smem() {                 // 16-byte
     return a > b ? a : b;
 }
 
+// One block per SM of MINB warps per scheduler; TierQueue hands out the items,
+// with the slot's counters as its heads.
 template <int C, int MINB>
-__global__ void __launch_bounds__(WARP_BLOCK_THREADS, MINB)
+__global__ void __launch_bounds__(WARP_BLOCK_THREADS * MINB, 1)
 tbf16_kernel(const DevBatch *__restrict__ d_batch, const TbItem *__restrict__ items, int32_t n_items,
-             int32_t *head, uint8_t *states, uint32_t *ops, int32_t *n_cigar) {
-    __shared__ Cold16 cold[WARP_BLOCK_THREADS / 32];
+             uint8_t *states, uint32_t *ops, int32_t *n_cigar) {
+    __shared__ Cold16 cold[WARP_BLOCK_THREADS * MINB / 32];
+    __shared__ TierQueue q;
+    __shared__ int32_t first[4], place[WARP_BLOCK_THREADS * MINB / 32];
     extern __shared__ uint4 lazy_smem[];
     const DevBatch B = *d_batch;
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, tier = warp >> 2;
+    const int32_t units = 4 * (int32_t)gridDim.x;
+    if (threadIdx.x == 0) q.open(&B.counters[CTR_HEAD], 0, n_items, units);
+    if (lane == 0) place[warp] = q.first_place(tier);
+    __syncthreads();
+    int32_t k = INT_MAX;
+    if (tier == 0 && lane == 0) first[warp] = k = q.next(place[warp]);
+    __syncthreads();
+    if (tier > 0) {
+        const auto steps = [&](int32_t i) { return items[i].end_t + items[i].end_q + 1; };
+        if (tier_crowded(q, first[warp & 3], tier, units, warp16_lone(C), steps)) k = n_items;
+        else if (lane == 0) k = q.next(place[warp]);
+    }
     for (;;) {
-        int32_t k = INT_MIN;
-        if (lane == 0) k = atomicAdd(head, 1);
-        k = __reduce_max_sync(FULL, k);
+        k = __reduce_min_sync(FULL, k);
         if (k >= n_items) break;
         const TbItem it = items[k];
-        TracePair<C> wp(cold[threadIdx.x >> 5]);
-        wp.ck = lazy_smem + (threadIdx.x >> 5) * tbf16_warp_smem<C>();
+        k = INT_MAX;
+        TracePair<C> wp(cold[warp]);
+        wp.ck = lazy_smem + warp * tbf16_warp_smem<C>();
         int32_t n = -1;
         if (!wp.run(B, it.pair, lane, true, states + it.dir_off)) {    // the int32 score kernel takes it
             if (lane == 0) {
@@ -514,25 +529,29 @@ tbf16_kernel(const DevBatch *__restrict__ d_batch, const TbItem *__restrict__ it
             n = wp.end_t < 0 || wp.end_q < 0 ? 0      // the maximum is the origin
                                              : tb_trace(wp, ops + it.ops_off, wp.end_t + wp.end_q + 2);
         }
-        if (lane == 0) n_cigar[it.pair] = n;
+        if (lane == 0) {
+            n_cigar[it.pair] = n;
+            k = q.next(place[warp]);
+        }
     }
 }
 
 template <int C, int MINB>
-cudaError_t launch_tbf16_c(const DevBatch *d_batch, const TbItem *items, int32_t n_items, int32_t *head,
+cudaError_t launch_tbf16_c(const DevBatch *d_batch, const TbItem *items, int32_t n_items,
                            uint8_t *dir, uint32_t *ops, int32_t *n_cigar, int n_blocks, cudaStream_t s) {
-    tbf16_kernel<C, MINB><<<n_blocks, WARP_BLOCK_THREADS, (WARP_BLOCK_THREADS / 32) * 16 * tbf16_warp_smem<C>(),
-                            s>>>(d_batch, items, n_items, head, dir, ops, n_cigar);
+    tbf16_kernel<C, MINB><<<n_blocks, WARP_BLOCK_THREADS * MINB,
+                            (WARP_BLOCK_THREADS * MINB / 32) * 16 * tbf16_warp_smem<C>(), s>>>(
+        d_batch, items, n_items, dir, ops, n_cigar);
     return cudaGetLastError();
 }
 
 template <int C, int MINB>
 int occupancy_tbf16_c() {
     int nb = 0;
-    constexpr int smem = (WARP_BLOCK_THREADS / 32) * 16 * tbf16_warp_smem<C>();
+    constexpr int smem = (WARP_BLOCK_THREADS * MINB / 32) * 16 * tbf16_warp_smem<C>();
     if (cudaFuncSetAttribute(tbf16_kernel<C, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
             cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, tbf16_kernel<C, MINB>, WARP_BLOCK_THREADS, smem) !=
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, tbf16_kernel<C, MINB>, WARP_BLOCK_THREADS * MINB, smem) !=
             cudaSuccess)
         return 1;
     return nb > 0 ? nb : 1;

@@ -169,7 +169,7 @@ struct WarpPair16 {
     // 16+2(p mod 8), of lo for p < 8 and of hi for p >= 8 (C = 24 only)
     struct Comb { uint32_t lo, hi; };
 
-    // each sequence as its own words: base k of the pair at index k + phase
+    // each sequence as its own words: base k of the pair at index k + place
     // of the words from tp (qp); reads outside [0, span) words give 0 (those
     // bases only reach cells outside the table)
     const uint32_t *tp, *qp;
@@ -201,7 +201,7 @@ struct WarpPair16 {
     uint32_t Tpf, Qpf;
     int32_t wcnt;          // pairs of shifts left in Tpf and Qpf (one count for both)
     int32_t tpos, qpos;    // next prefetch position (bases, word-relative)
-    int32_t tph, qph;      // phase of each sequence's first base in its first word
+    int32_t tph, qph;      // place of each sequence's first base in its first word
     uint4 *ck;             // LAZY: the warp's two checkpoints and edge ring
     // relative scores
     int32_t base, OFF, last_m;
@@ -1788,31 +1788,53 @@ struct WarpPair16 {
 
 // G = 16: each half warp aligns its own pairs (two pairs per warp), taking
 // them from the queue on its own.
+//
+// G = 32: one block per SM of MINB warps per scheduler (see TierQueue).
+__host__ __device__ constexpr int warp16_threads(int minb, int G) { return G == 32 ? WARP_BLOCK_THREADS * minb : WARP_BLOCK_THREADS; }
+// What a lone warp takes per anti-diagonal of what one costs on a full SM.
+__host__ __device__ constexpr float warp16_lone(int C) { return C <= 4 ? 1.75f : (C <= 8 ? 1.4f : 1.15f); }
+
 template <int C, int MINB, int G = 32>
-__global__ void __launch_bounds__(WARP_BLOCK_THREADS, MINB)
+__global__ void __launch_bounds__(warp16_threads(MINB, G), G == 32 ? 1 : MINB)
 warp16_align_kernel(const DevBatch *__restrict__ d_batch, int32_t use_fast, int32_t list) {
-    __shared__ Cold16 cold[WARP_BLOCK_THREADS / G];
+    __shared__ Cold16 cold[warp16_threads(MINB, G) / G];
     const DevBatch B = *d_batch;
     const int lane = threadIdx.x & (G - 1);
     const WorkList L = work_list(B, list);
     if constexpr (G == 32) {
         using Pair = WarpPair16<C, false, false, false, 1, true, false, 32, true>;
         extern __shared__ uint4 lazy_smem[];
+        __shared__ TierQueue q;
+        __shared__ int32_t first[4], place[warp16_threads(MINB, G) / 32];
         const int32_t l_end = __reduce_max_sync(FULL, L.end);
-        uint4 *ck = lazy_smem + (threadIdx.x >> 5) * (2 * Pair::CKV * 32 + Pair::RING / 4);
+        const int32_t warp = threadIdx.x >> 5, tier = warp >> 2;
+        uint4 *ck = lazy_smem + warp * (2 * Pair::CKV * 32 + Pair::RING / 4);
+        if (threadIdx.x == 0) q.open(L.head, L.begin, l_end, 4 * (int32_t)gridDim.x);
+        if (lane == 0) place[warp] = q.first_place(tier);
+        __syncthreads();
+        int32_t k = INT_MAX;
+        if (tier == 0 && lane == 0) first[warp] = k = q.next(place[warp]);
+        __syncthreads();
+        if (tier > 0) {
+            if (list_sorted(L, list) && tier_crowded(q, first[warp & 3], tier, 4 * (int32_t)gridDim.x, warp16_lone(C),
+                                                     ListSteps{L.items, B.t_len, B.q_len}))
+                k = l_end;
+            else if (lane == 0) k = q.next(place[warp]);
+        }
         for (;;) {
-            int32_t k = INT_MIN;
-            if (lane == 0) k = L.begin + atomicAdd(L.head, 1);
-            k = __reduce_max_sync(FULL, k);
+            k = __reduce_min_sync(FULL, k);
             if (k >= l_end) break;
             const int32_t pair = L.items ? L.items[k] : k;
-            if (__any_sync(FULL, !L.items && (!pair_valid(B, pair) || !warp_takes(B, pair)))) continue;
-            Pair wp(cold[threadIdx.x / G]);
-            wp.ck = ck;
-            if (!wp.run(B, pair, lane, use_fast != 0) && lane == 0) {
-                const int32_t slot = atomicAdd(&B.counters[CTR_NOVF], 1);
-                B.ovf_list[slot] = pair;
+            k = INT_MAX;
+            if (__any_sync(FULL, L.items || (pair_valid(B, pair) && warp_takes(B, pair)))) {
+                Pair wp(cold[warp]);
+                wp.ck = ck;
+                if (!wp.run(B, pair, lane, use_fast != 0) && lane == 0) {
+                    const int32_t slot = atomicAdd(&B.counters[CTR_NOVF], 1);
+                    B.ovf_list[slot] = pair;
+                }
             }
+            if (lane == 0) k = q.next(place[warp]);
         }
     } else {
         using Pair = WarpPair16<C, MINB < 4, true, false, 1, true, true, G>;
@@ -1893,17 +1915,17 @@ int occupancy_warp16k_c() {
 
 // Dynamic shared memory of a block: two checkpoints and the edge ring of every
 // warp.
-template <int C, int G>
+template <int C, int MINB, int G>
 constexpr int warp16_smem() {
     using Pair = WarpPair16<C, false, false, false, 1, true, false, 32, true>;
-    return G == 32 ? (WARP_BLOCK_THREADS / 32) * (2 * Pair::CKV * 32 * 16 + Pair::RING * 4) : 0;
+    return G == 32 ? (warp16_threads(MINB, G) / 32) * (2 * Pair::CKV * 32 * 16 + Pair::RING * 4) : 0;
 }
 
 template <int C, int MINB, int G>
 cudaError_t launch_warp16_c(const DevBatch *d_batch, int n_blocks, cudaStream_t s, int use_fast,
                             int list) {
-    warp16_align_kernel<C, MINB, G><<<n_blocks, WARP_BLOCK_THREADS, warp16_smem<C, G>(), s>>>(d_batch, use_fast,
-                                                                                              list);
+    warp16_align_kernel<C, MINB, G>
+        <<<n_blocks, warp16_threads(MINB, G), warp16_smem<C, MINB, G>(), s>>>(d_batch, use_fast, list);
     return cudaGetLastError();
 }
 
@@ -1915,8 +1937,8 @@ cudaError_t launch_warp16_prio(const DevBatch *d_batch, int n_blocks, cudaStream
                                int priority) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)n_blocks);
-    cfg.blockDim = dim3(WARP_BLOCK_THREADS);
-    cfg.dynamicSmemBytes = warp16_smem<C, 32>();
+    cfg.blockDim = dim3(warp16_threads(MINB, 32));
+    cfg.dynamicSmemBytes = warp16_smem<C, MINB, 32>();
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributePriority;
@@ -1932,9 +1954,9 @@ template <int C, int MINB, int G>
 int occupancy_warp16_c() {
     int nb = 0;
     if (cudaFuncSetAttribute(warp16_align_kernel<C, MINB, G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             warp16_smem<C, G>()) != cudaSuccess ||
+                             warp16_smem<C, MINB, G>()) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, warp16_align_kernel<C, MINB, G>,
-                                                      WARP_BLOCK_THREADS, warp16_smem<C, G>()) != cudaSuccess)
+                                                      warp16_threads(MINB, G), warp16_smem<C, MINB, G>()) != cudaSuccess)
         return 1;
     return nb > 0 ? nb : 1;
 }

@@ -1,5 +1,5 @@
 // Instantiation of the 16-bit packed-lane warp kernel for 20 band slots per
-// lane (a 640-slot frame, w <= 638) at two resident blocks per SM: the frame
+// lane (a 640-slot frame, w <= 638) at two warps per scheduler: the frame
 // of the pairs of a 24-slot batch whose own band fits it.
 #include "kernel_warp16.cuh"
 

@@ -1,5 +1,5 @@
 // Instantiations of the 16-bit packed-lane warp kernel for 24 band slots per
-// lane (w <= 767), at two register budgets (resident blocks per SM): the
+// lane (w <= 767), at two register budgets (warps per scheduler): the
 // autotuner picks one per length class.
 #include "kernel_tb.cuh"
 
@@ -11,7 +11,7 @@ template cudaError_t launch_warp16_prio<24, 2>(const DevBatch *, int, cudaStream
 template cudaError_t launch_tb16_c<24, 2>(const DevBatch *, const TbItem *, int32_t, int32_t *, uint8_t *,
                                           uint32_t *, int32_t *, int, cudaStream_t);
 template int occupancy_tb16_c<24, 2>();
-template cudaError_t launch_tbf16_c<24, 2>(const DevBatch *, const TbItem *, int32_t, int32_t *, uint8_t *,
-                                           uint32_t *, int32_t *, int, cudaStream_t);
+template cudaError_t launch_tbf16_c<24, 2>(const DevBatch *, const TbItem *, int32_t, uint8_t *, uint32_t *,
+                                           int32_t *, int, cudaStream_t);
 template int occupancy_tbf16_c<24, 2>();
 }  // namespace agatha

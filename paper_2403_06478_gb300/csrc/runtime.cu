@@ -155,10 +155,9 @@ int pick_slots_per_lane(int32_t w) {
 // The int32 score kernel's shape for a band of half-width w: slots per lane
 // and warps per pair.  One warp does the least work per cell as long as 16
 // slots per lane hold the band (20,000 pairs of 1,500 bp at w = 500: 17.8 ms
-// against 33.6 with three warps of 8 slots, and even 2,500 ONT-like pairs,
-// which the longest pair bounds, 23.7 against 30.9 ms).  Beyond that its six
-// arrays do not fit the registers any more, and three warps share the band
-// (1,000 ONT-like pairs at w = 1,000: 120 ms on one warp of 32 slots, 30 ms).
+// against 33.6 with three warps of 8 slots).  Beyond that its six arrays do not
+// fit the registers any more, and three warps share the band (1,000 ONT-like
+// pairs at w = 1,000: 120 ms on one warp of 32 slots, 21 ms).
 Shape32 pick_shape32(int32_t w) {
     if (w <= 511) return {w <= 127 ? 4 : (w <= 255 ? 8 : 16), 1};
     return {w <= 734 ? 8 : 12, 3};
@@ -186,12 +185,11 @@ int warp32_occupancy(Shape32 k) {
 
 // 16-bit kernel with C slots per lane at its default budget of registers or
 // (high) the second one, which the autotuner tries too.  The defaults are the
-// faster ones on the workloads: with 16 slots two blocks per SM of up to 255
-// registers, whose lazy loop has no register moves and whose longest pairs
-// have the SM to themselves sooner (20,000 ONT-like pairs 37.2 ms, three blocks
-// of 168 41.3; 5,000 HiFi-like 22.8 and 23.8); with 8 slots three blocks (20,000
-// pairs of 2 kbp at w = 200: 7.3 ms, two 8.4); with 4 slots four (200,000 reads
-// of 150 bp: 4.8 ms, three 5.4); with 24 only two fit.
+// faster ones on the workloads: with 16 slots two warps per scheduler of up to
+// 255 registers, whose lazy loop has no register moves (20,000 ONT-like pairs
+// 37.6 ms, three warps of 168 38.3; 5,000 HiFi-like 23.1 and 23.6); with 8 slots
+// three (20,000 pairs of 2 kbp at w = 200: 7.3 ms, two 8.4); with 4 slots four
+// (200,000 reads of 150 bp: 4.5 ms, three 5.4); with 24 only two fit.
 static cudaError_t launch_warp16(int C, int high, const DevBatch *d, int blocks, cudaStream_t s,
                                  int fast, int list) {
     switch (C * 2 + high) {

@@ -82,13 +82,13 @@ cudaError_t launch_tb16(int C, const DevBatch *d, const TbItem *items, int32_t n
 }
 
 // fused score path and traceback on 16-bit lanes
-cudaError_t launch_tbf16(int C, const DevBatch *d, const TbItem *items, int32_t n, int32_t *head,
-                         uint8_t *dir, uint32_t *ops, int32_t *ncig, int blocks, cudaStream_t s) {
+cudaError_t launch_tbf16(int C, const DevBatch *d, const TbItem *items, int32_t n, uint8_t *dir, uint32_t *ops,
+                         int32_t *ncig, int blocks, cudaStream_t s) {
     switch (C) {
-        case 4: return launch_tbf16_c<4, 4>(d, items, n, head, dir, ops, ncig, blocks, s);
-        case 8: return launch_tbf16_c<8, 3>(d, items, n, head, dir, ops, ncig, blocks, s);
-        case 16: return launch_tbf16_c<16, 2>(d, items, n, head, dir, ops, ncig, blocks, s);
-        default: return launch_tbf16_c<24, 2>(d, items, n, head, dir, ops, ncig, blocks, s);
+        case 4: return launch_tbf16_c<4, 4>(d, items, n, dir, ops, ncig, blocks, s);
+        case 8: return launch_tbf16_c<8, 3>(d, items, n, dir, ops, ncig, blocks, s);
+        case 16: return launch_tbf16_c<16, 2>(d, items, n, dir, ops, ncig, blocks, s);
+        default: return launch_tbf16_c<24, 2>(d, items, n, dir, ops, ncig, blocks, s);
     }
 }
 
@@ -308,7 +308,13 @@ extern "C" int agatha_align_cigar(agatha_ctx *ctx, const agatha_batch *batch, co
             uint8_t *dir = (uint8_t *)tb.dir.ptr;
             uint32_t *ops = (uint32_t *)tb.ops.ptr;
             int32_t *ncg = (int32_t *)tb.n_cigar.ptr;
-            if (kind == K_FUSED) e2 = launch_tbf16(C, sl->d_desc, d_items + b, (int32_t)cnt, head, dir, ops, ncg, blocks, s);
+            if (kind == K_FUSED && wv > 0) {          // its queue heads are the slot's counters
+                for (int p = 0; p < TierQueue::PARTS; ++p)
+                    if ((e2 = cudaMemsetAsync((int32_t *)sl->counters.ptr + CTR_HEAD + p * CTR_PART, 0,
+                                              sizeof(int32_t), s)) != cudaSuccess)
+                        return cuda_fail(ctx, e2, "clear queue heads");
+            }
+            if (kind == K_FUSED) e2 = launch_tbf16(C, sl->d_desc, d_items + b, (int32_t)cnt, dir, ops, ncg, blocks, s);
             else if (kind == K_16) e2 = launch_tb16(C, sl->d_desc, d_items + b, (int32_t)cnt, head, dir, ops, ncg, blocks, s);
             else e2 = launch_tb(C, sl->d_desc, d_items + b, (int32_t)cnt, head, dir, ops, ncg, blocks, s);
             if (e2 != cudaSuccess) return cuda_fail(ctx, e2, "traceback launch");

@@ -162,3 +162,32 @@ def test_local(ctx, name, w):
         got = ctx.align_local(A.pack_batch(batch), batch.scoring, h0)
         bad = A.results_equal(got, ref, O.COMPARE_FIELDS)
         assert bad.size == 0, (bad[:5], h0[bad[:5]], got[bad[:2]], ref[bad[:2]])
+
+
+@pytest.mark.parametrize("n", [1, 3, 151, 153, 607, 609, 1217, 1825, 2500])
+@pytest.mark.parametrize("w", [100, 200, 500, 750, 1000])
+def test_tiers(ctx, n, w):
+    """Batches that just fill a tier of the SMs' warps or not quite, with a few
+    pairs that bound the launch (whose later tiers stay away) or none, sorted
+    and unsorted: every pair is aligned once."""
+    from oracle import oracle as O
+    for long_ones in (0, min(n, 9)):
+        rng = np.random.default_rng(n + w + long_ones)
+        qs, ts = [], []
+        for i in range(n):
+            ql = int(rng.integers(30, 60)) if i >= long_ones else int(rng.integers(900, 1500))
+            q = rng.integers(0, 4, ql, dtype=np.uint8)
+            t, _ = W._mutate_chunk(rng, q, np.array([ql], np.int32), W.ErrorModel(0.05, 0.03, 0.03))
+            qs.append(q)
+            ts.append(t if len(t) else q)
+        batch = W.from_pairs(qs, ts, W.replace(TWO, w=w))
+        ref = O.align_batch(batch)
+        for flags in (0, A.AGATHA_FORCE32, A.AGATHA_NO_SORT):
+            got = A.agatha_align_batch(ctx, batch, flags=flags)
+            bad = A.results_equal(got, ref, O.COMPARE_FIELDS)
+            assert bad.size == 0, (flags, bad[:5])
+        if w < 768:
+            res, off, cig = ctx.align_cigar(A.pack_batch(batch), batch.scoring)
+            assert A.results_equal(res, ref, O.COMPARE_FIELDS).size == 0
+            want, _ = O.traceback_batch(batch, ref)
+            assert all(np.array_equal(cig[off[i]:off[i + 1]], want[i]) for i in range(n))
