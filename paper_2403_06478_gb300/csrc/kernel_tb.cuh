@@ -234,17 +234,20 @@ tb16_kernel(const DevBatch *__restrict__ d_batch, const TbItem *__restrict__ ite
 //
 // Each warp aligns a pair exactly as warp16_align_kernel does, on lazy blocks,
 // and keeps the band's state of every 32nd anti-diagonal in memory (TRACE).
-// Then it goes back over the segments between those states: it recomputes a
-// segment on the same lazy step, holds the scores of the 34 to 36 anti-diagonals
-// of the few lanes the path can reach in it in shared memory, and follows the
-// path through them.  No direction byte is computed or stored.
+// Then it goes back over the segments between those states: it recomputes the
+// 64 slots of a segment that the path can depend on by the same lazy step, two
+// slots per lane, holds their scores in shared memory and follows the path
+// through them.  No direction byte is computed or stored.
 //
-// What bounds it: the integer ALU pipe, twice the score kernel's work (and for
-// a few thousand pairs the longest one).  The form before wrote a direction
-// byte per cell from a step of 36 lane-instructions per cell (against 8 to 9 of
-// the lazy step, twice) and walked back through the table one cell at a time.
-// One GB300, kernel time: 20,000 ONT-like pairs 155 -> 95 ms, 2,000 56 -> 36
-// ms, 20,000 reads of 150 bp 2.4 -> 1.6 ms.
+// What bounds it: the score path's integer ALU pipe, and for a few thousand
+// pairs the longest one, whose 32 anti-diagonals of a segment take 4,500 clocks
+// (a chain of a shuffle and seven operations each) and the walk through them
+// 750 to 1,300.  The first form wrote a direction byte per cell from a step of
+// 36 lane-instructions per cell (against 8 to 9 of the lazy step) and walked
+// back through the table one cell at a time; the second kept states but took
+// every segment on the whole frame.  One GB300, kernel time of the three:
+// 20,000 ONT-like pairs 155, 95, 65 ms, 2,000 56, 29.6, 21.8, 20,000 of Pareto
+// lengths at w = 750 -, 94, 56, 20,000 reads of 150 bp 2.4, 1.11, 1.14.
 //
 // The path from scores alone (the rules at the top of this file): a diagonal
 // step is taken wherever H equals the diagonal's H plus the substitution, so
@@ -256,109 +259,204 @@ tb16_kernel(const DevBatch *__restrict__ d_batch, const TbItem *__restrict__ ite
 // Past the segment's start the state E (F, E2, F2) kept there stands for all
 // longer gaps: a gap that equals only that one continues in the segment
 // before, where the smallest l is looked for that opens it.
+// The scores of a segment's anti-diagonals on 64 slots around the path: a path
+// and the gaps from it move at most one slot per two anti-diagonals (39 slots
+// would hold them), and what the window's ends get wrong comes in as slowly.
 template <class S>
 struct TraceWin {
     static constexpr int C = S::P * 2, P = S::P;
-    // lanes that hold 39 neighbouring slots wherever they start: a path and
-    // the gaps from it move at most one slot per two anti-diagonals
-    static constexpr int NL = (39 + C - 1 + C - 1) / C;
     static constexpr int ROWS = 38;               // the first segment starts at -2
-    static constexpr int WORDS = NL * (ROWS + 4) * P + ROWS;
-    uint32_t *rows;                               // [lane - la][row][register]
-    uint32_t *st;                                 // [E, F, E2, F2][lane - la][register] leaving row rk
+    static constexpr int WORDS = 32 * (ROWS + 4) + ROWS;
+    uint32_t *rows;                               // [row][32], two slots per word
+    uint32_t *st;                                 // [E, F, E2, F2][32] leaving row rk
     int32_t *off;                                 // from a row's stored value to the score
-    int32_t la, rk, st_off;
+    int32_t jb, rk, st_off;                       // the window's first slot, even; the segment's start
     __device__ __forceinline__ explicit TraceWin(uint4 *mem)
-        : rows(reinterpret_cast<uint32_t *>(mem)), st(rows + NL * ROWS * P),
-          off(reinterpret_cast<int32_t *>(st + 4 * NL * P)) {}
+        : rows(reinterpret_cast<uint32_t *>(mem)), st(rows + 32 * ROWS), off(reinterpret_cast<int32_t *>(st + 4 * 32)) {}
+    __device__ __forceinline__ static int32_t at(const uint32_t *row, int32_t j) {
+        return reinterpret_cast<const uint16_t *>(row)[j];
+    }
     __device__ __forceinline__ int32_t score(const S &s, int32_t t, int32_t r) const {
-        const int32_t j = t - s.frame(r), local = j % C, i = r - rk + 1;
-        return S::half_of(rows[((j / C - la) * ROWS + i) * P + local % P], local) + off[i];
+        const int32_t i = r - rk + 1;
+        return at(rows + 32 * i, t - s.frame(r) - jb) + off[i];
     }
     // the gap state k (0 E, 1 F, 2 E2, 3 F2) leaving cell (t, rk - t)
     __device__ __forceinline__ int32_t state(const S &s, int k, int32_t t) const {
-        const int32_t j = t - s.frame(rk), local = j % C;
-        return S::half_of(st[k * (NL * P) + (j / C - la) * P + local % P], local) + st_off;
+        return at(st + 32 * k, t - s.frame(rk) - jb) + st_off;
     }
-    __device__ __forceinline__ void keep(const S &s, int32_t r, const uint32_t (&H)[P], int32_t o) {
-        const int32_t l = s.lane - la;
-        if (l >= 0 && l < NL) {
+    // the window's slots of a whole frame's registers
+    __device__ __forceinline__ void put(const S &s, uint32_t *row, const uint32_t (&x)[P]) const {
+        uint16_t *d = reinterpret_cast<uint16_t *>(row);
 #pragma unroll
-            for (int p = 0; p < P; ++p) rows[(l * ROWS + r - rk + 1) * P + p] = H[p];
+        for (int p = 0; p < P; ++p) {
+            const int32_t lo = s.j0 + p - jb, hi = lo + P;
+            if ((uint32_t)lo < 64u) d[lo] = (uint16_t)x[p];
+            if ((uint32_t)hi < 64u) d[hi] = (uint16_t)(x[p] >> 16);
         }
+    }
+    __device__ __forceinline__ void keep(const S &s, int32_t r, const uint32_t (&H)[P], int32_t o) const {
+        put(s, rows + 32 * (r - rk + 1), H);
         if (s.lane == 0) off[r - rk + 1] = o;
     }
 };
 
+// This lane's two slots of the six arrays of state `entry`: neighbouring
+// registers p, p + 1 of lane a / C, the same half of both.
+template <class S>
+__device__ __forceinline__ void trace_gather(const S &s, const TraceWin<S> &W, const uint4 *entry, uint32_t (&x)[6]) {
+    constexpr int P = S::P, C = S::P * 2;
+    const int32_t a = W.jb + 2 * s.lane, local = a % C, p = local % P;
+    const uint32_t sel = local < P ? 0x5410u : 0x7632u;
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+        const int32_t word = i * P + p;
+        const uint2 v = *reinterpret_cast<const uint2 *>(
+            reinterpret_cast<const uint32_t *>(entry + (word >> 2) * 32 + a / C) + (word & 3));
+        x[i] = prmt(v.x, v.y, sel);
+    }
+}
+// n pairs of anti-diagonals after rk on the window alone, from the arrays x
+// (H of rk - 1 and rk, E, F, E2, F2; drifting since rs): the lazy step
+// (WarpPair16::lazy_step) with two slots per lane.  The cuts at slots 0 and
+// w + 1 act where the window holds them; at its other ends garbage enters, one
+// slot per two anti-diagonals.  Cells past the table's last row and column
+// come out wrong and feed none of the table's.
+template <class S, bool TWO>
+__device__ __forceinline__ void trace_narrow(const S &s, TraceWin<S> &W, const uint32_t (&x)[6], int32_t rk, int32_t rs,
+                                             int32_t n, const typename S::LazyConst &k) {
+    const int32_t a = W.jb + 2 * s.lane, w1 = s.w + 1 - a, lane = s.lane;
+    uint32_t Hev = x[0], Hod = x[1], Eo = x[2], Fo = x[3], E2o = x[4], F2o = x[5];
+    const uint32_t NEG = s.NEGp;
+    const uint32_t low = a == 0 ? 0x0000ffffu : 0u;                      // slot 0
+    const uint32_t top = w1 == 0 ? 0x0000ffffu : (w1 == 1 ? 0xffff0000u : 0u);   // slot w + 1
+    const uint32_t past = lane == 31 && w1 == 2 ? 0xffff0000u : 0u;      // it would come in next
+    const int32_t B = s.frame(rk), tb = B + a + s.tph, qb = rk - B - a + s.qph + 1;    // (see lazy_windows)
+    uint32_t t0 = load_rel(s.tp, s.tspan, tb), t1 = load_rel(s.tp, s.tspan, tb + 16);
+    uint32_t q0 = rev2_32(load_rel(s.qp, s.qspan, qb)), q1 = rev2_32(load_rel(s.qp, s.qspan, qb - 16));
+    uint32_t *row = W.rows + 32 * (rk - W.rk) + lane;
+    const int32_t d = s.lazy_drift();
+    if (rk == W.rk) {
+        row[0] = Hev;
+        row[32] = Hod;
+        W.st[lane] = Eo;
+        W.st[32 + lane] = Fo;
+        W.st[64 + lane] = TWO ? E2o : Eo;
+        W.st[96 + lane] = TWO ? __vmaxu2(F2o, Hod) : Fo;
+        W.st_off = s.base - s.OFF - d * (rk + 1 - rs);
+        if (lane < 2) W.off[lane] = s.lazy_off() - d * (rk - 1 + lane - rs);
+    }
+    if (lane < 2 * n) W.off[rk - W.rk + 2 + lane] = s.lazy_off() - d * (rk + 1 + lane - rs);
+    const auto score = [&](uint32_t Hd, uint32_t E, uint32_t F, uint32_t E2, uint32_t F2, uint32_t &hoe) {
+        const uint32_t m = t0 ^ q1, mb = (((m | (m >> 1)) & 5u) * 0x4001u) & 0x10001u;
+        const uint32_t X = __viaddmax_u16x2(mb * s.NABs + Hd, k.A, E);
+        const uint32_t H = TWO ? __vmaxu2(__vimax3_u16x2(X, F, E2), F2) : __vmaxu2(X, F);
+        hoe = H - k.OE;
+        return H - k.H2;
+    };
+#pragma unroll 1
+    for (; n > 0; --n) {
+        row += 64;
+        t0 = __funnelshift_r(t0, t1, 2);
+        t1 >>= 2;
+        uint32_t F = mux(past, NEG, prmt(Fo, __shfl_down_sync(FULL, Fo, 1), 0x5432)), F2 = 0, hoe;
+        if constexpr (TWO) {
+            const uint32_t y = __vmaxu2(F2o, Hod);
+            F2 = mux(past, NEG, prmt(y, __shfl_down_sync(FULL, y, 1), 0x5432));
+        }
+        Hev = score(Hev, Eo, F, E2o, F2, hoe);
+        Eo = TWO ? __viaddmax_u16x2(Eo, k.NE, hoe) : __vmaxu2(Eo, Hev);
+        Fo = TWO ? __viaddmax_u16x2(F, k.NE, hoe) : __vmaxu2(F, Hev);
+        if constexpr (TWO) F2o = __vmaxu2(F2, Hev);
+        row[0] = Hev;
+        q1 = __funnelshift_l(q0, q1, 2);
+        q0 <<= 2;
+        uint32_t E = prmt(__shfl_up_sync(FULL, Eo, 1), Eo, 0x5432), E2 = 0;
+        if constexpr (TWO) {
+            const uint32_t y = __vmaxu2(E2o, Hev);
+            E2 = prmt(__shfl_up_sync(FULL, y, 1), y, 0x5432);
+        }
+        Hod = score(Hod, E, Fo, E2, F2o, hoe);
+        Eo = mux(low, NEG, TWO ? __viaddmax_u16x2(E, k.NE, hoe) : __vmaxu2(E, Hod));
+        Fo = mux(top, NEG, TWO ? __viaddmax_u16x2(Fo, k.NE, hoe) : __vmaxu2(Fo, Hod));
+        if constexpr (TWO) {
+            E2o = mux(low, NEG, __vmaxu2(E2, Hod));
+            F2o = mux(top, NEG, F2o);
+            Hod = mux(top, NEG, Hod);
+        }
+        row[32] = Hod;
+    }
+}
+
 // Recompute anti-diagonals rk + 1 .. target (or one more) from state seg into
-// the window.
+// the window: on its own slots, after the masked step on the whole frame at
+// the table's corner and where the virtual cells leave the band.
 template <class S>
 __device__ __forceinline__ void trace_segment(S &s, TraceWin<S> &W, int32_t seg, int32_t target,
-                                              const typename S::LazyConst &k, bool two, bool head, int32_t end) {
-    using TW = TraceWin<S>;
+                                              const typename S::LazyConst &k, bool two, bool head) {
     constexpr int P = S::P;
-    const int32_t w = s.w, d = s.lazy_drift();
-    const int32_t turn = s.cover ? INT_MAX : w - 3;
-    int32_t r, rs = 0;
-    bool drifting = false;
+    const int32_t w = s.w, turn = !head ? 0 : (s.cover ? INT_MAX : w - 3);
+    const auto runs_lazy = [&](int32_t r) { return r > w || ((target - r + 1) & ~1) <= turn - r; };
+    int32_t r = -3, rs = 0;
+    uint32_t x[6];
+    bool drifting = false, narrow = false;
     if (seg == 0) {
 #pragma unroll
         for (int p = 0; p < P; ++p)
             s.Hev[p] = s.Hod[p] = s.Eo[p] = s.E2o[p] = s.Fo[p] = s.F2o[p] = s.NEGp;
         s.base = 0;
-        r = -3;
     } else {
         r = W.rk;
-        drifting = s.trace_load(seg, rs);
-        if (!drifting) {
-            s.lazy_enter(k, two);
-            rs = r;
-            drifting = true;
-        }
-        W.keep(s, r - 1, s.Hev, s.lazy_off() - d * (r - 1 - rs));
-        W.keep(s, r, s.Hod, s.lazy_off() - d * (r - rs));
-        W.st_off = s.base - s.OFF - d * (r + 1 - rs);
-        const int32_t l = s.lane - W.la;
-        if (l >= 0 && l < TW::NL) {
-#pragma unroll
-            for (int p = 0; p < P; ++p) {
-                W.st[l * P + p] = s.Eo[p];
-                W.st[TW::NL * P + l * P + p] = s.Fo[p];
-                W.st[2 * TW::NL * P + l * P + p] = two ? s.E2o[p] : s.Eo[p];
-                W.st[3 * TW::NL * P + l * P + p] = two ? __vmaxu2(s.F2o[p], s.Hod[p]) : s.Fo[p];
-            }
+        drifting = s.trace_meta(seg, rs);
+        narrow = __any_sync(FULL, runs_lazy(r));
+        if (narrow) {
+            trace_gather(s, W, s.trace_entry(seg), x);
+        } else {
+            s.trace_load(seg);
+            if (drifting) s.lazy_leave(k, two, r - rs);
+            drifting = false;
+            W.keep(s, r - 1, s.Hev, s.base - s.OFF);
+            W.keep(s, r, s.Hod, s.base - s.OFF);
+            W.put(s, W.st, s.Eo);
+            W.put(s, W.st + 32, s.Fo);
+            W.put(s, W.st + 64, s.E2o);
+            W.put(s, W.st + 96, s.F2o);
+            W.st_off = s.base - s.OFF;
         }
     }
-    while (r < target) {
-        // the lazy step wherever it holds (lazy_drive), else the masked one
-        const int32_t limit = r <= w ? (head ? min(turn, end) : INT_MIN) : end;
-        if (r >= s.first_r() && ((r - w) & 1) && limit >= r + 2) {
-            if (!drifting) {
-                s.lazy_enter(k, two);
-                rs = r;
-                drifting = true;
-            }
-            const int32_t n = min((min(target + 1, limit) - r) >> 1, LAZY_PAIRS);
-            typename S::LazyWin B;
-            s.lazy_windows(B, r);
-            const int32_t l = s.lane - W.la;
-            const bool in = l >= 0 && l < TW::NL;
-            const uint32_t *first = W.rows + ((in ? l : 0) * TW::ROWS + r + 1 - W.rk + 1) * P;
-            LazyEdge g{__reduce_max_sync(FULL, 1), in ? 0 : -1, -(1 << 20),
-                       (uint32_t)__cvta_generic_to_shared(first), 0};
-            if (two) s.template lazy_block<true>(n, B, k, g);
-            else s.template lazy_block<false>(n, B, k, g);
-            if (s.lane < 2 * n) W.off[r + 1 + s.lane - W.rk + 1] = s.lazy_off() - d * (r + 1 + s.lane - rs);
-            r += 2 * n;
-        } else {
-            if (drifting) {
-                s.lazy_leave(k, two, r - rs);
-                drifting = false;
+    if (!narrow) {
+        while (r < target) {
+            if (r >= s.first_r() && ((r - w) & 1) && r + 6 <= target && runs_lazy(r)) {
+                uint32_t *tmp = W.rows + 32 * (r - W.rk + 2);      // six of the rows to come
+                __syncwarp();
+                W.put(s, tmp, s.Hev);
+                W.put(s, tmp + 32, s.Hod);
+                W.put(s, tmp + 64, s.Eo);
+                W.put(s, tmp + 96, s.Fo);
+                W.put(s, tmp + 128, s.E2o);
+                W.put(s, tmp + 160, s.F2o);
+                __syncwarp();
+#pragma unroll
+                for (int i = 0; i < 6; ++i) x[i] = tmp[32 * i + s.lane];
+                __syncwarp();
+                narrow = true;
+                break;
             }
             ++r;
             s.masked_step(r);
             W.keep(s, r, ((r - w) & 1) ? s.Hod : s.Hev, s.base - s.OFF);
         }
+    }
+    if (__any_sync(FULL, narrow)) {
+        if (!drifting) {                             // as lazy_enter
+            x[0] -= k.H2 + k.D;
+            x[1] -= k.H2;
+#pragma unroll
+            for (int i = 2; i < 6; ++i) x[i] += k.D;
+            rs = r;
+        }
+        const int32_t n = (target - r + 1) >> 1;
+        if (two) trace_narrow<S, true>(s, W, x, r, rs, n, k);
+        else trace_narrow<S, false>(s, W, x, r, rs, n, k);
     }
     __syncwarp();
 }
@@ -373,8 +471,6 @@ __device__ __forceinline__ int32_t tb_trace(S &s, uint32_t *ops, int32_t cap) {
     const int32_t w = s.w, g0 = s.first_r(), lane = s.lane;
     const bool two = prm.q2 != prm.q || prm.e2 != prm.e;
     const bool head = __any_sync(FULL, w >= 8 && s.lazy_head_ok());
-    const int32_t L = min(s.tlen, s.qlen);
-    const int32_t end = abs(s.tlen - s.qlen) <= w ? s.last_r - 1 : max(L - 2, 2 * L - 3 - w);
     const auto k = s.lazy_consts(two);
     s.blind = true;
     s.ovf = false;
@@ -384,8 +480,8 @@ __device__ __forceinline__ int32_t tb_trace(S &s, uint32_t *ops, int32_t cap) {
         const int32_t rc = t + q;
         const int32_t seg = rc <= g0 + 32 ? 0 : (rc - g0 - 1) >> 5;
         W.rk = seg ? g0 + 32 * seg : -2;
-        W.la = min(max(t - s.frame(rc) - 19, 0) / TW::C, 32 - TW::NL);
-        trace_segment(s, W, seg, rc, k, two, head, end);
+        W.jb = min(max(t - s.frame(rc) - 32, 0) & ~1, S::NS - 64);
+        trace_segment(s, W, seg, rc, k, two, head);
         while (t >= 0 && q >= 0 && t + q > W.rk) {
             int32_t r = t + q;
             if (kind < 0) {

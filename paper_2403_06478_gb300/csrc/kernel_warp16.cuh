@@ -1394,8 +1394,16 @@ struct WarpPair16 {
                 make_uint4(lazy_word(4 * i), lazy_word(4 * i + 1), lazy_word(4 * i + 2), lazy_word(4 * i + 3));
         if (lane == 0) d[CKV * 32] = make_uint4((uint32_t)rs, (uint32_t)base, drifting ? 1u : 0u, 0u);
     }
-    // Load state k; returns whether it is in the drifting form.
-    __device__ __forceinline__ bool trace_load(int32_t k, int32_t &rs) {
+    // State k's base and start of the drift; returns whether it is in the
+    // drifting form.
+    __device__ __forceinline__ bool trace_meta(int32_t k, int32_t &rs) {
+        uint4 m = make_uint4(0x80000000u, 0x80000000u, 0u, 0u);
+        if (lane == 0) m = trace_entry(k)[CKV * 32];
+        rs = __reduce_max_sync(FULL, (int32_t)m.x);
+        base = __reduce_max_sync(FULL, (int32_t)m.y);
+        return __any_sync(FULL, m.z != 0u);
+    }
+    __device__ __forceinline__ void trace_load(int32_t k) {
         const uint4 *d = trace_entry(k);
 #pragma unroll
         for (int i = 0; i < CKV; ++i) {
@@ -1405,11 +1413,6 @@ struct WarpPair16 {
             lazy_word(4 * i + 2) = v.z;
             lazy_word(4 * i + 3) = v.w;
         }
-        uint4 m = make_uint4(0x80000000u, 0x80000000u, 0u, 0u);
-        if (lane == 0) m = d[CKV * 32];
-        rs = __reduce_max_sync(FULL, (int32_t)m.x);
-        base = __reduce_max_sync(FULL, (int32_t)m.y);
-        return __any_sync(FULL, m.z != 0u);
     }
 
     // What lazy_drive asks of the lanes.
