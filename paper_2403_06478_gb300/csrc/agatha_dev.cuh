@@ -350,6 +350,7 @@ struct TierQueue {
             v = (v & ~3) | to;
         }
     }
+    __device__ __forceinline__ static bool had(int32_t place) { return (place & 16) != 0; }      // a pair
     __device__ __forceinline__ static int32_t first_place(int32_t tier) { return start(tier) * 5; }
 };
 
@@ -388,8 +389,9 @@ struct TbItem {
 };
 
 // Launchers (defined in the .cu files).
-cudaError_t launch_prep(const DevBatch *d_batch, int64_t n_pairs, int32_t sort, cudaStream_t s,
-                        int n_sm);
+cudaError_t launch_prep(const DevBatch *d_batch, int64_t n_pairs, int32_t sort, int32_t *counters, int64_t *hist,
+                        cudaStream_t s, int n_sm);
+inline bool prep_small(int64_t n_pairs) { return n_pairs <= 4096; }      // one launch does it all
 // The int32 kernel with C slots per lane; K warps share a pair's band (1 or 3).
 template <int C, int K = 1>
 cudaError_t launch_warp_c(const DevBatch *d_batch, int n_blocks, cudaStream_t s, int use_fast,

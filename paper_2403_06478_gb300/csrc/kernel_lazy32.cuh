@@ -640,6 +640,7 @@ warp_align_kernel(const DevBatch *__restrict__ d_batch, int32_t use_fast, int32_
     const bool asks = lane == 0 && wk == 0;
     const WorkList L = work_list(B, list);
     const int32_t l_end = __reduce_max_sync(FULL, L.end);
+    if (list == WARP_LIST_OVERFLOW && l_end == 0) return;        // nearly always
     if (threadIdx.x == 0) q.open(L.head, L.begin, l_end, U * (int32_t)gridDim.x);
     if (asks) place[g] = q.first_place(tier);
     __syncthreads();
@@ -671,7 +672,7 @@ warp_align_kernel(const DevBatch *__restrict__ d_batch, int32_t use_fast, int32_
         }
         if (asks) k = q.next(place[g]);
     }
-    if (lane == 0) mark_step_end(B.counters);
+    if (asks && (q.had(place[g]) || blockIdx.x == 0)) mark_step_end(B.counters);
 }
 
 template <int C, int K>

@@ -1839,6 +1839,7 @@ warp16_align_kernel(const DevBatch *__restrict__ d_batch, int32_t use_fast, int3
             }
             if (lane == 0) k = q.next(place[warp]);
         }
+        if (lane == 0 && (q.had(place[warp]) || blockIdx.x == 0)) mark_step_end(B.counters);
     } else {
         using Pair = WarpPair16<C, MINB < 4, true, false, 1, true, true, G>;
         // The warp takes two neighbouring pairs of the longest-first queue at
@@ -1863,8 +1864,8 @@ warp16_align_kernel(const DevBatch *__restrict__ d_batch, int32_t use_fast, int3
             }
             __syncwarp();
         }
+        if (lane == 0) mark_step_end(B.counters);
     }
-    if (lane == 0) mark_step_end(B.counters);
 }
 
 // K warps of a block share one pair's band (K = 2: two pairs per block at a

@@ -73,9 +73,8 @@ extern "C" int agatha_align_batch_local(agatha_ctx *ctx, const agatha_batch *bat
     if ((rc = stage_batch(ctx, batch, p, out, flags, s, lp, d_h0))) return rc;
     Slot *sl = &ctx->main;
     const DevBatch *d = sl->d_desc;
-    if ((e = cudaMemsetAsync(sl->counters.ptr, 0, CTR_COUNT * sizeof(int32_t), s)) != cudaSuccess ||
-        (e = cudaMemsetAsync(sl->hist.ptr, 0, 256 * sizeof(int64_t), s)) != cudaSuccess ||
-        (e = launch_prep(d, n, lp.sort, s, ctx->n_sm)) != cudaSuccess)
+    if ((e = launch_prep(d, n, lp.sort, (int32_t *)sl->counters.ptr, (int64_t *)sl->hist.ptr, s, ctx->n_sm)) !=
+        cudaSuccess)
         return cuda_fail(ctx, e, "prep");
     if (ctx->timing && (e = cudaEventRecord(ctx->ev_k0, s)) != cudaSuccess) return cuda_fail(ctx, e, "event");
     if ((e = launch_local(lp.C, d, ctx->n_sm, s)) != cudaSuccess)

@@ -134,9 +134,8 @@ extern "C" int agatha_align_batch_noalloc(const agatha_batch *batch, const agath
 
     // the array keeps the previous call's contents: reset what must start at zero
     cudaError_t e = cudaMemcpyAsync((void *)d_desc, &desc, sizeof(desc), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(desc.counters, 0, CTR_COUNT * sizeof(int32_t), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(desc.bucket_hist, 0, 256 * sizeof(int64_t), s);
-    if (e == cudaSuccess) e = launch_prep(d_desc, batch->n_pairs, 1, s, ds->n_sm);
+    if (e == cudaSuccess)
+        e = launch_prep(d_desc, batch->n_pairs, 1, desc.counters, desc.bucket_hist, s, ds->n_sm);
     if (e == cudaSuccess) e = launch_warp32(shape, d_desc, blocks, s, 1, WARP_LIST_MAIN);
     if (e == cudaSuccess && wide_w > 0) e = launch_plain_kernel(d_desc, (int64_t)ds->n_sm * 2, wide_w, 1, s);
     int32_t ctr[CTR_COUNT] = {0};

@@ -273,14 +273,9 @@ static cudaError_t enqueue_part(agatha_ctx *ctx, Slot *sl, const LaunchPlan &lp,
     cudaError_t e = cudaSuccess;
     const DevBatch *d = sl->d_desc;
     if (part == 0) {
-        e = cudaMemsetAsync(sl->counters.ptr, 0, CTR_COUNT * sizeof(int32_t), s);
-        if (e != cudaSuccess) return e;
-        if (!lp.plain) {
-            e = cudaMemsetAsync(sl->hist.ptr, 0, 256 * sizeof(int64_t), s);
-            if (e != cudaSuccess) return e;
-        }
         // the plain path only validates (no sort); the batched path also orders
-        return launch_prep(d, lp.n, lp.plain ? 0 : lp.sort, s, ctx->n_sm);
+        return launch_prep(d, lp.n, lp.plain ? 0 : lp.sort, (int32_t *)sl->counters.ptr,
+                           lp.plain ? nullptr : (int64_t *)sl->hist.ptr, s, ctx->n_sm);
     }
     if (lp.plain) return launch_plain_kernel(d, lp.plain_blocks, lp.plain_w, 0, s);
     bool any16 = false;

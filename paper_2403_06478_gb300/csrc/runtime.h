@@ -98,7 +98,8 @@ struct LaunchPlan {
     int32_t plain_w = 0;
     int64_t plain_blocks = 0;
     PlanKey key() const {
-        return {plain, C | (shape32.C << 8) | (shape32.K << 16), C16 * lane16, regs_high, sort, fast, wide_w, warp_blocks, split,
+        return {plain, C | (shape32.C << 8) | (shape32.K << 16), C16 * lane16, regs_high,
+                sort | (prep_small(n) ? 2 : 0), fast, wide_w, warp_blocks, split,
                 split ? cls_var[0] | (cls_var[1] << 4) | (cls_var[2] << 8) | (cls_var[3] << 12) : 0,
                 split ? 1 : groupk, (split ? 0 : half) | (narrow_w > 0 ? 2 : 0)};
     }
