@@ -450,6 +450,17 @@ int slot_ensure(agatha_ctx *ctx, Ledger &ledger, Slot *sl, int64_t n, int64_t q_
     return AGATHA_OK;
 }
 
+// A kernel's resident blocks per SM, asked of the runtime once per context
+// (which also lets the kernel have its shared memory): a plan asks for five,
+// 10 us of a call of 115.
+template <class Ask>
+static int plan_occupancy(agatha_ctx *ctx, int kind, int i, Ask ask) {
+    std::atomic<int> &c = ctx->occupancy[kind][i];
+    int v = c.load(std::memory_order_relaxed);
+    if (v == 0) c.store(v = ask() + 1, std::memory_order_relaxed);
+    return v - 1;
+}
+
 // Build the launch plan of a batch: which kernels, grids and graph key.
 int make_plan(agatha_ctx *ctx, const DevParams &p, const BatchShape &shape, uint32_t flags,
               LaunchPlan *lp) {
@@ -478,7 +489,9 @@ int make_plan(agatha_ctx *ctx, const DevParams &p, const BatchShape &shape, uint
         return set_error(ctx, AGATHA_ENOTSUP, "band of %d cells is wider than supported (%d)",
                          lp->wide_w, pmax);
     lp->shape32 = pick_shape32(std::min(shape.max_w_all, lp->warp_w_max));
-    lp->warp_blocks = ctx->n_sm * warp32_occupancy(lp->shape32);
+    const Shape32 s32 = lp->shape32;
+    lp->warp_blocks = ctx->n_sm * plan_occupancy(ctx, 0, s32.K == 1 ? s32.C / 4 : (s32.C == 8 ? 5 : 6),
+                                                 [&] { return warp32_occupancy(s32); });
     // 16-bit packed lanes when the band fits and one anti-diagonal changes a
     // score by at most 255 (the 16-bit kernel then still rebases at least
     // every 50 anti-diagonals)
@@ -491,10 +504,12 @@ int make_plan(agatha_ctx *ctx, const DevParams &p, const BatchShape &shape, uint
     lp->warp16h_blocks = 0;
     if (lp->lane16) {
         lp->warp_w_max = 32 * lp->C16 - 1;
-        lp->warp16_blocks[0] = ctx->n_sm * warp16_occupancy(lp->C16, 0);
-        lp->warp16_blocks[1] = ctx->n_sm * warp16_occupancy(lp->C16, 1);
-        lp->warp16k_blocks[0] = ctx->n_sm * warp16k_occupancy(lp->C16, 2);
-        lp->warp16k_blocks[1] = ctx->n_sm * warp16k_occupancy(lp->C16, 4);
+        const int C16 = lp->C16;
+        const auto blocks = [&](int kind, auto ask) { return ctx->n_sm * plan_occupancy(ctx, kind, C16 / 4, ask); };
+        lp->warp16_blocks[0] = blocks(1, [&] { return warp16_occupancy(C16, 0); });
+        lp->warp16_blocks[1] = blocks(2, [&] { return warp16_occupancy(C16, 1); });
+        lp->warp16k_blocks[0] = blocks(3, [&] { return warp16k_occupancy(C16, 2); });
+        lp->warp16k_blocks[1] = blocks(4, [&] { return warp16k_occupancy(C16, 4); });
         const int K = (flags & AGATHA_WARPS4) ? 4 : ((flags & AGATHA_WARPS2) ? 2 : 1);
         if (K > 1 && (flags & AGATHA_HALF_WARP))
             return set_error(ctx, AGATHA_EINVAL, "two pairs per warp and several warps per pair");
@@ -503,7 +518,7 @@ int make_plan(agatha_ctx *ctx, const DevParams &p, const BatchShape &shape, uint
                 return set_error(ctx, AGATHA_ENOTSUP, "%d warps per pair need a band of 256 to 767", K);
             lp->groupk = K;
         }
-        lp->warp16h_blocks = ctx->n_sm * warp16h_occupancy(lp->C16);
+        lp->warp16h_blocks = blocks(5, [&] { return warp16h_occupancy(C16); });
         if (flags & AGATHA_HALF_WARP) {
             if (!lp->warp16h_blocks)
                 return set_error(ctx, AGATHA_ENOTSUP, "two pairs per warp need a band of at most 127");
@@ -525,7 +540,7 @@ void apply_narrow(agatha_ctx *ctx, LaunchPlan *lp, uint32_t flags) {
     if ((flags & AGATHA_ONE_FRAME) || !lp->lane16 || lp->plain || !lp->sort || lp->split || lp->groupk != 1 ||
         lp->half || lp->wide_w || lp->C16 != 24)
         return;
-    const int occ = occupancy_warp16_c<20, 2>();
+    const int occ = plan_occupancy(ctx, 1, 20 / 4, [] { return occupancy_warp16_c<20, 2>(); });
     if (occ <= 0) return;
     lp->narrow_w = 32 * 20 - 2;
     lp->narrow_blocks = ctx->n_sm * occ;

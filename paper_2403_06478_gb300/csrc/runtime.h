@@ -1,6 +1,7 @@
 // Host-side internals of the library (not part of the C ABI).
 #pragma once
 
+#include <atomic>
 #include <array>
 #include <condition_variable>
 #include <cstdint>
@@ -189,6 +190,8 @@ struct agatha_ctx {
     agatha::Ledger ledger;
     std::string tune_cache_path;
     std::mutex mu;                     // serialises align_batch calls
+    // resident blocks of each kernel + 1 (0: not asked yet), see plan_occupancy
+    std::atomic<int> occupancy[6][8] = {};
     std::mutex err_mu;
     std::string last_error, last_error_copy;
     agatha::Slot main;                 // buffers of agatha_align_batch

@@ -17,7 +17,6 @@
 //    input order; a gather kernel reverses each pair's runs into one dense
 //    device array, copied to the caller's buffer in one transfer.
 #include <algorithm>
-#include <numeric>
 #include <vector>
 
 #include "runtime.h"
@@ -199,41 +198,42 @@ extern "C" int agatha_align_cigar(agatha_ctx *ctx, const agatha_batch *batch, co
         ctx->timed_once = true;
     }
 
+    const auto item_of = [&](int64_t i) {
+        const int32_t tl = batch->t_len[i], ql = batch->q_len[i];
+        TbItem it{(int32_t)i, tl - 1, ql - 1, 0, 0, 0};
+        if (!fused) {
+            const agatha_result &r = out[i];
+            it.end_t = r.reach_end ? r.mqe_t : r.te;
+            it.end_q = r.reach_end ? ql - 1 : r.qe;
+        }
+        return it;
+    };
+    constexpr int NO_ITEM = 255;
+
     // 2. items, longest predicted work first.  A fused item covers every
     //    anti-diagonal of its pair (its end is found on the way); a two-pass
     //    item ends at its end cell.
+    //    (a counting sort by quarters of an octave, as the score path's order)
     std::vector<TbItem> items;
-    items.reserve((size_t)n);
-    for (int64_t i = 0; i < n; ++i) {
-        const int32_t tl = batch->t_len[i], ql = batch->q_len[i];
-        if (tl <= 0 || ql <= 0) continue;
-        int32_t et = tl - 1, eq = ql - 1;
-        if (!fused) {
-            const agatha_result &r = out[i];
-            et = r.reach_end ? r.mqe_t : r.te;
-            eq = r.reach_end ? ql - 1 : r.qe;
-            if (et < 0 || eq < 0) continue;             // the maximum is the origin: empty CIGAR
+    {
+        std::vector<uint8_t> bucket((size_t)n, NO_ITEM);
+        int64_t at[NO_ITEM + 1] = {0};
+        for (int64_t i = 0; i < n; ++i) {
+            if (batch->t_len[i] <= 0 || batch->q_len[i] <= 0) continue;
+            const TbItem it = item_of(i);
+            if (it.end_t < 0 || it.end_q < 0) continue;     // the maximum is the origin: empty CIGAR
+            const int32_t w = effective_w(p.w, batch->t_len[i], batch->q_len[i]);
+            const uint64_t est = ((uint64_t)it.end_t + it.end_q + 1) * (uint64_t)(w + 1);
+            const int lg = 63 - __builtin_clzll(est);
+            bucket[(size_t)i] = (uint8_t)(NO_ITEM - 1 - (4 * lg + (lg >= 2 ? (int)(est >> (lg - 2) & 3) : 0)));
+            ++at[bucket[(size_t)i] + 1];
         }
-        TbItem it;
-        it.pair = (int32_t)i; it.end_t = et; it.end_q = eq; it.pad = 0;
-        it.dir_off = 0; it.ops_off = 0;
-        items.push_back(it);
+        for (int k = 0; k < NO_ITEM; ++k) at[k + 1] += at[k];
+        items.resize((size_t)at[NO_ITEM]);
+        for (int64_t i = 0; i < n; ++i)
+            if (bucket[(size_t)i] != NO_ITEM) items[(size_t)at[bucket[(size_t)i]]++] = item_of(i);
     }
     const int64_t n_items = (int64_t)items.size();
-    {
-        std::vector<int64_t> key((size_t)n_items);
-        for (int64_t k = 0; k < n_items; ++k) {
-            const TbItem &it = items[k];
-            const int32_t w = effective_w(p.w, batch->t_len[it.pair], batch->q_len[it.pair]);
-            key[k] = ((int64_t)it.end_t + it.end_q + 1) * (w + 1);
-        }
-        std::vector<int64_t> ord((size_t)n_items);
-        std::iota(ord.begin(), ord.end(), 0);
-        std::stable_sort(ord.begin(), ord.end(), [&](int64_t a, int64_t b) { return key[a] > key[b]; });
-        std::vector<TbItem> sorted((size_t)n_items);
-        for (int64_t k = 0; k < n_items; ++k) sorted[k] = items[ord[k]];
-        items.swap(sorted);
-    }
     int64_t ops_total = 0;
     for (TbItem &it : items) {
         it.ops_off = ops_total;
