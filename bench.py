@@ -111,7 +111,7 @@ def traffic_tb16(kernel, table_bytes):
     with open(path) as fh:
         d = json.load(fh)
     if d.get("kernel") != kernel or d.get("kernel_digest") != _kernel_digest(
-            ("kernel_tb.cuh", "kernel_warp16.cuh", "kernel_warp16_c16.cu", "agatha_dev.cuh")):
+            ("kernel_tb.cuh", "kernel_warp16.cuh", "lazy_drive.cuh", "kernel_warp16_c16.cu", "agatha_dev.cuh")):
         return None
     return int(d["dram_bytes_per_table_byte"] * table_bytes)
 
@@ -121,7 +121,7 @@ def _kernel_digest(files=None):
     for the build it was measured on."""
     import hashlib
     h = hashlib.sha256()
-    for f in files or ("kernel_warp16.cuh", "kernel_warp16_c4.cu", "kernel_warp16_c8.cu",
+    for f in files or ("kernel_warp16.cuh", "lazy_drive.cuh", "kernel_warp16_c4.cu", "kernel_warp16_c8.cu",
                        "kernel_warp16_c16.cu", "kernel_warp16_c24.cu", "agatha_dev.cuh"):
         with open(os.path.join(ROOT, "paper_2403_06478_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
@@ -362,7 +362,7 @@ def run_local(args):
         "e2e": {"value": round(all_cells * args.steps / (e2e_tot / 1e3) / 1e9, 3), "unit": "GCUPS",
                 "h2d_bytes_per_step": int(pin_pb.nbytes() + 4 * n), "d2h_bytes_per_step": int(n * 48 + 64),
                 "ms_per_step": round(e2e_tot / args.steps, 3)},
-        "gpu_launches": args.steps * 4,          # prep classify / scan / scatter, local kernel
+        "gpu_launches": args.steps * ((1 if n <= 4096 else 3) + 2),      # prep, the local kernels
         "roofline": {"bound": "alu", "achieved": round(achieved, 3), "peak": round(int_peak, 3),
                      "unit": "Tops/s", "frac": round(achieved / int_peak, 4), "traffic": None,
                      "kernel": f"local_align_kernel<{C}>", "kernel_ms": round(t_ms, 3),
@@ -470,7 +470,7 @@ def run_traceback(args):
     units = cells if fused else tcells
     achieved = units * ops_cell / (t_ms / 1e3) / 1e12
     w = batch.scoring.w
-    minb = dict([(4, 6), (8, 4), (16, 3), (24, 2)])
+    minb = {4: 4, 8: 3, 16: 2, 24: 2} if fused else {4: 6, 8: 4, 16: 3, 24: 2}
     nonempty = (batch.t_len > 0) & (batch.q_len > 0)
     if packed:
         C = next(c for c in (4, 8, 16, 24) if 32 * c - 1 >= w)
@@ -504,9 +504,10 @@ def run_traceback(args):
                 "h2d_bytes_per_step": int(pin_pb.nbytes()),
                 "d2h_bytes_per_step": int(n * 48 + 4 * n + 4 * int(off[-1])),
                 "ms_per_step": round(wall_tot / args.steps, 3)},
-        # score path (prep 3, 16-bit kernel, overflow kernel), one traceback
-        # launch per wave, the CIGAR gather
-        "gpu_launches": args.steps * (5 + info["waves"] + 1),
+        # one traceback launch per wave, the overflow kernel and the CIGAR
+        # gather; of the two-pass form the score path before (prep and 16-bit
+        # kernel)
+        "gpu_launches": args.steps * (info["waves"] + 2 + (0 if fused else (1 if n <= 4096 else 3) + 1)),
         "traceback_pairs": {"lanes16": info["pairs16"], "int32": info["pairs32"], "waves": info["waves"],
                             "fused": info["fused"]},
         "roofline": {"bound": "alu", "achieved": round(achieved, 3), "peak": round(int_peak, 3),
@@ -676,21 +677,21 @@ def main():
     ops = cells16 * OPS_PER_CELL_I16X2 + (cells - cells16) * OPS_PER_CELL_I32
     achieved = ops / (k_ms / 1e3) / 1e12
     # the kernel the (tuned) plan launches: slots per lane from the band, the
-    # resident blocks per SM from the register budget the tuner chose
+    # warps per scheduler from the register budget the tuner chose
     w = batch.scoring.w
     c16 = 4 if 0 < w <= 127 else (8 if 0 < w <= 255 else (16 if 0 < w <= 511 else 24))
     high = bool(tuned) and not tuned[4] and tuned[0] == 1
-    minb = {4: (6, 4), 8: (4, 3), 16: (4, 3), 24: (3, 2)}[c16][1 if high else 0]
+    minb = {4: (4, 3), 8: (3, 2), 16: (2, 3), 24: (2, 2)}[c16][1 if high else 0]
     kernel = f"warp16_align_kernel<{c16}, {minb}>" if cells16 * 2 > cells else "warp_align_kernel"
-    # kernels per step: prep classify/scan/scatter, the warp kernel (one per
-    # length class when the autotuner split the queue) and, with 16-bit lanes,
+    # kernels per step: prep classify/scan/scatter (up to 4,096 pairs one
+    # kernel for all of it), the warp kernel (one per length class when the autotuner split the queue) and, with 16-bit lanes,
     # the int32 kernel over the (usually empty) overflow list
     split = bool(tuned and tuned[4])
     # on a 24-slot batch run as one launch of one warp per pair, the pairs
     # whose own band fits 640 slots take the 20-slot kernel beside it
     narrow = c16 == 24 and bool(lane16.any()) and not split and (not tuned or tuned[0] in (0, 1))
     weff = np.minimum(np.maximum(batch.t_len, batch.q_len), w if w > 0 else np.iinfo(np.int32).max)
-    launches_per_step = 3 + (4 if split else 1) + (1 if narrow else 0) + (1 if lane16.any() else 0)
+    launches_per_step = (1 if n <= 4096 else 3) + (4 if split else 1) + (1 if narrow else 0) + (1 if lane16.any() else 0)
     line = {
         "metric": METRIC, "value": round(value, 3), "unit": "GCUPS", "n_gpus": world,
         "steps": args.steps, "warmup": args.warmup,

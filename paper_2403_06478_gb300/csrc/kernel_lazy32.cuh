@@ -15,7 +15,8 @@
 // every anti-diagonal, had about 30.  The substitution is a predicated add of
 // the mismatch bit (one lop3 into a predicate): as a shift, mask and
 // multiply-add, the form of the 16-bit kernel, 2,500 ONT-like pairs took 41
-// ms, so 23.7 (64.6 before lazy blocks; 20,000 pairs 232 -> 72.6 ms).
+// ms, so 23.7 (64.6 before lazy blocks, 20.4 with the longest pairs alone on
+// their schedulers; 20,000 pairs 232 -> 72.6 ms).
 #pragma once
 
 #include "lazy_drive.cuh"

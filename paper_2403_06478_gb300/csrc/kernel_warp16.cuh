@@ -51,9 +51,9 @@
 // because the integer ALU pipe bounds this kernel (80% busy) and that step
 // has 75 of its instructions per 16-slot anti-diagonal where the bulk step
 // has 114 and the masked step about 250.  Measured on one GB300, whole calls:
-// 20,000 ONT-like pairs 59.5 -> 40.0 ms, 5,000 HiFi-like 35.9 -> 24.2, 100,000
-// pairs of Pareto lengths at w = 750 195.5 -> 82.1, 200,000 reads of 150 bp
-// 15.2 -> 5.2.  One copy of the loop in the instruction cache matters as much:
+// 20,000 ONT-like pairs 59.3 -> 38.2 ms, 5,000 HiFi-like 35.8 -> 23.2, 100,000
+// pairs of Pareto lengths at w = 750 196.0 -> 66.2, 200,000 reads of 150 bp
+// 15.2 -> 4.8 (with the launches of TierQueue).  One copy of the loop in the instruction cache matters as much:
 // a second copy for the table's last rows took the Pareto batch from 75 to 100
 // ms, bands of many widths in one batch (each its own copy) 5x.
 #pragma once
@@ -997,7 +997,7 @@ struct WarpPair16 {
     // bounds and checkpoint, about 250 instructions) against what is taken again
     // at a pair's end and the instruction cache.  On 4 slots per lane, whose
     // pairs are short, 16 (200,000 reads of 150 bp 4.5 ms, with 32 4.7); on
-    // more 32 (20,000 ONT-like pairs 37.2 ms, with 16 38.5).
+    // more 32 (20,000 ONT-like pairs 37.2 ms, with 16 38.5; before TierQueue).
     static constexpr int BLOCK_PAIRS = C <= 4 ? 16 : 32;
     static constexpr int EDGE_PAIRS = LAZY_PAIRS;        // pairs of a block with the last row or column
     static constexpr int RING = 2 * 2 * EDGE_PAIRS * P;  // words of the edge ring (row | column)

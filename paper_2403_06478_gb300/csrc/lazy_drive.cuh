@@ -88,7 +88,8 @@ __device__ __forceinline__ void lazy_edges(S &s, int32_t r0, int32_t n, int32_t 
 // exact_until, where a rebase lies between).  If the head's end lies between,
 // it goes on from there as if for the first time, with the exact maximum up to
 // there: a read that diverges soon after took its masked steps all the way
-// from the checkpoint before (16 reads with one such 112 -> 69 us).  Blocks start and end on odd anti-diagonals ((r - w) odd).
+// from the checkpoint before (16 reads with one such 112 -> 69 us).  Blocks
+// start and end on odd anti-diagonals ((r - w) odd).
 // The head's last four anti-diagonals (w - 2 .. w + 1), where the virtual
 // cells leave the band, run the masked step without its test (blind), as a
 // block of their own; a band that covers the table (cover) has no such

@@ -164,12 +164,13 @@ def test_local(ctx, name, w):
         assert bad.size == 0, (bad[:5], h0[bad[:5]], got[bad[:2]], ref[bad[:2]])
 
 
-@pytest.mark.parametrize("n", [1, 3, 151, 153, 607, 609, 1217, 1825, 2500])
+@pytest.mark.parametrize("n", [1, 3, 151, 153, 607, 609, 1217, 1825, 2500, 4096, 4097])
 @pytest.mark.parametrize("w", [100, 200, 500, 750, 1000])
 def test_tiers(ctx, n, w):
     """Batches that just fill a tier of the SMs' warps or not quite, with a few
     pairs that bound the launch (whose later tiers stay away) or none, sorted
-    and unsorted: every pair is aligned once."""
+    and unsorted, prepared in one launch (up to 4,096) and in three: every pair
+    is aligned once."""
     from oracle import oracle as O
     for long_ones in (0, min(n, 9)):
         rng = np.random.default_rng(n + w + long_ones)
