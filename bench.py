@@ -464,7 +464,8 @@ def run_traceback(args):
     info = ctx.last_traceback_info()
     packed = info["pairs16"] > 0 and info["pairs32"] * 2 < info["pairs16"]
     fused = packed and info["fused"] * 2 > info["pairs16"]
-    ops_cell = OPS_PER_CELL_TB16 if packed else OPS_PER_CELL_TB
+    # (the fused kernel computes no direction byte: the score path's operations)
+    ops_cell = (OPS_PER_CELL_I16X2 if fused else OPS_PER_CELL_TB16) if packed else OPS_PER_CELL_TB
     # the fused kernel computes the score path's cells (up to termination),
     # the two-pass kernels the cells up to each end cell
     units = cells if fused else tcells
