@@ -192,3 +192,25 @@ def test_tiers(ctx, n, w):
             assert A.results_equal(res, ref, O.COMPARE_FIELDS).size == 0
             want, _ = O.traceback_batch(batch, ref)
             assert all(np.array_equal(cig[off[i]:off[i + 1]], want[i]) for i in range(n))
+
+
+@pytest.mark.parametrize("n", [1, 153, 609, 2500, 4097])
+@pytest.mark.parametrize("w", [100, 200, 500])
+def test_local_tiers(ctx, n, w):
+    """The local extension's queue over the tiers of the SMs' warps, some pairs
+    bounding the launch and some for the per-cell step."""
+    from oracle import oracle as O
+    rng = np.random.default_rng(5 * n + w)
+    qs, ts = [], []
+    for i in range(n):
+        q = rng.integers(0, 4, int(rng.integers(30, 60) if i >= 9 else rng.integers(700, 1100)), dtype=np.uint8)
+        t, _ = W._mutate_chunk(rng, q, np.array([len(q)], np.int32), W.ErrorModel(0.05, 0.03, 0.03))
+        qs.append(q)
+        ts.append(t if len(t) else q)
+    batch = W.from_pairs(qs, ts, W.replace(ONE, w=w))
+    h0 = rng.integers(19, 61, n).astype(np.int32)
+    h0[::17] = 1 << 24
+    ref = O.align_batch(batch, h0=h0)
+    for flags in (0, A.AGATHA_NO_SORT):
+        got = ctx.align_local(A.pack_batch(batch), batch.scoring, h0, flags=flags)
+        assert A.results_equal(got, ref, O.COMPARE_FIELDS).size == 0
