@@ -161,7 +161,7 @@ struct LazyPair32 {
         }
         const int32_t lo = st - B - j0, hi = en - B - j0;
         int32_t v1 = -1, v2 = -1;                          // local slots of virtual cells
-        if (r <= w + 1) {
+        if (r < w) {                                       // (see WarpPair16::virtual_bits)
             if (r + 1 < qlen) v1 = -1 - B - j0;                // (-1, r + 1)
             if (r >= -1 && r + 1 < tlen) v2 = r + 1 - B - j0;  // (r + 1, -1)
         }
@@ -173,7 +173,7 @@ struct LazyPair32 {
             // slot NS of r - 1: the virtual column cell (t, -1) when q == -1 there
             fR = f2R = K_NEG;
             const int32_t ts = floor_div2(r - 1 - w) + NS, qs = r - 1 - ts;
-            if (qs == -1 && ts >= 0 && ts < tlen && r <= w + 1) {
+            if (qs == -1 && ts >= 0 && ts < tlen && ts <= w) {
                 const int32_t v = -gap_cost(prm, ts + 1);
                 fR = v - oe;
                 f2R = v - oe2;

@@ -145,7 +145,7 @@ struct WarpPair {
         if (lane == 0) {
             // slot -1 of r-1 is cell (B-1, r-B): a virtual row cell only when B == 0
             const int32_t ts = B - 1, qs = r - B;
-            if (ts == -1 && qs >= -1 && qs < qlen) {
+            if (ts == -1 && qs >= -1 && qs < qlen && qs <= w) {
                 const int32_t v = (qs == -1) ? 0 : -gap_cost(P, qs + 1);
                 eL = v - oe; e2L = v - oe2;
             } else {
@@ -176,7 +176,9 @@ struct WarpPair {
             const int32_t k = t - q;
             const bool real = t >= 0 && q >= 0 && t < tlen && q < qlen && k <= w && -k <= w;
             if (!real) {
-                const bool virt = (t == -1 && q >= -1 && q < qlen) || (q == -1 && t >= 0 && t < tlen);
+                // (virtual cells up to w: see WarpPair16::virtual_bits)
+                const bool virt = (t == -1 && q >= -1 && q < min(qlen, w + 1)) ||
+                                  (q == -1 && t >= 0 && t < min(tlen, w + 1));
                 if (virt) {
                     const int32_t v = (t == -1 && q == -1) ? 0 : -gap_cost(P, (t == -1 ? q : t) + 1);
                     H = v; ne = nf = v - oe; ne2 = nf2 = v - oe2;

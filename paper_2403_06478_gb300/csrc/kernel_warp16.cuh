@@ -595,8 +595,7 @@ struct WarpPair16 {
             rb = range_bits(st - B - j0, en - B - j0);
         }
         if constexpr (MODE == HEAD) {
-            if (r + 1 < qlen) vb |= slot_bit(-1 - B - j0);                 // (-1, r+1)
-            if (r >= -1 && r + 1 < tlen) vb |= slot_bit(r + 1 - B - j0);  // (r+1, -1)
+            vb = virtual_bits(r);
             const int32_t vv = to_u(r == -2 ? 0 : -gap_cost(prm, r + 2));
             if (__any_sync(gmask(), vb != 0u) && (vv < cold.LOWCHK || vv > 0xffff - cold.Dp)) ovf = true;
             VVp = (uint32_t)vv * 0x10001u;
@@ -621,9 +620,9 @@ struct WarpPair16 {
             uint32_t inj = NEGp, inj2 = NEGp;
             if (MODE == HEAD && lane == G - 1 && (K == 1 || wk == K - 1)) {
                 // beyond the last lane: slot NS of r-1, the virtual column
-                // cell (t, -1) when q == -1 there
+                // cell (t, -1) when q == -1 there (t <= w: see virtual_bits)
                 const int32_t ts = frame(r - 1) + NS, qs = r - 1 - ts;
-                if (qs == -1 && ts >= 0 && ts < tlen) {
+                if (qs == -1 && ts >= 0 && ts < tlen && ts <= w) {
                     const int32_t v = to_u(-gap_cost(prm, ts + 1));
                     if (v < cold.LOWCHK || v > 0xffff - cold.Dp) ovf = true;
                     inj = ((uint32_t)(v - oe) << 16) | (NEGp & 0xffffu);
@@ -919,8 +918,13 @@ struct WarpPair16 {
         const uint32_t y = __vmaxu2(SUB ? __vsubus2(x, d2) : __vaddus2(x, d2), NEGp + 0x10001u);
         x = mux(reset, NEGp, y);
     }
-    // lane bits of the virtual row/column cells among the slots of anti-diagonal r
+    // lane bits of the virtual row/column cells (-1, r + 1) and (r + 1, -1)
+    // among the slots of anti-diagonal r: those up to w.  The table's cells
+    // beside the later ones lie outside the band, so nothing may come out of
+    // them (a gap state that did would be back in the band two to four
+    // anti-diagonals on).
     __device__ __forceinline__ uint32_t virtual_bits(int32_t r) const {
+        if (r >= w) return 0u;
         const int32_t B = frame(r);
         uint32_t vb = 0;
         if (r + 1 < qlen) vb |= slot_bit(-1 - B - j0);
@@ -1177,11 +1181,7 @@ struct WarpPair16 {
             if (st > en) { zdropped = 1; return true; }    // the band left the table
         }
         const uint32_t rb = range_bits(st - B - j0, en - B - j0);
-        uint32_t vb = 0;
-        if (r <= w + 1) {
-            if (r + 1 < qlen) vb |= slot_bit(-1 - B - j0);                 // (-1, r+1)
-            if (r >= -1 && r + 1 < tlen) vb |= slot_bit(r + 1 - B - j0);  // (r+1, -1)
-        }
+        const uint32_t vb = virtual_bits(r);
         const int32_t vv = to_u(r == -2 ? 0 : -gap_cost(prm, r + 2));
         if (vb != 0u && (vv < cold.LOWCHK || vv > 0xffff - cold.Dp)) ovf = true;
         const uint32_t VVp = (uint32_t)vv * 0x10001u;
@@ -1189,7 +1189,7 @@ struct WarpPair16 {
         uint32_t inj = NEGp, inj2 = NEGp;
         if (lane == 31) {
             const int32_t ts = frame(r - 1) + NS, qs = r - 1 - ts;
-            if (qs == -1 && ts >= 0 && ts < tlen && r <= w + 1) {
+            if (qs == -1 && ts >= 0 && ts < tlen && ts <= w) {
                 const int32_t v = to_u(-gap_cost(prm, ts + 1));
                 if (v < cold.LOWCHK || v > 0xffff - cold.Dp) ovf = true;
                 inj = ((uint32_t)(v - oe) << 16) | (NEGp & 0xffffu);
