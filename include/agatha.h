@@ -289,10 +289,12 @@ int agatha_tune_variants(agatha_ctx *ctx, const agatha_params *params, int32_t w
  * Kernels: when the scoring allows 16-bit packed lanes (as for the score
  * path), one fused kernel aligns each pair, keeps the band's state of every
  * 32nd anti-diagonal, then recomputes its way back from the end cell segment
- * by segment and follows the path.  With AGATHA_TB_TWO_PASS (or AGATHA_PLAIN,
- * or a scoring whose steps leave too few anti-diagonals between two rebases)
- * the score path runs first and a traceback kernel then recomputes each band
- * up to its end cell, recording one direction byte per band slot.
+ * by segment and follows the path.  Where the Z-drop threshold is low against
+ * the penalties, or a scoring's steps leave too few anti-diagonals between two
+ * rebases, the fused kernel records one direction byte per band slot instead.
+ * With AGATHA_TB_TWO_PASS (or AGATHA_PLAIN) the score path runs first and a
+ * traceback kernel then recomputes each band up to its end cell, recording
+ * direction bytes.
  * AGATHA_FORCE32, a scoring beyond the 16-bit lanes, or a pair whose scores
  * leave their range use int32 lanes (two passes).  Every form gives the same
  * results and CIGARs.

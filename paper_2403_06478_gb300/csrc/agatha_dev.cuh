@@ -179,6 +179,24 @@ __host__ __device__ inline int32_t lazy_step_max(const DevParams &p) {
     const int32_t d = step_change_max(p), g = (p.a + 1) / 2 + p.e2;
     return d > g ? d : g;
 }
+// Whether a scoring leaves room for lazy blocks (lazy_drive.cuh).  A block needs
+// the Z-drop threshold to exceed what the maximum may fall by unseen: off the
+// table's edges and over the first four pairs of anti-diagonals (the drive's gate,
+// o1 + 4 c1), from where it stands after one gap opening or below four matches.
+// With less, most anti-diagonals would take the drive's masked step, and a step
+// that tests every one of them is faster (kernel_step.cuh).  Measured on both
+// sides of the line, times of the lazy kernel over the other's: minimap2's
+// short-read scoring (line at 80) 1.2 to 3.5 at 75 and 0.5 to 0.8 at 100, its
+// asm10 (99) 1.6 to 3.5 at 75, 0.5 to 0.85 at 100, its asm5 (218) 1.5 to 2.4 at
+// 200, 0.5 to 0.9 at 300, ONT (38) 1.6 to 3.5 at 30, 0.6 to 1.04 at 40.
+__host__ __device__ inline bool lazy_pays(const DevParams &p) {
+    if (p.zdrop < 0) return true;
+    const bool second = (int64_t)p.q + p.e > (int64_t)p.q2 + p.e2;       // it is the only piece then
+    const int64_t q = second ? p.q2 : p.q, e = second ? p.e2 : p.e;
+    const int64_t c1 = p.b > 2 * e ? p.b : 2 * e, rise = 4 * (int64_t)p.a;
+    return p.zdrop >= (q + e) + q + c1 + 4 * c1 + (rise > q + e ? rise : q + e);
+}
+
 // The 16-bit traceback recomputes up to 36 anti-diagonals between two rebases,
 // which steps of at most this admit (rebase_interval: 44).
 constexpr int32_t TRACE_STEP_MAX = 300;
@@ -398,6 +416,16 @@ cudaError_t launch_warp_c(const DevBatch *d_batch, int n_blocks, cudaStream_t s,
                           int list = WARP_LIST_MAIN);
 template <int C, int K = 1>
 int occupancy_warp_c();
+// The score kernels that test every anti-diagonal (kernel_step.cuh).
+template <int C>
+cudaError_t launch_step_c(const DevBatch *d_batch, int n_blocks, cudaStream_t s, int use_fast, int list);
+template <int C>
+int occupancy_step_c();
+template <int C, int MINB>
+cudaError_t launch_step16_c(const DevBatch *d_batch, int n_blocks, cudaStream_t s, int use_fast, int list,
+                            const int *priority = nullptr);
+template <int C, int MINB>
+int occupancy_step16_c();
 // MINB: warps per scheduler the 16-bit kernel's registers are cut for (one
 // block per SM holds them; with G = 16 that many blocks of four).
 // G: lanes per pair (32, or 16 for two pairs per warp).
@@ -429,6 +457,11 @@ cudaError_t launch_tbf16_c(const DevBatch *d_batch, const TbItem *items, int32_t
                            uint32_t *ops, int32_t *n_cigar, int n_blocks, cudaStream_t s);
 template <int C, int MINB>
 int occupancy_tbf16_c();
+template <int C, int MINB>
+cudaError_t launch_tbs16_c(const DevBatch *d_batch, const TbItem *items, int32_t n_items, int32_t *head,
+                           uint8_t *dir, uint32_t *ops, int32_t *n_cigar, int n_blocks, cudaStream_t s);
+template <int C, int MINB>
+int occupancy_tbs16_c();
 // Copy each pair's runs (written end first) to dense[dst_off[pair]..] in order.
 cudaError_t launch_cigar_gather(const TbItem *items, int32_t n_items, const int32_t *n_cigar,
                                 const int64_t *dst_off, const uint32_t *ops, uint32_t *dense,

@@ -5,7 +5,8 @@
 // Used where 16-bit lanes do not apply: scorings beyond them, bands of 768 to
 // 1023, the pairs they hand back, and callers that ask for int32 lanes.
 //
-// Nearly all anti-diagonals run in lazy blocks (lazy_drive.cuh).  What bounds
+// Nearly all anti-diagonals run in lazy blocks (lazy_drive.cuh; scorings that
+// leave them no room take the kernel of kernel_step.cuh).  What bounds
 // it: the integer ALU pipe when the chip is full (add-max and 3-input max
 // issue at half rate on 32 bits too, so a cell costs twice what it does on
 // 16-bit lanes), and for batches of a few thousand long pairs the longest

@@ -185,7 +185,7 @@ tb_kernel(const DevBatch *__restrict__ d_batch, const TbItem *__restrict__ items
         const TbItem it = items[k];
         uint8_t *dt = dir + it.dir_off;
         {
-            WarpPair<C> wp;
+            WarpPair<C, true> wp;
             wp.run_dir(B, it.pair, lane, it.end_t + it.end_q, dt);
         }
         __syncwarp();   // the table rows this warp wrote are read by other lanes
@@ -230,7 +230,79 @@ tb16_kernel(const DevBatch *__restrict__ d_batch, const TbItem *__restrict__ ite
     }
 }
 
-// Fused score path and traceback on 16-bit lanes.
+// Fused score path and traceback on 16-bit lanes, with direction bytes: for the
+// scorings of kernel_step.cuh, and for steps too steep for the kept states below
+// (TRACE_STEP_MAX).  Each warp aligns a pair as warp16_step_kernel does, writing
+// the direction bytes of every anti-diagonal, then walks back from the end cell
+// it found.  The table of an item has room for every anti-diagonal of the pair
+// and its run scratch for tlen + qlen runs; a pair that leaves the 16-bit range
+// goes to the int32 score kernel's list and gets n = -1.  Against kept states
+// whose score path finds no room for lazy blocks: 2,666 pairs of 600 bp at w =
+// 100, ONT scoring at a threshold of 30, 1.31 ms a call and 2.74.
+template <int C, int MINB>
+__global__ void __launch_bounds__(WARP_BLOCK_THREADS, MINB)
+tbs16_kernel(const DevBatch *__restrict__ d_batch, const TbItem *__restrict__ items, int32_t n_items,
+             int32_t *head, uint8_t *dir, uint32_t *ops, int32_t *n_cigar) {
+    __shared__ Cold16 cold[WARP_BLOCK_THREADS / 32];
+    __shared__ __align__(16) uint8_t win[WARP_BLOCK_THREADS / 32][TB_WIN_ROWS * TbLayout<C, true>::WB];
+    const DevBatch B = *d_batch;
+    const int lane = threadIdx.x & 31;
+    uint8_t *my_win = win[threadIdx.x >> 5];
+    for (;;) {
+        int32_t k = 0;
+        if (lane == 0) k = atomicAdd(head, 1);
+        k = __shfl_sync(FULL, k, 0);
+        if (k >= n_items) break;
+        const TbItem it = items[k];
+        uint8_t *dt = dir + it.dir_off;
+        bool ok;
+        int32_t et, eq;
+        {
+            // without the deferred arg-max (DEFER): its saved registers cost
+            // more here, beside the direction bits, than the searches they save
+            // (20,000 ONT-like pairs: 171 against 179 ms)
+            WarpPair16<C, (MINB < 4 && C <= 16) || MINB < 3, false, true, true> wp(cold[threadIdx.x >> 5]);
+            ok = wp.run(B, it.pair, lane, true, dt);
+            et = wp.end_t;
+            eq = wp.end_q;
+        }
+        if (!ok) {                                  // the int32 score kernel takes it
+            if (lane == 0) {
+                const int32_t slot = atomicAdd(&B.counters[CTR_NOVF], 1);
+                B.ovf_list[slot] = it.pair;
+                n_cigar[it.pair] = -1;
+            }
+            continue;
+        }
+        if (et < 0 || eq < 0) {                     // the maximum is the origin
+            if (lane == 0) n_cigar[it.pair] = 0;
+            continue;
+        }
+        __syncwarp();   // the table rows this warp wrote are read by other lanes
+        const int32_t w = effective_w(B.params.w, B.t_len[it.pair], B.q_len[it.pair]);
+        const int32_t n = tb_walk<C, true>(my_win, dt, ops + it.ops_off, et + eq + 2, et, eq, w, lane);
+        if (lane == 0) n_cigar[it.pair] = n;
+    }
+}
+
+template <int C, int MINB>
+cudaError_t launch_tbs16_c(const DevBatch *d_batch, const TbItem *items, int32_t n_items, int32_t *head,
+                           uint8_t *dir, uint32_t *ops, int32_t *n_cigar, int n_blocks, cudaStream_t s) {
+    tbs16_kernel<C, MINB><<<n_blocks, WARP_BLOCK_THREADS, 0, s>>>(d_batch, items, n_items, head, dir, ops,
+                                                                  n_cigar);
+    return cudaGetLastError();
+}
+
+template <int C, int MINB>
+int occupancy_tbs16_c() {
+    int nb = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, tbs16_kernel<C, MINB>, WARP_BLOCK_THREADS, 0) !=
+        cudaSuccess)
+        return 1;
+    return nb > 0 ? nb : 1;
+}
+
+// Fused score path and traceback on 16-bit lanes, from kept states.
 //
 // Each warp aligns a pair exactly as warp16_align_kernel does, on lazy blocks,
 // and keeps the band's state of every 32nd anti-diagonal in memory (TRACE).
@@ -575,7 +647,7 @@ __device__ __forceinline__ int32_t tb_trace(S &s, uint32_t *ops, int32_t cap) {
 // that leaves the 16-bit range goes to the int32 score kernel's list and gets
 // n = -1.
 template <int C>
-using TracePair = WarpPair16<C, false, false, false, 1, true, false, 32, true, true>;
+using TracePair = WarpPair16<C, false, false, false, true, 1, true, false, 32, true, true>;
 template <int C>
 __host__ __device__ constexpr int tbf16_warp_smem() {                 // 16-byte words of a warp
     using S = TracePair<C>;

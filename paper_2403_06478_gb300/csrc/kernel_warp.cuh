@@ -1,6 +1,6 @@
-// The int32 warp step of the traceback (kernel_tb.cuh): one warp runs one
-// pair's band from the first anti-diagonal to a given end and records, per
-// band slot and anti-diagonal, one direction byte.
+// The int32 warp step with a maximum and a termination test on every
+// anti-diagonal (the score kernel of kernel_step.cuh) or with a direction byte
+// per cell (the traceback, kernel_tb.cuh).
 //
 // Layout of a pair's band in the warp: lane L owns the C consecutive slots
 // j = L*C .. L*C + C - 1 (slot j is the cell t = B(r) + j of anti-diagonal r,
@@ -12,12 +12,17 @@
 // One anti-diagonal is one step of the warp: every lane updates its C cells,
 // the only cross-lane inputs are the E states of the left neighbour's last
 // slot or the F states of the right neighbour's first slot (warp shuffles).
+// The anti-diagonal maximum and its lowest t come from a warp reduction, and
+// the exact termination test (Eq. 4-7) runs after every anti-diagonal, so no
+// cell beyond the stopping anti-diagonal is ever computed.
 //
 // Steps near the table's edges (the first w+4 anti-diagonals, where virtual
 // row/column cells enter, and the ones that touch t = tlen-1 or q = qlen-1)
 // run a masked variant; the bulk in between runs unmasked.
 //
-// The direction byte:
+// With DIR the same steps also record, per band slot and anti-diagonal, one
+// direction byte for the traceback (kernel_tb.cuh) and run to a given end
+// anti-diagonal instead of testing termination:
 //   bits 0-2  which input H took: 0 diagonal, 1 E, 2 F, 3 E2, 4 F2 (the first
 //             of these that equals H)
 //   bits 3-6  whether Eo, Fo, E2o, F2o leaving this cell extend the cell's
@@ -41,7 +46,7 @@ struct WarpWin {
     static constexpr T LOW = (sizeof(T) == 4) ? T(0x55555555u) : T(0x5555555555555555ull);
 };
 
-template <int C>
+template <int C, bool DIR = false>
 struct WarpPair {
     using W = typename WarpWin<C>::T;
     static constexpr int32_t DIR_ROW = 32 * C;   // direction bytes per anti-diagonal
@@ -58,9 +63,13 @@ struct WarpPair {
     uint32_t Tpf, Qpf;       // next 16 bases to shift in
     int32_t tcnt, qcnt;      // bases left in Tpf / Qpf
     int64_t tpos, qpos;      // base index of the next refill
-    uint8_t *dtab;           // this lane's bytes of anti-diagonal 0
+    // anti-diagonal bookkeeping (uniform across the warp)
+    int32_t gmax, gt, gq, mqe, mqe_t, mte, mte_q, gscore;
+    int64_t cells;
+    int32_t zdropped;
+    uint8_t *dtab;           // DIR: this lane's bytes of anti-diagonal 0
 
-    // the direction byte of one cell (see the top of this file)
+    // DIR: the direction byte of one cell (see the top of this file)
     __device__ __forceinline__ uint32_t dir_bits(int32_t hd, int32_t Ein, int32_t Fin, int32_t E2in,
                                                  int32_t F2in, int32_t H, int32_t hoe,
                                                  int32_t hoe2) const {
@@ -72,7 +81,7 @@ struct WarpPair {
         return b;
     }
 
-    // this lane's C bytes of anti-diagonal r, one aligned vector store
+    // DIR: this lane's C bytes of anti-diagonal r, one aligned vector store
     __device__ __forceinline__ void store_dir(int32_t r, const uint32_t (&wd)[C / 4]) const {
         uint8_t *p = dtab + (int64_t)r * DIR_ROW;
         if constexpr (C % 16 == 0) {
@@ -133,10 +142,41 @@ struct WarpPair {
         }
     }
 
+    // Global max update, else the Z-drop test (Eq. 4-7).  Returns true to stop.
+    __device__ __forceinline__ bool max_and_zdrop(int32_t m, int32_t tstar, int32_t r) {
+        const int32_t qstar = r - tstar;
+        if (m > gmax) {
+            gmax = m; gt = tstar; gq = qstar;
+            return false;
+        }
+        if (tstar >= gt && qstar >= gq && P.zdrop >= 0) {
+            int32_t l = (tstar - gt) - (qstar - gq);
+            l = l < 0 ? -l : l;
+            if (gmax - m > P.zdrop + l * P.e2) return true;
+        }
+        return false;
+    }
+
+    // Lowest-t argmax of the anti-diagonal from per-lane (max, first index).
+    __device__ __forceinline__ void warp_argmax(int32_t lm, int32_t li, int32_t B, int32_t &m,
+                                                int32_t &tstar) const {
+        m = __reduce_max_sync(FULL, lm);
+        unsigned ball = __ballot_sync(FULL, lm == m && li >= 0);
+        int src = __ffs(ball) - 1;
+        int32_t lj = __shfl_sync(FULL, li, src);
+        tstar = B + src * C + lj;
+    }
+
     // One anti-diagonal with every edge case handled per cell.
-    __device__ __forceinline__ void masked_step(int32_t r) {
+    __device__ __forceinline__ bool masked_step(int32_t r) {
         const int32_t B = ceil_div2(r - w);
         const int32_t d = (r - w) & 1;
+        if (!DIR && r >= 0) {
+            const int32_t st = max(max(0, r - qlen + 1), B);
+            const int32_t en = min(min(tlen - 1, r), floor_div2(r + w));
+            if (st > en) { zdropped = 1; return true; }    // the band left the table
+            cells += en - st + 1;
+        }
         // cross-lane neighbours
         int32_t eL = __shfl_up_sync(FULL, Eo[C - 1], 1);
         int32_t e2L = __shfl_up_sync(FULL, E2o[C - 1], 1);
@@ -159,6 +199,7 @@ struct WarpPair {
         uint32_t wd[C / 4];
 #pragma unroll
         for (int k = 0; k < C / 4; ++k) wd[k] = 0;
+        int32_t lm = INT_MIN, li = -1, te_c = INT_MIN, qe_c = INT_MIN;
 #pragma unroll
         for (int jl = 0; jl < C; ++jl) {
             const int32_t t = B + j0 + jl;
@@ -172,10 +213,15 @@ struct WarpPair {
             int32_t hoe = H - oe, hoe2 = H - oe2;
             int32_t ne = max(hoe, Ein - P.e), nf = max(hoe, Fin - P.e);
             int32_t ne2 = max(hoe2, E2in - P.e2), nf2 = max(hoe2, F2in - P.e2);
-            wd[jl >> 2] |= dir_bits(H2[jl] + s, Ein, Fin, E2in, F2in, H, hoe, hoe2) << (8 * (jl & 3));
+            if constexpr (DIR)
+                wd[jl >> 2] |= dir_bits(H2[jl] + s, Ein, Fin, E2in, F2in, H, hoe, hoe2) << (8 * (jl & 3));
             const int32_t k = t - q;
             const bool real = t >= 0 && q >= 0 && t < tlen && q < qlen && k <= w && -k <= w;
-            if (!real) {
+            if (real) {
+                if (H > lm) { lm = H; li = jl; }
+                if (t == tlen - 1) te_c = H;
+                if (q == qlen - 1) qe_c = H;
+            } else {
                 // (virtual cells up to w: see WarpPair16::virtual_bits)
                 const bool virt = (t == -1 && q >= -1 && q < min(qlen, w + 1)) ||
                                   (q == -1 && t >= 0 && t < min(tlen, w + 1));
@@ -193,13 +239,28 @@ struct WarpPair {
             H2[jl] = H1[jl]; H1[jl] = nH[jl];
             Eo[jl] = nE[jl]; E2o[jl] = nE2[jl]; Fo[jl] = nF[jl]; F2o[jl] = nF2[jl];
         }
-        if (r >= 0) store_dir(r, wd);
+        if (r < 0) return false;
+        if constexpr (DIR) {
+            store_dir(r, wd);
+            return false;
+        }
+        // last target row / last query column
+        const int32_t te_v = __reduce_max_sync(FULL, te_c);
+        if (te_v != INT_MIN && te_v > mte) { mte = te_v; mte_q = r - (tlen - 1); }
+        const int32_t qe_v = __reduce_max_sync(FULL, qe_c);
+        if (qe_v != INT_MIN && qe_v > mqe) { mqe = qe_v; mqe_t = r - (qlen - 1); }
+        int32_t m, tstar;
+        warp_argmax(lm, li, B, m, tstar);
+        if (max_and_zdrop(m, tstar, r)) { zdropped = 1; return true; }
+        if (r == last_r && te_v != INT_MIN && (r - (tlen - 1)) == qlen - 1) gscore = te_v;
+        return false;
     }
 
     // One bulk anti-diagonal: every band cell is a real cell away from the last
     // row/column, so only the band's own edges need care.  D = (r - w) & 1.
     template <int D>
-    __device__ __forceinline__ void fast_step(int32_t r, int32_t vcnt) {
+    __device__ __forceinline__ bool fast_step(int32_t r, int32_t vcnt) {
+        const int32_t B = ceil_div2(r - w);
         int32_t eL = 0, e2L = 0, fR = 0, f2R = 0;
         if constexpr (D == 0) {
             eL = __shfl_up_sync(FULL, Eo[C - 1], 1);
@@ -216,6 +277,7 @@ struct WarpPair {
         uint32_t wd[C / 4];
 #pragma unroll
         for (int k = 0; k < C / 4; ++k) wd[k] = 0;
+        int32_t lm = INT_MIN, li = -1;
 #pragma unroll
         for (int jl = 0; jl < C; ++jl) {
             const int32_t Ein = D ? Eo[jl] : (jl ? Eo[jl - 1] : eL);
@@ -229,25 +291,97 @@ struct WarpPair {
             // flows back into the band; their E states only flow further out
             const int32_t hoe = valid ? H - oe : K_NEG;
             const int32_t hoe2 = valid ? H - oe2 : K_NEG;
-            wd[jl >> 2] |= dir_bits(H2[jl] + s, Ein, Fin, E2in, F2in, H, hoe, hoe2) << (8 * (jl & 3));
+            if constexpr (DIR)
+                wd[jl >> 2] |= dir_bits(H2[jl] + s, Ein, Fin, E2in, F2in, H, hoe, hoe2) << (8 * (jl & 3));
             nE[jl] = max(hoe, Ein - P.e);
             nF[jl] = max(hoe, Fin - P.e);
             nE2[jl] = max(hoe2, E2in - P.e2);
             nF2[jl] = max(hoe2, F2in - P.e2);
             nH[jl] = H;
+            if (valid && H > lm) { lm = H; li = jl; }
         }
 #pragma unroll
         for (int jl = 0; jl < C; ++jl) {
             H2[jl] = H1[jl]; H1[jl] = nH[jl];
             Eo[jl] = nE[jl]; E2o[jl] = nE2[jl]; Fo[jl] = nF[jl]; F2o[jl] = nF2[jl];
         }
-        store_dir(r, wd);
+        if constexpr (DIR) {
+            store_dir(r, wd);
+            return false;
+        }
+        cells += w + 1 - D;
+        int32_t m, tstar;
+        warp_argmax(lm, li, B, m, tstar);
+        if (max_and_zdrop(m, tstar, r)) { zdropped = 1; return true; }
+        return false;
     }
 
-    // Anti-diagonals 0..r_end of a pair with its direction bytes in
+    __device__ __forceinline__ void run(const DevBatch &Bt, int32_t pair, int32_t lane_, bool use_fast) {
+        P = Bt.params;
+        lane = lane_;
+        tp = Bt.t_packed; qp = Bt.q_packed; tw = Bt.t_words; qw = Bt.q_words;
+        tlen = Bt.t_len[pair]; qlen = Bt.q_len[pair];
+        toff = Bt.t_off[pair]; qoff = Bt.q_off[pair];
+        agatha_result *out = Bt.out + pair;
+        if (tlen <= 0 || qlen <= 0) {
+            if (lane == 0) write_empty_result(out);
+            return;
+        }
+        w = effective_w(P.w, tlen, qlen);
+        oe = P.q + P.e; oe2 = P.q2 + P.e2;
+        j0 = lane * C;
+        last_r = tlen + qlen - 2;
+#pragma unroll
+        for (int i = 0; i < C; ++i) { H1[i] = H2[i] = Eo[i] = E2o[i] = Fo[i] = F2o[i] = K_NEG; }
+        gmax = 0; gt = -1; gq = -1;
+        mqe = K_NEG_OUT; mqe_t = -1; mte = K_NEG_OUT; mte_q = -1; gscore = K_NEG_OUT;
+        cells = 0; zdropped = 0;
+
+        int32_t r = -2;
+        init_windows(r);
+        bool stop = masked_step(r);
+        const int32_t head_end = min(last_r, w + 1);
+        while (!stop && r < head_end) {
+            ++r;
+            if ((r - w) & 1) shift_t(); else shift_q();
+            stop = masked_step(r);
+        }
+        // bulk: pairs of anti-diagonals (even, odd) starting at r = w + 2
+        const int32_t L = min(tlen, qlen);
+        const int32_t bulk_last = 2 * L - 3 - w;
+        if (use_fast && !stop && r == w + 1) {
+            const int32_t vcnt0 = max(0, min(C, w + 1 - j0));
+            const int32_t vcnt1 = max(0, min(C, w - j0));
+            while (r + 2 <= bulk_last) {
+                ++r; shift_q();
+                if (fast_step<0>(r, vcnt0)) { stop = true; break; }
+                ++r; shift_t();
+                if (fast_step<1>(r, vcnt1)) { stop = true; break; }
+            }
+        }
+        while (!stop && r < last_r) {
+            ++r;
+            if ((r - w) & 1) shift_t(); else shift_q();
+            stop = masked_step(r);
+        }
+        if (lane == 0) {
+            agatha_result o;
+            o.max = gmax; o.te = gt; o.qe = gq;
+            o.gscore = gscore; o.mqe = mqe; o.mqe_t = mqe_t; o.mte = mte; o.mte_q = mte_q;
+            o.cells = cells;
+            o.zdropped = (uint8_t)zdropped;
+            o.reach_end = (uint8_t)(!zdropped && mqe != K_NEG_OUT && mqe + P.end_bonus > gmax);
+            o.lane16 = 0;
+            for (int i = 0; i < 5; ++i) o.pad[i] = 0;
+            *out = o;
+        }
+    }
+
+    // DIR: anti-diagonals 0..r_end of a pair with its direction bytes in
     // dt[r * DIR_ROW + slot] (no termination test: r_end is known).
     __device__ __forceinline__ void run_dir(const DevBatch &Bt, int32_t pair, int32_t lane_,
                                             int32_t r_end, uint8_t *dt) {
+        static_assert(DIR, "run_dir needs the direction variant");
         P = Bt.params;
         lane = lane_;
         tp = Bt.t_packed; qp = Bt.q_packed; tw = Bt.t_words; qw = Bt.q_words;
@@ -260,6 +394,7 @@ struct WarpPair {
         dtab = dt + j0;
 #pragma unroll
         for (int i = 0; i < C; ++i) { H1[i] = H2[i] = Eo[i] = E2o[i] = Fo[i] = F2o[i] = K_NEG; }
+        cells = 0; zdropped = 0;
         int32_t r = -2;
         init_windows(r);
         masked_step(r);

@@ -45,7 +45,8 @@
 // of the table, where the virtual row and column enter, runs the bulk or the
 // tail step wherever their values follow from the recurrence itself).
 //
-// The score path with one warp per pair (LAZY) goes further: nearly all its
+// The score path with one warp per pair (LAZY; lazy_pays tells for which
+// scorings) goes further: nearly all its
 // anti-diagonals, the head's and the tail's too, run in blocks whose step
 // leaves out the maximum, the test and every mask (lazy_step, lazy_drive),
 // because the integer ALU pipe bounds this kernel (80% busy) and that step
@@ -125,7 +126,9 @@ struct Xchg16 {
 //   bits 4-7  Eo, Fo, E2o, F2o leaving the cell extend the cell's own gap
 //             state (strictly better than opening from H)
 // Each bit is one 16x2 minimum of an exclusive or (0 or 1 per half).
-// With DIR (run_dir) the end anti-diagonal is given and nothing else is tracked.
+// SCORE: the termination test and the result.  DIR with SCORE aligns and writes
+// the direction bytes in one pass; without SCORE (run_dir) the end
+// anti-diagonal is given and nothing else is tracked.
 // K: warps sharing one pair's band (1, 2 or 4).  Warp k of the group holds
 // slots 32kC .. 32(k+1)C - 1 of the frame; after every anti-diagonal the warps
 // exchange their edge gap states and anti-diagonal maxima through shared
@@ -138,7 +141,7 @@ struct Xchg16 {
 // TRACE (with LAZY): the score path also keeps the band's state of every 32nd
 // anti-diagonal in memory, from which the traceback recomputes its way back
 // (tb_trace in kernel_tb.cuh).
-template <int C, bool DMREG, bool DEFER = false, bool DIR = false, int K = 1,
+template <int C, bool DMREG, bool DEFER = false, bool DIR = false, bool SCORE = !DIR, int K = 1,
           bool FHEAD = false, bool EDEFER = false, int G = 32, bool LAZY = false, bool TRACE_ = false>
 struct WarpPair16 {
     static_assert(C == 4 || C == 6 || C == 8 || C == 12 || C == 16 || C == 20 || C == 24,
@@ -189,7 +192,7 @@ struct WarpPair16 {
     uint32_t Hsave[DEFER ? P : 1]; // DEFER: H of the pending maximum's anti-diagonal
     uint8_t *dtab;                 // DIR: this lane's bytes of anti-diagonal 0
     uint4 *gck;                    // TRACE: the pair's states in memory
-    int32_t end_t, end_q;          // TRACE: where the traceback starts (-1: empty)
+    int32_t end_t, end_q;          // TRACE, DIR with SCORE: where the traceback starts (-1: empty)
     int32_t pend_r, pend_m, pend_lm;   // its anti-diagonal (-3: none), maximum, lane maximum
     uint32_t pend_rb;              // lane bits of its band slots (~0: every slot of the bulk)
     bool in_head;                  // FHEAD: the pair loop is running head anti-diagonals
@@ -709,7 +712,10 @@ struct WarpPair16 {
             else if (i == P - 1) lmax = __vmaxu2(lmax, mx);
             else pend = mx;
         }
-        if constexpr (DIR) return dir_finish<ODD, MODE>(r, lmax, rb, vb, dbits);
+        if constexpr (DIR && !SCORE) return dir_finish<ODD, MODE>(r, lmax, rb, vb, dbits);
+        if constexpr (DIR && SCORE) {
+            if (r >= 0) store_row(r, dbits);
+        }
         const int32_t lm = (int32_t)max(lmax & 0xffffu, lmax >> 16);
         int32_t m_grp = 0;
         if constexpr (K > 1) m_grp = exchange<!ODD, MODE != BULK>(r, lm);
@@ -788,7 +794,7 @@ struct WarpPair16 {
         }
     }
 
-    // DIR: end of a step.  Store the row, then what the rebase
+    // DIR without SCORE: end of a step.  Store the row, then what the rebase
     // needs: the anti-diagonal maximum (only when a rebase follows) and the
     // rebase.
     template <bool ODD, int MODE>
@@ -1558,7 +1564,8 @@ struct WarpPair16 {
 
     // ------------------------------------------------------------------ pair
     // Returns false if the pair must be recomputed with int32 lanes.
-    // TRACE: states is the memory for the pair's states.
+    // TRACE: states is the memory for the pair's states; DIR: its direction
+    // table, one row per anti-diagonal up to the last one.
     __device__ __forceinline__ bool run(const DevBatch &Bt, int32_t pair, int32_t lane_, bool use_fast,
                                         uint8_t *states = nullptr) {
         prm = Bt.params;
@@ -1586,11 +1593,11 @@ struct WarpPair16 {
             qspan = (int32_t)min(Bt.q_words - qw0, (int64_t)((qph + qlen + 15) >> 4));
         }
         agatha_result *out = Bt.out + pair;
-        if constexpr (TRACE) {
+        if constexpr (TRACE || DIR) {
             end_t = -1;
             end_q = -1;
-            gck = reinterpret_cast<uint4 *>(states);
         }
+        if constexpr (TRACE) gck = reinterpret_cast<uint4 *>(states);
         if (tlen <= 0 || qlen <= 0) {
             if (leader()) write_empty_result(out);
             return true;
@@ -1611,6 +1618,7 @@ struct WarpPair16 {
         oe = prm.q + prm.e; oe2 = prm.q2 + prm.e2;
         j0 = (wk * G + lane) * C;
         last_r = tlen + qlen - 2;
+        if constexpr (DIR) dtab = states + j0;
         {
             const int32_t Dp = LAZY ? lazy_step_max(prm) : step_change_max(prm);
             const int32_t kint = rebase_interval(Dp);
@@ -1671,7 +1679,7 @@ struct WarpPair16 {
         }
         if (ovf) return false;
         locate_pending();
-        if constexpr (TRACE) {
+        if constexpr (TRACE || DIR) {
             // the traceback's start: the query end when reached, else the maximum
             const bool reach = !zdropped && cold.mqe != K_NEG_OUT && cold.mqe + prm.end_bonus > gmax;
             end_t = __reduce_max_sync(FULL, reach ? cold.mqe_t : cold.gt);
@@ -1805,7 +1813,7 @@ warp16_align_kernel(const DevBatch *__restrict__ d_batch, int32_t use_fast, int3
     const int lane = threadIdx.x & (G - 1);
     const WorkList L = work_list(B, list);
     if constexpr (G == 32) {
-        using Pair = WarpPair16<C, false, false, false, 1, true, false, 32, true>;
+        using Pair = WarpPair16<C, false, false, false, true, 1, true, false, 32, true>;
         extern __shared__ uint4 lazy_smem[];
         __shared__ TierQueue q;
         __shared__ int32_t first[4], place[warp16_threads(MINB, G) / 32];
@@ -1841,7 +1849,7 @@ warp16_align_kernel(const DevBatch *__restrict__ d_batch, int32_t use_fast, int3
         }
         if (lane == 0 && (q.had(place[warp]) || blockIdx.x == 0)) mark_step_end(B.counters);
     } else {
-        using Pair = WarpPair16<C, MINB < 4, true, false, 1, true, true, G>;
+        using Pair = WarpPair16<C, MINB < 4, true, false, true, 1, true, true, G>;
         // The warp takes two neighbouring pairs of the longest-first queue at
         // once (about the same length), one per half, and both halves start
         // their next pairs together: the two then pass through the same step
@@ -1885,7 +1893,7 @@ warp16k_align_kernel(const DevBatch *__restrict__ d_batch, int32_t use_fast, int
     const int32_t bar = 1 + g;                           // named barrier of the group
     const WorkList L = work_list(B, list);
     for (;;) {
-        WarpPair16<C, (MINB < 4 && C <= 16) || MINB < 3, true, false, K> wp(cold[g], &xch[g], wk, bar);
+        WarpPair16<C, (MINB < 4 && C <= 16) || MINB < 3, true, false, true, K> wp(cold[g], &xch[g], wk, bar);
         if (wk == 0 && lane == 0) xch[g].pair = L.begin + atomicAdd(L.head, 1);
         wp.group_sync();
         const int32_t k = xch[g].pair;
@@ -1921,7 +1929,7 @@ int occupancy_warp16k_c() {
 // warp.
 template <int C, int MINB, int G>
 constexpr int warp16_smem() {
-    using Pair = WarpPair16<C, false, false, false, 1, true, false, 32, true>;
+    using Pair = WarpPair16<C, false, false, false, true, 1, true, false, 32, true>;
     return G == 32 ? (warp16_threads(MINB, G) / 32) * (2 * Pair::CKV * 32 * 16 + Pair::RING * 4) : 0;
 }
 

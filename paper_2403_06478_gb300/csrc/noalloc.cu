@@ -108,7 +108,8 @@ extern "C" int agatha_align_batch_noalloc(const agatha_batch *batch, const agath
         if (wide_w > plain_kernel_max_w()) return AGATHA_ENOTSUP;
     }
     const Shape32 shape = pick_shape32(w_plan < warp_w_max ? w_plan : warp_w_max);
-    const int blocks = ds->n_sm * warp32_occupancy(shape);
+    const bool lazy = lazy_pays(p);
+    const int blocks = ds->n_sm * (lazy ? warp32_occupancy(shape) : step32_occupancy(C));
 
     DevBatch desc;
     desc.q_packed = batch->q_packed;
@@ -136,7 +137,9 @@ extern "C" int agatha_align_batch_noalloc(const agatha_batch *batch, const agath
     cudaError_t e = cudaMemcpyAsync((void *)d_desc, &desc, sizeof(desc), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess)
         e = launch_prep(d_desc, batch->n_pairs, 1, desc.counters, desc.bucket_hist, s, ds->n_sm);
-    if (e == cudaSuccess) e = launch_warp32(shape, d_desc, blocks, s, 1, WARP_LIST_MAIN);
+    if (e == cudaSuccess)
+        e = lazy ? launch_warp32(shape, d_desc, blocks, s, 1, WARP_LIST_MAIN)
+                 : launch_step32(C, d_desc, blocks, s, 1, WARP_LIST_MAIN);
     if (e == cudaSuccess && wide_w > 0) e = launch_plain_kernel(d_desc, (int64_t)ds->n_sm * 2, wide_w, 1, s);
     int32_t ctr[CTR_COUNT] = {0};
     if (e == cudaSuccess)

@@ -183,15 +183,55 @@ int warp32_occupancy(Shape32 k) {
     }
 }
 
+// The int32 score kernel with a test on every anti-diagonal, C slots per lane.
+cudaError_t launch_step32(int C, const DevBatch *d, int blocks, cudaStream_t s, int fast, int list) {
+    switch (C) {
+        case 4: return launch_step_c<4>(d, blocks, s, fast, list);
+        case 8: return launch_step_c<8>(d, blocks, s, fast, list);
+        case 16: return launch_step_c<16>(d, blocks, s, fast, list);
+        case 24: return launch_step_c<24>(d, blocks, s, fast, list);
+        default: return launch_step_c<32>(d, blocks, s, fast, list);
+    }
+}
+
+int step32_occupancy(int C) {
+    switch (C) {
+        case 4: return occupancy_step_c<4>();
+        case 8: return occupancy_step_c<8>();
+        case 16: return occupancy_step_c<16>();
+        case 24: return occupancy_step_c<24>();
+        default: return occupancy_step_c<32>();
+    }
+}
+
+// The int32 score kernel of a plan.
+static cudaError_t launch_plan32(const LaunchPlan &lp, const DevBatch *d, cudaStream_t s, int list) {
+    return lp.lazy ? launch_warp32(lp.shape32, d, lp.warp_blocks, s, lp.fast, list)
+                   : launch_step32(lp.C, d, lp.warp_blocks, s, lp.fast, list);
+}
+
 // 16-bit kernel with C slots per lane at its default budget of registers or
 // (high) the second one, which the autotuner tries too.  The defaults are the
 // faster ones on the workloads: with 16 slots two warps per scheduler of up to
 // 255 registers, whose lazy loop has no register moves (20,000 ONT-like pairs
 // 37.6 ms, three warps of 168 38.3; 5,000 HiFi-like 23.1 and 23.6); with 8 slots
 // three (20,000 pairs of 2 kbp at w = 200: 7.3 ms, two 8.4); with 4 slots four
-// (200,000 reads of 150 bp: 4.5 ms, three 5.4); with 24 only two fit.
-static cudaError_t launch_warp16(int C, int high, const DevBatch *d, int blocks, cudaStream_t s,
+// (200,000 reads of 150 bp: 4.5 ms, three 5.4); with 24 only two fit.  Without
+// lazy blocks the default is the smaller budget, the second the larger.
+static cudaError_t launch_warp16(int C, int high, int lazy, const DevBatch *d, int blocks, cudaStream_t s,
                                  int fast, int list) {
+    if (!lazy) {
+        switch (C * 2 + high) {
+            case 8: return launch_step16_c<4, 6>(d, blocks, s, fast, list);
+            case 9: return launch_step16_c<4, 4>(d, blocks, s, fast, list);
+            case 16: return launch_step16_c<8, 4>(d, blocks, s, fast, list);
+            case 17: return launch_step16_c<8, 3>(d, blocks, s, fast, list);
+            case 32: return launch_step16_c<16, 4>(d, blocks, s, fast, list);
+            case 33: return launch_step16_c<16, 3>(d, blocks, s, fast, list);
+            case 48: return launch_step16_c<24, 3>(d, blocks, s, fast, list);
+            default: return launch_step16_c<24, 2>(d, blocks, s, fast, list);
+        }
+    }
     switch (C * 2 + high) {
         case 8: return launch_warp16_c<4, 4>(d, blocks, s, fast, list);
         case 9: return launch_warp16_c<4, 3>(d, blocks, s, fast, list);
@@ -237,10 +277,22 @@ int warp16k_occupancy(int C16, int K) {
 }
 
 cudaError_t launch_overflow_int32(const Slot *sl, const LaunchPlan &lp, cudaStream_t s) {
-    return launch_warp32(lp.shape32, sl->d_desc, lp.warp_blocks, s, lp.fast, WARP_LIST_OVERFLOW);
+    return launch_plan32(lp, sl->d_desc, s, WARP_LIST_OVERFLOW);
 }
 
-int warp16_occupancy(int C, int high) {
+int warp16_occupancy(int C, int high, int lazy) {
+    if (!lazy) {
+        switch (C * 2 + high) {
+            case 8: return occupancy_step16_c<4, 6>();
+            case 9: return occupancy_step16_c<4, 4>();
+            case 16: return occupancy_step16_c<8, 4>();
+            case 17: return occupancy_step16_c<8, 3>();
+            case 32: return occupancy_step16_c<16, 4>();
+            case 33: return occupancy_step16_c<16, 3>();
+            case 48: return occupancy_step16_c<24, 3>();
+            default: return occupancy_step16_c<24, 2>();
+        }
+    }
     switch (C * 2 + high) {
         case 8: return occupancy_warp16_c<4, 4>();
         case 9: return occupancy_warp16_c<4, 3>();
@@ -287,12 +339,14 @@ static cudaError_t enqueue_part(agatha_ctx *ctx, Slot *sl, const LaunchPlan &lp,
             // and the second's fill them as the first's leave
             if ((e = cudaEventRecord(sl->fork, s)) != cudaSuccess) return e;
             if ((e = cudaStreamWaitEvent(sl->aux[0], sl->fork, 0)) != cudaSuccess) return e;
-            e = launch_warp16_prio<24, 2>(d, lp.warp16_blocks[lp.regs_high], s, lp.fast, WARP_LIST_MAIN,
-                                          ctx->prio_greatest);
+            const int blocks = lp.warp16_blocks[lp.regs_high], first = ctx->prio_greatest, after = ctx->prio_least;
+            if (lp.lazy) e = launch_warp16_prio<24, 2>(d, blocks, s, lp.fast, WARP_LIST_MAIN, first);
+            else if (lp.regs_high) e = launch_step16_c<24, 2>(d, blocks, s, lp.fast, WARP_LIST_MAIN, &first);
+            else e = launch_step16_c<24, 3>(d, blocks, s, lp.fast, WARP_LIST_MAIN, &first);
             if (e != cudaSuccess) return e;
-            if ((e = launch_warp16_prio<20, 2>(d, lp.narrow_blocks, sl->aux[0], lp.fast, WARP_LIST_NARROW,
-                                               ctx->prio_least)) != cudaSuccess)
-                return e;
+            e = lp.lazy ? launch_warp16_prio<20, 2>(d, lp.narrow_blocks, sl->aux[0], lp.fast, WARP_LIST_NARROW, after)
+                        : launch_step16_c<20, 2>(d, lp.narrow_blocks, sl->aux[0], lp.fast, WARP_LIST_NARROW, &after);
+            if (e != cudaSuccess) return e;
             if ((e = cudaEventRecord(sl->join[0], sl->aux[0])) != cudaSuccess) return e;
             if ((e = cudaStreamWaitEvent(s, sl->join[0], 0)) != cudaSuccess) return e;
             any16 = true;
@@ -304,11 +358,11 @@ static cudaError_t enqueue_part(agatha_ctx *ctx, Slot *sl, const LaunchPlan &lp,
                                WARP_LIST_MAIN);
             any16 = true;
         } else if (lp.lane16) {
-            e = launch_warp16(lp.C16, lp.regs_high, d, lp.warp16_blocks[lp.regs_high], s, lp.fast,
+            e = launch_warp16(lp.C16, lp.regs_high, lp.lazy, d, lp.warp16_blocks[lp.regs_high], s, lp.fast,
                               WARP_LIST_MAIN);
             any16 = true;
         } else {
-            e = launch_warp32(lp.shape32, d, lp.warp_blocks, s, lp.fast, WARP_LIST_MAIN);
+            e = launch_plan32(lp, d, s, WARP_LIST_MAIN);
         }
         if (e != cudaSuccess) return e;
     } else {
@@ -320,7 +374,7 @@ static cudaError_t enqueue_part(agatha_ctx *ctx, Slot *sl, const LaunchPlan &lp,
             if ((e = cudaStreamWaitEvent(sc, sl->fork, 0)) != cudaSuccess) return e;
             const int v = lp.cls_var[c];
             if (v == VAR_32) {
-                e = launch_warp32(lp.shape32, d, lp.warp_blocks, sc, lp.fast, WARP_LIST_CLASS + c);
+                e = launch_plan32(lp, d, sc, WARP_LIST_CLASS + c);
             } else if (v == VAR_16_HALF) {
                 e = launch_warp16h(lp.C16, d, lp.warp16h_blocks, sc, lp.fast, WARP_LIST_CLASS + c);
                 any16 = true;
@@ -329,7 +383,7 @@ static cudaError_t enqueue_part(agatha_ctx *ctx, Slot *sl, const LaunchPlan &lp,
                 e = launch_warp16k(lp.C16, K, d, lp.warp16k_blocks[K == 4], sc, lp.fast, WARP_LIST_CLASS + c);
                 any16 = true;
             } else {
-                e = launch_warp16(lp.C16, v == VAR_16_HIGHREG, d, lp.warp16_blocks[v == VAR_16_HIGHREG],
+                e = launch_warp16(lp.C16, v == VAR_16_HIGHREG, lp.lazy, d, lp.warp16_blocks[v == VAR_16_HIGHREG],
                                   sc, lp.fast, WARP_LIST_CLASS + c);
                 any16 = true;
             }
@@ -339,8 +393,7 @@ static cudaError_t enqueue_part(agatha_ctx *ctx, Slot *sl, const LaunchPlan &lp,
         }
     }
     // pairs whose scores left the 16-bit range, recomputed on int32 lanes
-    if (any16 && (e = launch_warp32(lp.shape32, d, lp.warp_blocks, s, lp.fast, WARP_LIST_OVERFLOW)) != cudaSuccess)
-        return e;
+    if (any16 && (e = launch_plan32(lp, d, s, WARP_LIST_OVERFLOW)) != cudaSuccess) return e;
     if (lp.wide_w > 0) e = launch_plain_kernel(d, (int64_t)ctx->n_sm * 2, lp.wide_w, 1, s);
     return e;
 }
@@ -490,8 +543,12 @@ int make_plan(agatha_ctx *ctx, const DevParams &p, const BatchShape &shape, uint
                          lp->wide_w, pmax);
     lp->shape32 = pick_shape32(std::min(shape.max_w_all, lp->warp_w_max));
     const Shape32 s32 = lp->shape32;
-    lp->warp_blocks = ctx->n_sm * plan_occupancy(ctx, 0, s32.K == 1 ? s32.C / 4 : (s32.C == 8 ? 5 : 6),
-                                                 [&] { return warp32_occupancy(s32); });
+    const int C32 = lp->C;
+    lp->lazy = lazy_pays(p) ? 1 : 0;
+    lp->warp_blocks =
+        ctx->n_sm * (lp->lazy ? plan_occupancy(ctx, 0, s32.K == 1 ? s32.C / 4 : (s32.C == 8 ? 5 : 6),
+                                               [&] { return warp32_occupancy(s32); })
+                              : plan_occupancy(ctx, 6, C32 / 4, [&] { return step32_occupancy(C32); }));
     // 16-bit packed lanes when the band fits and one anti-diagonal changes a
     // score by at most 255 (the 16-bit kernel then still rebases at least
     // every 50 anti-diagonals)
@@ -504,10 +561,10 @@ int make_plan(agatha_ctx *ctx, const DevParams &p, const BatchShape &shape, uint
     lp->warp16h_blocks = 0;
     if (lp->lane16) {
         lp->warp_w_max = 32 * lp->C16 - 1;
-        const int C16 = lp->C16;
+        const int C16 = lp->C16, lazy = lp->lazy;
         const auto blocks = [&](int kind, auto ask) { return ctx->n_sm * plan_occupancy(ctx, kind, C16 / 4, ask); };
-        lp->warp16_blocks[0] = blocks(1, [&] { return warp16_occupancy(C16, 0); });
-        lp->warp16_blocks[1] = blocks(2, [&] { return warp16_occupancy(C16, 1); });
+        lp->warp16_blocks[0] = blocks(lazy ? 1 : 7, [&] { return warp16_occupancy(C16, 0, lazy); });
+        lp->warp16_blocks[1] = blocks(lazy ? 2 : 8, [&] { return warp16_occupancy(C16, 1, lazy); });
         lp->warp16k_blocks[0] = blocks(3, [&] { return warp16k_occupancy(C16, 2); });
         lp->warp16k_blocks[1] = blocks(4, [&] { return warp16k_occupancy(C16, 4); });
         const int K = (flags & AGATHA_WARPS4) ? 4 : ((flags & AGATHA_WARPS2) ? 2 : 1);
@@ -540,7 +597,8 @@ void apply_narrow(agatha_ctx *ctx, LaunchPlan *lp, uint32_t flags) {
     if ((flags & AGATHA_ONE_FRAME) || !lp->lane16 || lp->plain || !lp->sort || lp->split || lp->groupk != 1 ||
         lp->half || lp->wide_w || lp->C16 != 24)
         return;
-    const int occ = plan_occupancy(ctx, 1, 20 / 4, [] { return occupancy_warp16_c<20, 2>(); });
+    const int occ = lp->lazy ? plan_occupancy(ctx, 1, 20 / 4, [] { return occupancy_warp16_c<20, 2>(); })
+                             : plan_occupancy(ctx, 7, 20 / 4, [] { return occupancy_step16_c<20, 2>(); });
     if (occ <= 0) return;
     lp->narrow_w = 32 * 20 - 2;
     lp->narrow_blocks = ctx->n_sm * occ;

@@ -79,6 +79,7 @@ struct Shape32 {
 struct LaunchPlan {
     int64_t n = 0;
     int plain = 0, sort = 1, fast = 1, use_graph = 1;
+    int lazy = 1;               // score kernels on lazy blocks, or with a test on every anti-diagonal
     int C = 16;                 // slots per lane that hold the widest band on one warp
     Shape32 shape32 = {16, 1};  // the int32 score kernel's
     int32_t warp_w_max = 0;
@@ -100,7 +101,7 @@ struct LaunchPlan {
     int64_t plain_blocks = 0;
     PlanKey key() const {
         return {plain, C | (shape32.C << 8) | (shape32.K << 16), C16 * lane16, regs_high,
-                sort | (prep_small(n) ? 2 : 0), fast, wide_w, warp_blocks, split,
+                sort | (prep_small(n) ? 2 : 0) | (lazy ? 0 : 4), fast, wide_w, warp_blocks, split,
                 split ? cls_var[0] | (cls_var[1] << 4) | (cls_var[2] << 8) | (cls_var[3] << 12) : 0,
                 split ? 1 : groupk, (split ? 0 : half) | (narrow_w > 0 ? 2 : 0)};
     }
@@ -139,7 +140,9 @@ int pick_slots16(int32_t w);
 Shape32 pick_shape32(int32_t w);
 cudaError_t launch_warp32(Shape32 k, const DevBatch *d, int blocks, cudaStream_t s, int fast, int list);
 int warp32_occupancy(Shape32 k);
-int warp16_occupancy(int C, int high);
+cudaError_t launch_step32(int C, const DevBatch *d, int blocks, cudaStream_t s, int fast, int list);
+int step32_occupancy(int C);
+int warp16_occupancy(int C, int high, int lazy);
 int warp16h_occupancy(int C16);   // two pairs per warp; 0 where none exists
 void apply_narrow(agatha_ctx *ctx, LaunchPlan *lp, uint32_t flags);
 int warp16k_occupancy(int C16, int K);
@@ -191,7 +194,7 @@ struct agatha_ctx {
     std::string tune_cache_path;
     std::mutex mu;                     // serialises align_batch calls
     // resident blocks of each kernel + 1 (0: not asked yet), see plan_occupancy
-    std::atomic<int> occupancy[6][8] = {};
+    std::atomic<int> occupancy[9][9] = {};
     std::mutex err_mu;
     std::string last_error, last_error_copy;
     agatha::Slot main;                 // buffers of agatha_align_batch

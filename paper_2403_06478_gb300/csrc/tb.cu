@@ -80,7 +80,7 @@ cudaError_t launch_tb16(int C, const DevBatch *d, const TbItem *items, int32_t n
     }
 }
 
-// fused score path and traceback on 16-bit lanes
+// fused score path and traceback on 16-bit lanes, from kept states
 cudaError_t launch_tbf16(int C, const DevBatch *d, const TbItem *items, int32_t n, uint8_t *dir, uint32_t *ops,
                          int32_t *ncig, int blocks, cudaStream_t s) {
     switch (C) {
@@ -97,6 +97,26 @@ int tbf16_occupancy(int C) {
         case 8: return occupancy_tbf16_c<8, 3>();
         case 16: return occupancy_tbf16_c<16, 2>();
         default: return occupancy_tbf16_c<24, 2>();
+    }
+}
+
+// the same with direction bytes
+cudaError_t launch_tbs16(int C, const DevBatch *d, const TbItem *items, int32_t n, int32_t *head, uint8_t *dir,
+                         uint32_t *ops, int32_t *ncig, int blocks, cudaStream_t s) {
+    switch (C) {
+        case 4: return launch_tbs16_c<4, 6>(d, items, n, head, dir, ops, ncig, blocks, s);
+        case 8: return launch_tbs16_c<8, 4>(d, items, n, head, dir, ops, ncig, blocks, s);
+        case 16: return launch_tbs16_c<16, 3>(d, items, n, head, dir, ops, ncig, blocks, s);
+        default: return launch_tbs16_c<24, 2>(d, items, n, head, dir, ops, ncig, blocks, s);
+    }
+}
+
+int tbs16_occupancy(int C) {
+    switch (C) {
+        case 4: return occupancy_tbs16_c<4, 6>();
+        case 8: return occupancy_tbs16_c<8, 4>();
+        case 16: return occupancy_tbs16_c<16, 3>();
+        default: return occupancy_tbs16_c<24, 2>();
     }
 }
 
@@ -182,8 +202,10 @@ extern "C" int agatha_align_cigar(agatha_ctx *ctx, const agatha_batch *batch, co
     const int C32 = pick_slots_per_lane(std::max<int32_t>(shape.max_w_all, 1));
     const int C16 = pick_slots16(std::max<int32_t>(shape.max_w_all, 1));
     const bool use16 = C16 > 0 && step_change_max(p) <= STEP16_MAX && !(flags & AGATHA_FORCE32);
-    const bool fused = use16 && lp.lane16 && !lp.wide_w && !(flags & (AGATHA_PLAIN | AGATHA_TB_TWO_PASS)) &&
-                       lazy_step_max(p) <= TRACE_STEP_MAX;
+    const bool fused = use16 && lp.lane16 && !lp.wide_w && !(flags & (AGATHA_PLAIN | AGATHA_TB_TWO_PASS));
+    // from kept states, unless lazy blocks have no room or the steps are too
+    // steep between two rebases; else from direction bytes
+    const bool states = lp.lazy && lazy_step_max(p) <= TRACE_STEP_MAX;
     Slot *sl = &ctx->main;
     if (fused) {
         if ((rc = stage_batch(ctx, batch, p, out, flags, s, lp))) return rc;
@@ -299,7 +321,8 @@ extern "C" int agatha_align_cigar(agatha_ctx *ctx, const agatha_batch *batch, co
                                          cudaMemcpyHostToDevice, s);
         if (e2 != cudaSuccess) return cuda_fail(ctx, e2, "copy traceback items");
         if (ctx->timing && (e2 = cudaEventRecord(ctx->ev_tb0, s)) != cudaSuccess) return cuda_fail(ctx, e2, "event");
-        const int occ = kind == K_INT32 ? tb_occupancy(C) : (kind == K_16 ? tb16_occupancy(C) : tbf16_occupancy(C));
+        const int occ = kind == K_INT32 ? tb_occupancy(C) : (kind == K_16 ? tb16_occupancy(C) :
+                        (states ? tbf16_occupancy(C) : tbs16_occupancy(C)));
         const int resident = ctx->n_sm * occ;
         for (size_t wv = 0; wv + 1 < begin.size(); ++wv) {
             const int64_t b = begin[wv], cnt = begin[wv + 1] - b;
@@ -308,13 +331,15 @@ extern "C" int agatha_align_cigar(agatha_ctx *ctx, const agatha_batch *batch, co
             uint8_t *dir = (uint8_t *)tb.dir.ptr;
             uint32_t *ops = (uint32_t *)tb.ops.ptr;
             int32_t *ncg = (int32_t *)tb.n_cigar.ptr;
-            if (kind == K_FUSED && wv > 0) {          // its queue heads are the slot's counters
+            if (kind == K_FUSED && states && wv > 0) {          // its queue heads are the slot's counters
                 for (int p = 0; p < TierQueue::PARTS; ++p)
                     if ((e2 = cudaMemsetAsync((int32_t *)sl->counters.ptr + CTR_HEAD + p * CTR_PART, 0,
                                               sizeof(int32_t), s)) != cudaSuccess)
                         return cuda_fail(ctx, e2, "clear queue heads");
             }
-            if (kind == K_FUSED) e2 = launch_tbf16(C, sl->d_desc, d_items + b, (int32_t)cnt, dir, ops, ncg, blocks, s);
+            if (kind == K_FUSED && !states)
+                e2 = launch_tbs16(C, sl->d_desc, d_items + b, (int32_t)cnt, head, dir, ops, ncg, blocks, s);
+            else if (kind == K_FUSED) e2 = launch_tbf16(C, sl->d_desc, d_items + b, (int32_t)cnt, dir, ops, ncg, blocks, s);
             else if (kind == K_16) e2 = launch_tb16(C, sl->d_desc, d_items + b, (int32_t)cnt, head, dir, ops, ncg, blocks, s);
             else e2 = launch_tb(C, sl->d_desc, d_items + b, (int32_t)cnt, head, dir, ops, ncg, blocks, s);
             if (e2 != cudaSuccess) return cuda_fail(ctx, e2, "traceback launch");
