@@ -967,12 +967,15 @@ struct WarpPair16 {
         return head_bounds_ok();
     }
     __device__ __forceinline__ bool head_bounds_ok() const {
-        const int64_t n = w + 6;
-        const int64_t lo = (int64_t)U_NEG - (int64_t)prm.b * n / 2 - oe2;
-        const int64_t hi = (int64_t)U_NEG + (int64_t)prm.a * n / 2;
-        const int64_t floor_virt = (int64_t)OFF - (int64_t)cold.kint * cold.Dp - gap_cost(prm, w + 3) -
-                                   (int64_t)prm.a * (w + 3);
-        return lo > 2 * (int64_t)(prm.a + prm.b + oe2) && hi + 4 * (int64_t)cold.Dp < floor_virt;
+        const int64_t lo = (int64_t)U_NEG - (int64_t)prm.b * (w + 6) / 2 - oe2;
+        return lo > 2 * (int64_t)(prm.a + prm.b + oe2) && head_rise_ok(w, cold.kint, cold.Dp);
+    }
+    // The upper half of it for a band of wh: all the lazy step asks for, whose
+    // scores fall no lower than they start (see lazy_head_ok).
+    __device__ __forceinline__ bool head_rise_ok(int32_t wh, int32_t kint, int32_t Dp) const {
+        const int32_t hi = (int32_t)U_NEG + prm.a * (wh + 6) / 2;
+        const int32_t floor_virt = OFF - kint * Dp - gap_cost(prm, wh + 3) - prm.a * (wh + 3);
+        return hi + 4 * Dp < floor_virt;
     }
 
     // ------------------------------------------------------- lazy blocks
@@ -999,9 +1002,9 @@ struct WarpPair16 {
     //    w + 1; PR = P where the frame ends with slot w, whose F then comes
     //    from past the last lane), so the shuffles' other end lanes need no
     //    mask.  Cells past the table's end, or beyond the virtual row and
-    //    column, feed nothing of the table (see step and head_bounds_ok).
-    // Minus infinity stays at U_NEG under the drift; every score is then at
-    // least U_NEG, because the drifting gap state never falls.
+    //    column, feed nothing of the table (see step and lazy_head_ok).
+    // Minus infinity stays at U_NEG under the drift, because the drifting gap
+    // state never falls (see lazy_head_ok).
     static constexpr int CKV = 6 * P / 4;                // 16-byte words of a checkpoint per lane
     // Most pairs of a block: what a block costs besides its steps (its maximum,
     // bounds and checkpoint, about 250 instructions) against what is taken again
@@ -1444,7 +1447,14 @@ struct WarpPair16 {
     __device__ __forceinline__ void lazy_rebase(int32_t m, int32_t r) {
         rebase(to_u(m), r, table_bits(r) | virtual_bits(r), table_bits(r - 1) | virtual_bits(r - 1));
     }
-    __device__ __forceinline__ bool lazy_head_ok() const { return head_bounds_ok(); }
+    // The lazy step in the head: cells beyond the virtual row and column must
+    // stay below the virtual cells.  They need no bound from below: no score of
+    // the lazy step falls under where it starts.  The second piece's states (the
+    // only piece's, if there is one) drift with their extension, so they never
+    // fall, and H is at least theirs; they start at U_NEG - q2 - e2 or above (what
+    // the masked step leaves off the table, or lazy_leave's clamp), so h - a - b,
+    // the lowest value formed, stays 3,000 above 0 for steps of up to 255.
+    __device__ __forceinline__ bool lazy_head_ok() const { return head_rise_ok(w, cold.kint, cold.Dp); }
     __device__ __forceinline__ uint32_t ring_address() const {
         return (uint32_t)__cvta_generic_to_shared(ck + 2 * CKV * 32);
     }
@@ -1608,12 +1618,6 @@ struct WarpPair16 {
             // the only one
             if (prm.q + prm.e > prm.q2 + prm.e2) { prm.q = prm.q2; prm.e = prm.e2; }
             blind = false;
-            // a band that covers the table may as well be the whole frame: the
-            // virtual cells then never leave it, and all such pairs run the
-            // same copy of the lazy step
-            const int32_t len = max(tlen, qlen);
-            cover = w >= len && len < NS - 1;
-            if (cover) w = NS - 1;
         }
         oe = prm.q + prm.e; oe2 = prm.q2 + prm.e2;
         j0 = (wk * G + lane) * C;
@@ -1628,6 +1632,16 @@ struct WarpPair16 {
                 cold.Dp = Dp;
                 cold.kint = kint;
                 cold.LOWCHK = (int32_t)U_NEG + (kint + 3) * Dp;
+            }
+            if constexpr (LAZY) {
+                // a band that covers the table may as well be the whole frame:
+                // the virtual cells then never leave it, and all such pairs run
+                // the same copy of the lazy step.  Not where the head of that
+                // wider band could not run lazily: such a pair has the masked
+                // step for its own head at most
+                const int32_t len = max(tlen, qlen);
+                cover = w >= len && len < NS - 1 && __any_sync(FULL, head_rise_ok(NS - 1, kint, Dp));
+                if (cover) w = NS - 1;
             }
         }
         base = 0;
