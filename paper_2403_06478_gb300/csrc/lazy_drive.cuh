@@ -97,6 +97,7 @@ __device__ __forceinline__ void lazy_edges(S &s, int32_t r0, int32_t n, int32_t 
 template <class S>
 __device__ __forceinline__ int32_t lazy_drive(S &s, bool use_fast) {
     constexpr int32_t NONE = INT_MIN;
+    constexpr int32_t LOW_UNTIL = S::TRACE ? 40 : 16;  // rebase when fewer anti-diagonals are left to it
     const DevParams &prm = s.prm;
     const int32_t w = s.w, tlen = s.tlen, qlen = s.qlen, last_r = s.last_r;
     // lazy blocks in the head too (by a vote: shared memory's values are not
@@ -128,7 +129,7 @@ __device__ __forceinline__ int32_t lazy_drive(S &s, bool use_fast) {
     for (;;) {
         if constexpr (S::REBASES) {
             // (one place for it: a second copy costs the instruction cache)
-            if (s.until_rebase < (S::TRACE ? 40 : 16) && r >= 0) {
+            if (s.until_rebase < LOW_UNTIL && r >= 0) {
                 s.lazy_rebase(open ? m0 : s.last_max(), r);
                 if (s.ovf) return r;
             }
@@ -209,8 +210,12 @@ __device__ __forceinline__ int32_t lazy_drive(S &s, bool use_fast) {
                 if (!stop) {
                     int32_t left = S::BLOCK_PAIRS;
                     if constexpr (S::REBASES) {
+                        // a rebase is due: no block, and so no checkpoint, lies
+                        // closer before one, because the pair may come back to
+                        // it with another place's maximum, to which it must not
+                        // rebase before the next masked step has taken its own
                         left = (u0 - (r - rs) - 4) >> 1;
-                        if (left < (S::TRACE ? 2 : 4)) break;  // a rebase is due
+                        if (left < (LOW_UNTIL - 4) / 2) break;
                     }
                     edge = cross || r + 2 > r_in;
                     n = (min(edge ? end : r_in, r < turn ? min(turn, end) : end) - r) >> 1;
