@@ -259,6 +259,7 @@ __device__ __forceinline__ int32_t lazy_drive(S &s, bool use_fast) {
                         break;
                     }
                     target = goal;
+                    exact_until = goal;                // (a crossing done before is undone)
                     seen = NONE;
                     fresh = 0;
                 } else {
