@@ -533,7 +533,9 @@ __device__ __forceinline__ void trace_segment(S &s, TraceWin<S> &W, int32_t seg,
     __syncwarp();
 }
 
-// Walk back from (s.end_t, s.end_q).  Returns the number of runs.
+// Walk back from (s.end_t, s.end_q).  Returns the number of runs, or -1 if no
+// move explains a score: the pair is then traced on int32 lanes like one that left
+// the 16-bit range, rather than by a path that is not its own.
 template <class S>
 __device__ __forceinline__ int32_t tb_trace(S &s, uint32_t *ops, int32_t cap) {
     using TW = TraceWin<S>;
@@ -620,13 +622,7 @@ __device__ __forceinline__ int32_t tb_trace(S &s, uint32_t *ops, int32_t cap) {
                 }
             }
             const int32_t n = at ? at : D;
-            if (pick < 0) {                       // (cannot be; keeps the walk moving)
-                runs.push(TB_OP_M, 1u, lane);
-                --t;
-                --q;
-                kind = -1;
-                continue;
-            }
+            if (pick < 0) return -1;              // (cannot be)
             runs.push((pick & 1) ? TB_OP_I : TB_OP_D, (uint32_t)n, lane);
             if (pick & 1) q -= n;
             else t -= n;
