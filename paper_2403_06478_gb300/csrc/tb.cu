@@ -152,7 +152,8 @@ int ensure_exact(agatha_ctx *ctx, DevBuf &b, size_t need) {
 // most of the device's free memory (a few GB kept back for everything else).
 int64_t dir_bytes_available(agatha_ctx *ctx) {
     const int64_t mine = (int64_t)ctx->tb.dir.cap;
-    if (ctx->ledger.budget > 0) return ctx->ledger.budget - (ctx->ledger.held - mine);
+    // (a buffer takes whole 256-byte granules)
+    if (ctx->ledger.budget > 0) return (ctx->ledger.budget - (ctx->ledger.held - mine)) & ~(int64_t)255;
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
         cudaGetLastError();
