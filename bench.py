@@ -480,7 +480,9 @@ def run_traceback(args):
         C = next(c for c in (4, 8, 16, 24, 32) if 32 * c - 1 >= w)
         kernel = f"tb_kernel<{C}>"
     if fused:                 # room for every anti-diagonal of each pair
-        table_bytes = int((batch.t_len[nonempty].astype(np.int64) + batch.q_len[nonempty] - 1).sum()) * 32 * C
+        # the states of every 32nd anti-diagonal
+        table_bytes = int(((batch.t_len[nonempty].astype(np.int64) + batch.q_len[nonempty] - 1) // 32 + 1).sum()) * (
+            384 * C + 16)
     else:
         table_bytes = sum(((int(r["mqe_t"]) + int(batch.q_len[i]) - 1) if r["reach_end"] else
                            (int(r["te"]) + int(r["qe"]))) + 1 for i, r in enumerate(res)

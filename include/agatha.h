@@ -298,12 +298,12 @@ int agatha_tune_variants(agatha_ctx *ctx, const agatha_params *params, int32_t w
  * AGATHA_FORCE32, a scoring beyond the 16-bit lanes, or a pair whose scores
  * leave their range use int32 lanes (two passes).  Every form gives the same
  * results and CIGARs.
- * Device memory: besides the score path's buffers, a table of 32*C bytes per
- * anti-diagonal (C the kernel's slots per lane for the batch's widest band: 4,
- * 8, 16 or 24 on 16-bit lanes, up to 32 on int32 lanes), for every
- * anti-diagonal of a pair in the fused form (its states), up to the end cell
- * in the two-pass form (its direction bytes), plus about 8 bytes per base of
- * the pair for the runs.
+ * Device memory: besides the score path's buffers, per pair a table of kept
+ * states, 384*C + 16 bytes for every 32 anti-diagonals or part of them, or of
+ * direction bytes, 32*C per anti-diagonal (in the two-pass form up to the end
+ * cell), C the kernel's slots per lane for the batch's widest band (4, 8, 16 or
+ * 24 on 16-bit lanes, up to 32 on int32 lanes); and about 8 bytes per base of the
+ * pair for the runs.
  * Pairs run in waves whose tables fit in the context's budget (else in the
  * device's free memory less min(1/16 of it, 4 GiB)); the context keeps the
  * largest table made until agatha_destroy.

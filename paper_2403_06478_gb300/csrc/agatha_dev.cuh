@@ -201,6 +201,12 @@ __host__ __device__ inline bool lazy_pays(const DevParams &p) {
 // which steps of at most this admit (rebase_interval: 44).
 constexpr int32_t TRACE_STEP_MAX = 300;
 
+// The fused traceback keeps the band's state of every 32nd anti-diagonal: six
+// arrays of 32 C 16-bit values, and 16 bytes of where it stands.  Room for those of
+// a pair with n anti-diagonals (the first is kept after at least 33 of them).
+__host__ __device__ constexpr int64_t trace_entry_bytes(int C) { return 384 * (int64_t)C + 16; }
+__host__ __device__ constexpr int64_t trace_bytes(int C, int64_t n) { return (n / 32 + 1) * trace_entry_bytes(C); }
+
 // One packed word of a stream, zero outside it (reads are clamped).
 __device__ __forceinline__ uint32_t load_word(const uint32_t *__restrict__ p, int64_t n_words,
                                               int64_t i) {

@@ -637,11 +637,9 @@ __device__ __forceinline__ int32_t tb_trace(S &s, uint32_t *ops, int32_t cap) {
     return runs.n;
 }
 
-// The memory of an item has room for the direction table of every
-// anti-diagonal of the pair (tlen + qlen - 1 rows of 32 C bytes), of which the
-// states take three eighths, and its run scratch for tlen + qlen runs.  A pair
-// that leaves the 16-bit range goes to the int32 score kernel's list and gets
-// n = -1.
+// The memory of an item has room for the states of every anti-diagonal of the pair
+// (trace_bytes), and its run scratch for tlen + qlen runs.  A pair that leaves the
+// 16-bit range goes to the int32 score kernel's list and gets n = -1.
 template <int C>
 using TracePair = WarpPair16<C, false, false, false, true, 1, true, false, 32, true, true>;
 template <int C>

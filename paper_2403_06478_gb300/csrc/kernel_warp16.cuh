@@ -1388,6 +1388,7 @@ struct WarpPair16 {
     // drifting form (rs: its start) or, from the masked step, the plain one.
     // An entry is the checkpoint's words and one of {rs, base, drifting}.
     static constexpr int TRACE_ENTRY = CKV * 32 + 1;     // 16-byte words
+    static_assert(!TRACE_ || TRACE_ENTRY * 16 == trace_entry_bytes(C), "the room the host reserves");
     __device__ __forceinline__ int32_t first_r() const { return 1 + (w & 1); }
     __device__ __forceinline__ bool trace_mark(int32_t r) const {
         return r > first_r() && ((r - first_r()) & 31) == 0;

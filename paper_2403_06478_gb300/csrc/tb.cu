@@ -1,18 +1,20 @@
 // Traceback entry point: the CIGAR of each extension of a host batch.
 //
-// 1. The score path runs as in agatha_align_batch (same plan, tuning and
-//    results); it leaves the batch staged on the device.
-// 2. Each pair's end cell follows from its result: the query end when the
-//    extension reached it, else the cell of the maximum.  Pairs with an end
-//    cell become traceback items, ordered by predicted work (anti-diagonals
-//    up to the end x band width), longest first.
-// 3. A direction table takes (r_end + 1) x 32C bytes per pair (C: slots per
-//    lane of the warp kernel for the batch's widest band).  Items run in
-//    waves whose tables fit the device memory this call may use; each wave
-//    is one persistent launch of a traceback kernel (kernel_tb.cuh): the
-//    16-bit one when the score path may use 16-bit lanes, else (and for the
-//    pairs whose scores leave the 16-bit range, found from the run counts)
-//    the int32 one.
+// 1. Two forms.  Fused, on 16-bit lanes (the default where they apply): one
+//    kernel aligns each pair and traces it, from band states kept on the way or
+//    from direction bytes.  Two passes: the score path runs as in
+//    agatha_align_batch (same plan, tuning and results) and leaves the batch
+//    staged on the device; each pair's end cell follows from its result (the
+//    query end when the extension reached it, else the cell of the maximum).
+// 2. The pairs become traceback items, ordered by predicted work (anti-diagonals
+//    x band width; in two passes up to the end cell, and only pairs that have
+//    one), longest first.
+// 3. Items run in waves whose tables fit the device memory this call may use:
+//    kept states take trace_bytes per pair, direction bytes 32C per anti-diagonal
+//    (C: slots per lane of the kernel for the batch's widest band).  Each wave
+//    is one persistent launch of a kernel of kernel_tb.cuh; the pairs whose scores
+//    leave the 16-bit range, found from the run counts, take the int32 score and
+//    traceback kernels after the others.
 // 4. The run counts come back to the host, which lays the CIGARs out in
 //    input order; a gather kernel reverses each pair's runs into one dense
 //    device array, copied to the caller's buffer in one transfer.
@@ -291,16 +293,19 @@ extern "C" int agatha_align_cigar(agatha_ctx *ctx, const agatha_batch *batch, co
         NvtxRange waves(kind == K_FUSED ? "traceback waves (fused)" :
                         (kind == K_16 ? "traceback waves (16-bit)" : "traceback waves (int32)"));
         const int C = kind == K_INT32 ? C32 : C16;
-        const int64_t row = 32 * C;
+        const auto table = [&](const TbItem &it) {
+            const int64_t steps = (int64_t)it.end_t + it.end_q + 1;
+            return kind == K_FUSED && states ? trace_bytes(C, steps) : steps * 32 * C;
+        };
         int64_t total = 0, largest = 0;
         for (const TbItem &it : list) {
-            const int64_t bytes = ((int64_t)it.end_t + it.end_q + 1) * row;
+            const int64_t bytes = table(it);
             total += bytes;
             largest = std::max(largest, bytes);
         }
         int64_t cap = std::min(total, dir_bytes_available(ctx));
         if (cap < largest)
-            return set_error(ctx, AGATHA_ENOMEM, "a direction table of %lld bytes does not fit in %lld",
+            return set_error(ctx, AGATHA_ENOMEM, "a pair's table of %lld bytes does not fit in %lld",
                              (long long)largest, (long long)cap);
         int r2 = ensure_exact(ctx, tb.dir, (size_t)cap);
         if (r2) return r2;
@@ -308,7 +313,7 @@ extern "C" int agatha_align_cigar(agatha_ctx *ctx, const agatha_batch *batch, co
         std::vector<int64_t> begin;
         int64_t used = cap;                      // forces a new wave at the first item
         for (size_t k = 0; k < list.size(); ++k) {
-            const int64_t bytes = ((int64_t)list[k].end_t + list[k].end_q + 1) * row;
+            const int64_t bytes = table(list[k]);
             if (used + bytes > cap) {
                 begin.push_back((int64_t)k);
                 used = 0;

@@ -1,4 +1,6 @@
-"""The traceback's memory under a budget."""
+"""The traceback's memory under a budget: its tables take what is left of it, and the
+kept states of the fused form ask for what they take, not for a direction byte per
+band slot and anti-diagonal."""
 import numpy as np
 import pytest
 
@@ -33,3 +35,40 @@ def test_waves_under_any_budget(flags, odd):
         assert small.last_traceback_info()["waves"] > 1
     assert A.results_equal(r1, r2).size == 0
     assert np.array_equal(o1, o2) and np.array_equal(c1, c2)
+
+
+def _states(batch, C=16):
+    n = batch.q_len.astype(np.int64) + batch.t_len - 1
+    return (n // 32 + 1) * (384 * C + 16)
+
+
+@pytest.mark.parametrize("lengths,waves", [([40000], 1), ([9000] * 12, 1), ([9000] * 12, 3)])
+def test_a_budget_for_the_states_is_enough(lengths, waves):
+    batch = _batch(lengths)
+    states = _states(batch)
+    rows = (batch.q_len.astype(np.int64) + batch.t_len - 1) * 512
+    # besides the tables: results, sequences, runs and lists
+    rest = (1 << 20) + 10 * int((batch.q_len.astype(np.int64) + batch.t_len).sum())
+    room = int(states.sum()) if waves == 1 else int(states.max()) * -(-len(lengths) // waves)
+    assert waves > 1 or room + rest < rows.sum()
+    ref = O.align_batch(batch)
+    want, _ = O.traceback_batch(batch, ref)
+    with A.Context(0, mem_budget_bytes=room + rest) as ctx:
+        res, off, cig = ctx.align_cigar(A.pack_batch(batch), batch.scoring)
+        info = ctx.last_traceback_info()
+    assert info["waves"] <= waves and info["fused"] == batch.n_pairs, info
+    assert A.results_equal(res, ref, O.COMPARE_FIELDS).size == 0
+    assert all(np.array_equal(cig[off[i]:off[i + 1]], want[i]) for i in range(batch.n_pairs))
+
+
+@pytest.mark.parametrize("w", [100, 200, 500, 750])
+def test_every_length_around_a_state(w):
+    """Pairs whose last anti-diagonals lie around the first states kept."""
+    lengths = list(range(1, 70)) + [4 * w]
+    batch = _batch(lengths, w)
+    ref = O.align_batch(batch)
+    want, _ = O.traceback_batch(batch, ref)
+    with A.Context(0) as ctx:
+        res, off, cig = ctx.align_cigar(A.pack_batch(batch), batch.scoring)
+    assert A.results_equal(res, ref, O.COMPARE_FIELDS).size == 0
+    assert all(np.array_equal(cig[off[i]:off[i + 1]], want[i]) for i in range(batch.n_pairs))
