@@ -106,6 +106,11 @@ __host__ __device__ inline uint64_t predicted_cells(int32_t tlen, int32_t qlen, 
     return (uint64_t)(tlen + qlen) * (uint64_t)(w + 1) / 2 + 1;
 }
 
+// The local extension's row key of a cell: 1024 times its score (below 2^20), from
+// the drifting H and zk = -1024 z of the drifting zero z.  The drift may pass 2^21,
+// so the product wraps and only the difference is in range: unsigned arithmetic.
+__host__ __device__ inline int32_t row_key(int32_t H, uint32_t zk) { return (int32_t)((uint32_t)H * 1024u + zk); }
+
 // Largest initial score of the local extension (keeps every score in int32
 // beside the length bound of pair_valid).
 constexpr int32_t LOCAL_H0_MAX = 1 << 24;

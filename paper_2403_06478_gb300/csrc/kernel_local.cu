@@ -358,7 +358,7 @@ struct LocalRows {
         }
         const int32_t nab = -(prm.a + prm.b);
         const int32_t live = z - 2 * prm.e2 - prm.q2;  // h of r - 2 above this: a live cell
-        const int32_t zk = -z * 1024;
+        const uint32_t zk = 0u - (uint32_t)z * 1024u;
 #pragma unroll
         for (int i = 0; i < C; ++i) {
             const int p = ODD ? C - 1 - i : i;
@@ -388,7 +388,7 @@ struct LocalRows {
                 Fo[p] = max(Fin, h);
                 Hd[p] = h;
             }
-            int32_t key = H * 1024 + zk;
+            int32_t key = row_key(H, zk);
             if constexpr (MASK) key = p >= lo ? key : LOW;
             RM[p] = __viaddmax_s32(RMin, 1, key);
         }
