@@ -68,7 +68,8 @@ extern "C" {
                                      through the masked edge path (testing)  */
 #define AGATHA_REGS_HIGH   0x80u  /* 16-bit kernel at its second register
                                      budget (the first is the default; another
-                                     number of resident blocks per SM)        */
+                                     number of warps per SM; bands of 512 to
+                                     767 may have one budget only)            */
 #define AGATHA_NO_TUNE     0x100u /* ignore the autotuner for this call       */
 #define AGATHA_TB_TWO_PASS 0x200u /* agatha_align_cigar: score path, then a
                                      separate traceback pass (not fused)    */
@@ -237,7 +238,8 @@ int64_t agatha_band_cells(int32_t tlen, int32_t qlen, int32_t w);
  * four length classes by predicted band cells (the Section 4.5 model:
  * >= 2^25, >= 2^23, >= 2^21, smaller; up to 4096 pairs each) is timed with
  * each variant (0: 16-bit lanes, 1: 16-bit lanes at the second register
- * budget, 2: int32 lanes).  The batch (up to 131072 of its pairs) is then
+ * budget - not where that is the same kernel, bands of 512 to 767 -, 2: int32
+ * lanes).  The batch (up to 131072 of its pairs) is then
  * timed as one launch of each 16-bit variant (and of int32 lanes if a class
  * preferred them) and, if the classes disagree, with one launch per class.  The fastest plan
  * is kept (anything but one launch of variant 0 must win by 2% on a class's

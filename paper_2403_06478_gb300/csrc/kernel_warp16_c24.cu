@@ -1,6 +1,6 @@
 // Instantiations of the 16-bit packed-lane warp kernel for 24 band slots per
-// lane (w <= 767), at two register budgets (warps per scheduler): the
-// autotuner picks one per length class.
+// lane (w <= 767) at two warps per scheduler: more do not fit the registers, so
+// both of the plan's budgets are this one.
 #include "kernel_tb.cuh"
 
 namespace agatha {

@@ -3,7 +3,8 @@
 // The paper picks its slice width and subwarp size by sweeping them on its
 // datasets (Sections 5.5 and 5.7).  Here the knobs are those of the warp
 // kernels: 16-bit packed lanes or int32 lanes, the register budget of the
-// 16-bit kernel (fewer resident warps, more registers each), and how many
+// 16-bit kernel (fewer resident warps, more registers each; not with 24 slots on
+// lazy blocks, whose two budgets are one), and how many
 // warps share one pair's band (1, 2 or 4: lanes per pair, for the classes of
 // long pairs, whose anti-diagonals then take fewer steps of each warp).  They are
 // chosen per length class, by measurement, the first time a host batch
@@ -87,9 +88,16 @@ LaunchPlan single_variant(LaunchPlan vp, int variant) {
     return vp;
 }
 
+// Whether the two register budgets are one kernel: with 24 slots on lazy blocks
+// only two warps per scheduler fit.  The second one is then the first.
+bool one_budget(const LaunchPlan &lp) { return lp.lazy && lp.C16 == 24; }
+int8_t own_variant(const LaunchPlan &lp, int8_t v) { return v == VAR_16_HIGHREG && one_budget(lp) ? VAR_16 : v; }
+
 // Whether this plan can run a variant (the 2- and 4-warp kernels exist for
-// the 16- and 24-slot bands only, two pairs per warp for the 4-slot band).
+// the 16- and 24-slot bands only, two pairs per warp for the 4-slot band) that is
+// a kernel of its own.
 bool variant_available(const LaunchPlan &lp, int v) {
+    if (v == VAR_16_HIGHREG) return !one_budget(lp);
     if (v == VAR_16_HALF) return lp.warp16h_blocks > 0;
     const int K = variant_warps(v);
     return K == 1 || lp.warp16k_blocks[K == 4] > 0;
@@ -164,7 +172,7 @@ int tune_run(agatha_ctx *ctx, const agatha_batch *b, const DevParams &p, uint32_
     //    16-bit variant (samples of a class can hide a few percent that the
     //    whole batch shows) and of int32 lanes if a class preferred them, and
     //    as one launch per class; the fastest plan is kept
-    wins[VAR_16_HIGHREG] = true;
+    wins[VAR_16_HIGHREG] = variant_available(lp, VAR_16_HIGHREG);
     SubBatch whole(b, all, kTuneSplitPairs);
     float best = 0.f;
     int best_v = VAR_16;
@@ -241,6 +249,8 @@ int tune_apply(agatha_ctx *ctx, const agatha_batch *batch, const DevParams &p, u
         ctx->tune_table[key] = choice;
         tune_save(ctx);
     }
+    // (a file may name the second budget where it is the first)
+    for (int8_t &v : choice.var) v = own_variant(*lp, v);
     if (!choice.split) {                        // one launch of one variant
         const int v = choice.var[0];
         if (!variant_available(*lp, v)) return AGATHA_OK;
