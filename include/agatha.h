@@ -244,8 +244,9 @@ int64_t agatha_band_cells(int32_t tlen, int32_t qlen, int32_t w);
  * preferred them) and, if the classes disagree, with one launch per class.  The fastest plan
  * is kept (anything but one launch of variant 0 must win by 2% on a class's
  * sample and by 1% on the batch), per context
- * and in tune_cache_path (one line per key, read at agatha_init).  Every
- * variant gives bit-identical results.  agatha_tune_variants writes what was
+ * and in tune_cache_path (one line per key, read at agatha_init, and one that
+ * names the build; a file of another build is not read, and written over at the
+ * next tuning).  Every variant gives bit-identical results.  agatha_tune_variants writes what was
  * tuned for `params` (band half-width w_max: the widest effective band of
  * the batches) into variants[0..4]: the four class variants (all equal when
  * one launch is used), then 1 if one launch per class is used.  AGATHA_OK,

@@ -50,9 +50,9 @@ def _inputs_digest() -> str:
     return h.hexdigest()
 
 
-def _compile(src: str, verbose: bool) -> str:
+def _compile(src: str, verbose: bool, build_id: str) -> str:
     obj = os.path.join(BUILD_DIR, os.path.basename(src) + ".o")
-    cmd = [_nvcc()] + ARCH + NVCC_FLAGS + ["-c", src, "-o", obj]
+    cmd = [_nvcc()] + ARCH + NVCC_FLAGS + [f'-DAGATHA_BUILD_ID="{build_id}"', "-c", src, "-o", obj]
     if verbose:
         cmd += ["-Xptxas", "-v"]
     res = subprocess.run(cmd, capture_output=True, text=True)
@@ -85,7 +85,7 @@ def _build_locked(force: bool, verbose: bool) -> str:
     srcs = sources()
     workers = max(1, min(len(srcs), os.cpu_count() or 1))
     with cf.ThreadPoolExecutor(max_workers=workers) as ex:
-        objs = list(ex.map(lambda s: _compile(s, verbose), srcs))
+        objs = list(ex.map(lambda s: _compile(s, verbose, digest[:16]), srcs))
     tmp = LIB + f".tmp{os.getpid()}"
     cmd = [_nvcc()] + ARCH + ["-shared", "-o", tmp] + objs + ["-cudart", "static", "-lpthread"]
     res = subprocess.run(cmd, capture_output=True, text=True)

@@ -18,10 +18,13 @@
 // default variant).
 // Every variant computes the same exact results, so the choice only moves
 // time.  Choices are kept per context and, with a cache path, in a text file
-// (one line per key: the key, the four class variants and the split flag).
+// (one line per key: the key, the four class variants and the split flag; then a
+// line with the build that measured them, whose file another build leaves unread:
+// its variants are other kernels.  A file without that line is taken as it is).
 #include <algorithm>
 #include <cstdio>
 #include <fstream>
+#include <map>
 #include <sstream>
 #include <string>
 #include <vector>
@@ -31,6 +34,11 @@
 namespace agatha {
 
 namespace {
+
+// The build: a digest of the sources, given by the build script.
+#ifndef AGATHA_BUILD_ID
+#define AGATHA_BUILD_ID "unnamed"
+#endif
 
 constexpr int64_t kTuneMaxPairs = 4096;       // per class, to pick its variant
 constexpr int64_t kTuneSplitPairs = 131072;   // of the whole batch, to decide the plan
@@ -54,6 +62,7 @@ void tune_save(agatha_ctx *ctx) {
             for (int8_t v : kv.second.var) f << ' ' << (int)v;
             f << ' ' << (int)kv.second.split << '\n';
         }
+        f << "build " << AGATHA_BUILD_ID << '\n';
     }
     std::rename(tmp.c_str(), ctx->tune_cache_path.c_str());
 }
@@ -209,11 +218,17 @@ void tune_load(agatha_ctx *ctx) {
     if (ctx->tune_cache_path.empty()) return;
     std::ifstream f(ctx->tune_cache_path);
     std::string line;
+    std::map<std::string, TuneChoice> table;
     while (f && std::getline(f, line)) {
         std::istringstream is(line);
         std::string key;
         TuneChoice v;
         bool ok = (bool)(is >> key);
+        if (ok && key == "build") {
+            std::string id;
+            if ((is >> id) && id != AGATHA_BUILD_ID) return;
+            continue;
+        }
         for (int c = 0; ok && c < N_CLASSES; ++c) {
             int x = -1;
             ok = (bool)(is >> x) && x >= 0 && x < N_VARIANTS;
@@ -222,8 +237,9 @@ void tune_load(agatha_ctx *ctx) {
         int sp = -1;
         ok = ok && (bool)(is >> sp) && (sp == 0 || sp == 1);
         v.split = (int8_t)sp;
-        if (ok) ctx->tune_table[key] = v;        // malformed lines are ignored
+        if (ok) table[key] = v;                  // malformed lines are ignored
     }
+    ctx->tune_table.insert(table.begin(), table.end());
 }
 
 int tune_apply(agatha_ctx *ctx, const agatha_batch *batch, const DevParams &p, uint32_t flags,
