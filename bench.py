@@ -365,7 +365,7 @@ def run_local(args):
         "gpu_launches": args.steps * ((1 if n <= 4096 else 3) + 2),      # prep, the local kernels
         "roofline": {"bound": "alu", "achieved": round(achieved, 3), "peak": round(int_peak, 3),
                      "unit": "Tops/s", "frac": round(achieved / int_peak, 4), "traffic": None,
-                     "kernel": f"local_align_kernel<{C}>", "kernel_ms": round(t_ms, 3),
+                     "kernel": f"local_rows_kernel<{C}>", "kernel_ms": round(t_ms, 3),
                      "ops_per_cell": OPS_PER_CELL_LOCAL,
                      "peak_basis": f"{n_sm} SMs x 128 int32 lanes x {sm_max_mhz:.0f} MHz ({peak_kind})"},
         "clocks": clocks,

@@ -603,8 +603,10 @@ struct LazyPair32 {
     }
 };
 
-// Warps per scheduler (K > 1: groups per SM) the registers are cut for: six arrays of C values and
-// no spills in the lazy loop, within what the checkpoints' shared memory admits.
+// Warps per scheduler (K > 1: groups per SM) the registers are cut for: the faster
+// count on the workloads, within what the checkpoints' shared memory admits.  Not
+// all of it fits: <4, 1> spills 8 bytes, <8, 1> 74, <8, 3> 152, <12, 3> 206 (whose 9
+// warps leave 168 registers a thread, since one scheduler holds three), <16, 1> none.
 template <int C, int K>
 __host__ __device__ constexpr int warp32_blocks() {
     return K > 1 ? (C <= 8 ? 5 : 3) : (C <= 4 ? 5 : (C <= 8 ? 4 : 2));

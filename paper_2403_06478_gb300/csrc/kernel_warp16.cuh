@@ -1154,10 +1154,10 @@ struct WarpPair16 {
                 // pair's registers for lazy_edges; the row's slot moved down
                 // before the first anti-diagonal, the column's moves up
                 // before the second
-                g.dt -= g.step;
+                --g.dt;
                 ring_store(g.ring, g.dt, Hev);
                 ring_store(g.ring + 2 * RING, g.dq, Hev);
-                g.dq += g.step;
+                ++g.dq;
                 ring_store(g.ring + 4 * P, g.dt, Hod);
                 ring_store(g.ring + 4 * P + 2 * RING, g.dq, Hod);
                 g.ring += 8 * P;

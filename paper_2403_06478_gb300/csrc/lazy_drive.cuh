@@ -24,8 +24,7 @@ struct Cold16 {
 
 // Where the last row's and column's cells sit, as slots of this lane (on: the
 // block may hold such cells; uniform), and the ring's shared address.
-// step: 1 (0: the same lanes keep every anti-diagonal, for the traceback).
-struct LazyEdge { int32_t on, dt, dq; uint32_t ring; int32_t step; };
+struct LazyEdge { int32_t on, dt, dq; uint32_t ring; };
 
 // Pairs of anti-diagonals the next block may hold: n, 16, 8, 4 or 2 (0: none) such
 // that no anti-diagonal of it can fire the Z-drop test.  g, m, mu: an upper
@@ -281,7 +280,7 @@ __device__ __forceinline__ int32_t lazy_drive(S &s, bool use_fast) {
             }
             const bool rim = edge && target == NONE;
             const int32_t B = floor_div2(r - w);
-            LazyEdge g{__reduce_max_sync(FULL, rim ? 1 : 0), tlen - 1 - B - s.j0, r - qlen + 1 - B - s.j0, ring, 1};
+            LazyEdge g{__reduce_max_sync(FULL, rim ? 1 : 0), tlen - 1 - B - s.j0, r - qlen + 1 - B - s.j0, ring};
             if (!s.owns()) g.dt = g.dq = -(1 << 20);
 #pragma unroll 1
             for (int32_t done = 0;;) {

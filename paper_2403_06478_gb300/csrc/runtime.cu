@@ -550,8 +550,8 @@ int make_plan(agatha_ctx *ctx, const DevParams &p, const BatchShape &shape, uint
                                                [&] { return warp32_occupancy(s32); })
                               : plan_occupancy(ctx, 6, C32 / 4, [&] { return step32_occupancy(C32); }));
     // 16-bit packed lanes when the band fits and one anti-diagonal changes a
-    // score by at most 255 (the 16-bit kernel then still rebases at least
-    // every 50 anti-diagonals)
+    // score by at most 255 (the 16-bit kernel then rebases every 34
+    // anti-diagonals or less often: the drift of the lazy blocks counts too)
     lp->C16 = pick_slots16(shape.max_w_all);
     lp->lane16 = !(flags & AGATHA_FORCE32) && lp->C16 > 0 && step_change_max(p) <= STEP16_MAX && !lp->wide_w;
     lp->regs_high = (flags & AGATHA_REGS_HIGH) ? 1 : 0;
