@@ -108,7 +108,7 @@ extern "C" int agatha_align_batch_noalloc(const agatha_batch *batch, const agath
         if (wide_w > plain_kernel_max_w()) return AGATHA_ENOTSUP;
     }
     const Shape32 shape = pick_shape32(w_plan < warp_w_max ? w_plan : warp_w_max);
-    const bool lazy = lazy_pays(p);
+    const bool lazy = lazy32_pays(p, shape, C, batch->n_pairs, ds->n_sm);
     const int blocks = ds->n_sm * (lazy ? warp32_occupancy(shape) : step32_occupancy(C));
 
     DevBatch desc;

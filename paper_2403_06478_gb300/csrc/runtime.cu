@@ -163,6 +163,18 @@ Shape32 pick_shape32(int32_t w) {
     return {w <= 734 ? 8 : 12, 3};
 }
 
+// Whether the int32 score kernel runs on lazy blocks (shape k) or tests every
+// anti-diagonal (C slots per lane, one warp per pair).  Where the scoring leaves
+// lazy blocks no room, three warps per pair are still the shorter chain as long as
+// the batch does not fill the chip with them: one wave of their groups, two against
+// 32 slots per lane, which spill.  (Pairs of 3 kbp, ONT scoring at a threshold of
+// 30, lazy kernel and the other: w = 600, one wave 760, 600 pairs 10.2 and 11.4 ms,
+// 1,500 20.4 and 16.9; w = 1,000, one wave 456, 1 pair 6.4 and 13.5, 600 17.0 and
+// 19.6, 1,500 35.2 and 33.0.)
+bool lazy32_pays(const DevParams &p, Shape32 k, int C, int64_t n, int n_sm) {
+    return lazy_pays(p) || (k.K == 3 && n <= (int64_t)n_sm * (k.C == 8 ? 5 : 3) * (C == 32 ? 2 : 1));
+}
+
 cudaError_t launch_warp32(Shape32 k, const DevBatch *d, int blocks, cudaStream_t s, int fast, int list) {
     switch (k.C * 4 + k.K) {
         case 4 * 4 + 1: return launch_warp_c<4, 1>(d, blocks, s, fast, list);
@@ -206,8 +218,8 @@ int step32_occupancy(int C) {
 
 // The int32 score kernel of a plan.
 static cudaError_t launch_plan32(const LaunchPlan &lp, const DevBatch *d, cudaStream_t s, int list) {
-    return lp.lazy ? launch_warp32(lp.shape32, d, lp.warp_blocks, s, lp.fast, list)
-                   : launch_step32(lp.C, d, lp.warp_blocks, s, lp.fast, list);
+    return lp.lazy32 ? launch_warp32(lp.shape32, d, lp.warp_blocks, s, lp.fast, list)
+                     : launch_step32(lp.C, d, lp.warp_blocks, s, lp.fast, list);
 }
 
 // 16-bit kernel with C slots per lane at its default budget of registers or
@@ -545,8 +557,9 @@ int make_plan(agatha_ctx *ctx, const DevParams &p, const BatchShape &shape, uint
     const Shape32 s32 = lp->shape32;
     const int C32 = lp->C;
     lp->lazy = lazy_pays(p) ? 1 : 0;
+    lp->lazy32 = lazy32_pays(p, s32, C32, shape.n, ctx->n_sm) ? 1 : 0;
     lp->warp_blocks =
-        ctx->n_sm * (lp->lazy ? plan_occupancy(ctx, 0, s32.K == 1 ? s32.C / 4 : (s32.C == 8 ? 5 : 6),
+        ctx->n_sm * (lp->lazy32 ? plan_occupancy(ctx, 0, s32.K == 1 ? s32.C / 4 : (s32.C == 8 ? 5 : 6),
                                                [&] { return warp32_occupancy(s32); })
                               : plan_occupancy(ctx, 6, C32 / 4, [&] { return step32_occupancy(C32); }));
     // 16-bit packed lanes when the band fits and one anti-diagonal changes a

@@ -80,6 +80,7 @@ struct LaunchPlan {
     int64_t n = 0;
     int plain = 0, sort = 1, fast = 1, use_graph = 1;
     int lazy = 1;               // score kernels on lazy blocks, or with a test on every anti-diagonal
+    int lazy32 = 1;             // the same for the int32 one
     int C = 16;                 // slots per lane that hold the widest band on one warp
     Shape32 shape32 = {16, 1};  // the int32 score kernel's
     int32_t warp_w_max = 0;
@@ -101,7 +102,7 @@ struct LaunchPlan {
     int64_t plain_blocks = 0;
     PlanKey key() const {
         return {plain, C | (shape32.C << 8) | (shape32.K << 16), C16 * lane16, regs_high,
-                sort | (prep_small(n) ? 2 : 0) | (lazy ? 0 : 4), fast, wide_w, warp_blocks, split,
+                sort | (prep_small(n) ? 2 : 0) | (lazy ? 0 : 4) | (lazy32 ? 0 : 8), fast, wide_w, warp_blocks, split,
                 split ? cls_var[0] | (cls_var[1] << 4) | (cls_var[2] << 8) | (cls_var[3] << 12) : 0,
                 split ? 1 : groupk, (split ? 0 : half) | (narrow_w > 0 ? 2 : 0)};
     }
@@ -138,6 +139,7 @@ int validate_host_batch(agatha_ctx *ctx, const agatha_batch *b, const DevParams 
 int pick_slots_per_lane(int32_t w);
 int pick_slots16(int32_t w);
 Shape32 pick_shape32(int32_t w);
+bool lazy32_pays(const DevParams &p, Shape32 k, int C, int64_t n, int n_sm);
 cudaError_t launch_warp32(Shape32 k, const DevBatch *d, int blocks, cudaStream_t s, int fast, int list);
 int warp32_occupancy(Shape32 k);
 cudaError_t launch_step32(int C, const DevBatch *d, int blocks, cudaStream_t s, int fast, int list);

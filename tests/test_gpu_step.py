@@ -138,3 +138,29 @@ def test_a_low_threshold_costs_no_more_for_cigars(ctx):
             t.append(ctx.last_traceback_ms())
         ms[z] = sorted(t)[2]
     assert ms[30] < 2.6 * ms[-1], ms
+
+
+@pytest.mark.parametrize("w,n", [(600, 1), (600, 700), (600, 800), (1000, 1), (1000, 900), (1000, 950)])
+def test_three_warps_below_the_line(ctx, w, n):
+    """int32 lanes on bands of more than 511: three warps per pair up to one wave
+    of them (two for the widest), one warp beyond."""
+    rng = np.random.default_rng(n)
+    qs = [rng.integers(0, 4, 640 if i else 1300, dtype=np.uint8) for i in range(n)]
+    ts = [W._mutate_chunk(rng, q, np.array([len(q)], np.int32), W.ErrorModel(0.02, 0.01, 0.01))[0] for q in qs]
+    batch = W.from_pairs(qs, ts, W.replace(W.ONT_SCORING, w=w, zdrop=30))
+    got = A.agatha_align_batch(ctx, batch, flags=A.AGATHA_FORCE32)
+    assert A.results_equal(got, O.align_batch(batch), O.COMPARE_FIELDS).size == 0
+
+
+def test_a_lone_wide_pair_keeps_three_warps(ctx):
+    """4.5 times the lazy time on the masked step of three warps, 9.5 on one warp."""
+    ms = {}
+    for z in (30, -1):
+        s = W.replace(W.ONT_SCORING, w=1000, zdrop=z)
+        pb = A.pack_batch(_accurate(1, 3000, s))
+        t = []
+        for _ in range(7):
+            ctx.align_host(pb, s)
+            t.append(ctx.last_kernel_ms())
+        ms[z] = sorted(t)[2]
+    assert ms[30] < 6.5 * ms[-1], ms
