@@ -355,13 +355,12 @@ typedef struct {
     int32_t linger_us;          /* hold a short head batch this long for   */
                                 /* more requests; 0: launch at once        */
     uint32_t launch_flags;      /* plan of every launch: 0 = the context's */
-                                /* autotuned plan; AGATHA_WARPS2 or        */
-                                /* AGATHA_WARPS4 = 2 or 4 warps per pair   */
-                                /* (shorter latency for long pairs; a     */
-                                /* launch whose band has no such kernel    */
-                                /* runs one warp per pair), with or       */
-                                /* without AGATHA_REGS_HIGH; any other bit */
-                                /* is EINVAL                               */
+                                /* autotuned plan (the fastest measured);  */
+                                /* AGATHA_WARPS2 or AGATHA_WARPS4 = 2 or 4 */
+                                /* warps per pair (a launch whose band has */
+                                /* no such kernel runs one warp per pair), */
+                                /* with or without AGATHA_REGS_HIGH; any   */
+                                /* other bit is EINVAL                     */
 } agatha_serve_config;
 
 typedef struct {

@@ -2,8 +2,8 @@
 // for scorings whose Z-drop threshold leaves the lazy blocks no room
 // (lazy_pays in agatha_dev.cuh).  There lazy_drive would run its masked step,
 // which keeps one copy of the code for both parities and every edge, nearly
-// everywhere: about 350 instructions per 16-slot anti-diagonal against the 114
-// of the bulk step here.  One GB300, whole calls, lazy blocks against this
+// everywhere: 250 ALU instructions per 16-slot anti-diagonal against the 114 of
+// the bulk step here.  One GB300, whole calls, lazy blocks against this
 // kernel at a threshold of 30 with minimap2's ONT scoring: 8,000 pairs of 600 bp
 // at w = 100 4.21 and 1.37 ms, 1,500 ONT-like pairs of 5 kbp at w = 500 17.2 and
 // 6.2, int32 lanes 27.5 and 15.1; the assembly preset (b = 19, threshold 200)
