@@ -1,5 +1,5 @@
 """The autotuner on 24-slot bands, where lazy blocks have one register budget: it
-never chooses between a kernel and itself (with noise as the judge), and a file that
+never chooses between a kernel and itself (noise would decide), and a file that
 names the second budget there still gives a plan."""
 import numpy as np
 import pytest
